@@ -16,18 +16,34 @@
 // trajectory-major and gathered for the denoiser (k_srds_plan_gather); then
 // the step (k_srds_apply) takes eps from the batch (miss, updating the entry,
 // Eq. 7) or from the cache (hit, Eq. 6). The distances of a stage's rows are
-// summed by the kernel that produced those rows (the previous stage's
-// k_srds_apply, or k_srds_err for the first fine stage of an iteration) into
+// summed by the previous stage's k_srds_apply, which produced those rows, into
 // fp64 accumulators, one set per stage parity, while the new values are in
-// registers.
+// registers. The rows of an iteration's first fine stage are the boundaries
+// U_n, whose distances the coarse stages' own hit tests have already summed;
+// they are kept per block (dist0). The Eq. 2 partials of a boundary come from
+// the coarse stage that overwrites it, which also starts the next fine sweep
+// (Y_n <- U_n) where it has just read F_n: no separate pass over the
+// boundaries at the end of an iteration.
 //
-// Data (rows of D): U, Up [B][N+1][D] fp64 boundaries now and before this
-// iteration; Y [B][N][D] fp64 fine states (F after the sweep); G [B][N][D]
-// fp64 coarse results; Xh [B][T][D] fp64 and Eh [B][T][D] fp32 the cache;
-// batch_x [B*N][D] fp32. The trajectory states are fp64: a sample passes
-// through about T steps plus N corrections, one rounding each, and fp32
-// states drift by ~1e-5 of the latent scale over T = 100 (measured); the
-// denoiser still sees fp32 rows and returns fp32 eps.
+// Data (rows of D): U [B][N+1] boundaries; Y [B][N] fine states (F after the
+// sweep); G [B][N] coarse results; Xh [B][T] and Eh [B][T] the cache; batch_x
+// [B*N][D] fp32. The trajectory states U, Y, G, Xh are pairs of fp32 values,
+// an unevaluated sum hi + lo of about 48 bits, a row being D hi parts and then
+// D lo parts: a sample passes through about T steps plus N corrections, one
+// rounding each, and single fp32 states drift by ~1e-5 of the latent scale over
+// T = 100 (measured). Eh is fp32: the denoiser sees fp32 rows and returns fp32
+// eps.
+//
+// What bounds it: a coarse stage has B rows and is a latency chain; a fine
+// stage moves 24 to 44 bytes per value (x in and out, eps, the next entry's
+// xhat, a miss's entry and batch row). Pairs and not fp64: this GPU's fp64 unit
+// takes two operations per clock and SM, and the six per value of a fine step,
+// with the fp64 shuffles of its sums, were what the stage waited for (25 us of
+// a 42 us stage at 8 trajectories of 16,384 values); about 50 fp32 operations
+// in their place take 2. The hi parts alone are what the denoiser's batch
+// needs, so the gather reads half a row. Every thread takes four values with
+// all of its loads issued before the first store, the ones that earlier stages
+// wrote before the dependency wait.
 #include <cmath>
 #include <string>
 #include <vector>
@@ -42,7 +58,8 @@ void set_error(const std::string& msg);  // pa_solver.cpp
 namespace {
 
 constexpr int kSThreads = 256;
-constexpr int kSStrip = 1024;        // columns per error CTA
+constexpr int kSCols = 4;            // values per thread: 32 bytes of an fp64 row
+constexpr int kSChunk = kSThreads * kSCols;  // columns per apply CTA
 constexpr int kSMaxRows = 2048;      // B * N
 
 enum StageKind : int32_t { kCoarseInit = 0, kFine = 1, kCoarse = 2 };
@@ -55,27 +72,28 @@ struct SCtl {
 struct SDev {
   int T, B, N, s, nstrip;
   int64_t D;
-  double* U;
-  double* Up;
-  double* Y;
-  double* G;
-  double* Xh;
+  float* U;           // pairs: row pitch 2 D
+  float* Y;
+  float* G;
+  float* Xh;
   float* Eh;
   int32_t* has;      // [B][T]
   float* batch_x;    // [B*N][D]
   int32_t* miss_bt;  // [B*N][2]
   int32_t* rank;     // [B*N]: miss rank, -1 hit, -2 not live
-  double* part;      // [B*N][nstrip] Eq. 2 partials of the block boundaries
+  double* part;      // [B*N][nstrip] Eq. 2 partials of the block boundaries, one per apply CTA
+  double* dist0;     // [B*N] Eq. 4 sums of the next fine sweep's first rows (Y_n = U_n)
   double* sacc;      // [2][B*N] x kAccStride: Eq. 4 sums of the next stage's rows, set = stage number mod 2
   int32_t* active;   // [B]
   int32_t* iters;    // [B]
   float* err_log;    // [N][B]
-  const double* cm1;  // [T] single steps: c_i - 1
-  const double* e1;   // [T]
-  const double* cjm1; // [N] block jumps: c - 1
-  const double* ej;   // [N]
+  const float2* cm1;  // [T] single steps: c_i - 1, a pair like the states
+  const float2* e1;   // [T]
+  const float2* cjm1; // [N] block jumps: c - 1
+  const float2* ej;   // [N]
   SCtl* ctl;
   double tol, cache_thresh;
+  double thr_d;      // cache_thresh * D, the bound on a distance's undivided sum
 };
 
 struct Stage {
@@ -89,19 +107,19 @@ __device__ __forceinline__ int stage_rows(const SDev& d, const Stage& st) {
 // Row r of a stage: trajectory b, sampling index i, its input row; false if
 // the row takes no part (frozen trajectory, or past the end of a short block).
 __device__ __forceinline__ bool row_info(const SDev& d, const Stage& st, int r, int& b, int& n, int& i,
-                                         double*& x) {
+                                         float*& x) {
   if (st.kind == kFine) {
     b = r / d.N;
     n = r % d.N;
     i = n * d.s + st.j;
     const int end = min((n + 1) * d.s, d.T);
-    x = d.Y + ((int64_t)b * d.N + n) * d.D;
+    x = d.Y + ((int64_t)b * d.N + n) * 2 * d.D;
     return d.active[b] && i < end;
   }
   b = r;
   n = st.n;
   i = n * d.s;
-  x = d.U + ((int64_t)b * (d.N + 1) + n) * d.D;
+  x = d.U + ((int64_t)b * (d.N + 1) + n) * 2 * d.D;
   return d.active[b] != 0;
 }
 
@@ -114,17 +132,124 @@ __device__ __forceinline__ double quantize_sum(double v) {
   return ceil(v * 4294967296.0) * (1.0 / 4294967296.0);
 }
 
-__device__ __forceinline__ double block_sum(double v, double* s_w) {
+// ---- pairs: an unevaluated sum h + l of two fp32 values, |l| <= ulp(h) / 2.
+// Error-free sums and products (Dekker, Knuth: TwoSum, FastTwoSum, and TwoProd
+// by fused multiply-add); an operation's result is within a few 2^-48 of the
+// exact one. Where a value is not finite the error terms are not either, and
+// the plain fp32 result stands alone.
+struct Pair {
+  float h, l;
+};
+// (the _rn intrinsics: nothing here may be contracted into a multiply-add)
+__device__ __forceinline__ Pair pair_quick(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Pair pair_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const Pair s = pair_sum(a.h, b.h);
+  return pair_quick(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Pair pair_sub(Pair a, Pair b) { return pair_add(a, Pair{-b.h, -b.l}); }
+__device__ __forceinline__ Pair pair_mul(Pair a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return {p, fmaf(a.l, b, fmaf(a.h, b, -p))};
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return {p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+__device__ __forceinline__ Pair pair_or(Pair a, float plain) {  // the pair, or the fp32 value where it is not finite
+  return finite(__fadd_rn(a.h, a.l)) ? a : Pair{plain, 0.f};
+}
+__device__ __forceinline__ double pair_value(Pair a) { return (double)a.h + (double)a.l; }
+
+// The sum over a warp (in every lane): a butterfly of pairs, beside one of
+// plain values for a sum that is not finite.
+__device__ __forceinline__ double warp_sum(Pair v) {
+  float plain = v.h;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) {
+    v = pair_add(v, Pair{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+    plain += __shfl_xor_sync(0xffffffffu, plain, o);
+  }
+  return pair_value(pair_or(v, plain));
+}
+
+// The CTA's sums of v (if with_v) and w (if with_w) in a fixed order, valid in
+// thread 0: pairs within a warp, fp64 over the warps.
+__device__ __forceinline__ double2 block_sum2(Pair v, bool with_v, Pair w, bool with_w, double2* s_w) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) s_w[warp] = v;
+  const double sv = with_v ? warp_sum(v) : 0.0, sw = with_w ? warp_sum(w) : 0.0;
+  if (lane == 0) s_w[warp] = make_double2(sv, sw);
   __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < kSThreads / 32; ++w) t += s_w[w];  // fixed order
+  double2 t = make_double2(0.0, 0.0);
+  if (warp == 0) {
+    static_assert(kSThreads / 32 == 8, "three halvings");
+    t = s_w[lane & 7];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      if (with_v) t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+      if (with_w) t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+    }
+  }
   return t;
 }
+
+// A thread's kSCols values of a row piece of kSChunk columns: adjacent ones
+// (VEC: D % 4 == 0, 16-byte accesses), or every kSThreads-th one, so that a
+// warp still touches adjacent columns. Columns past D are left alone.
+template <bool VEC>
+struct Piece {
+  int64_t c;  // first column
+  int n;      // of kSCols columns, how many lie inside the row
+  __device__ Piece(int64_t base, int64_t D) {
+    if constexpr (VEC) {
+      c = base + (int64_t)threadIdx.x * kSCols;
+      n = c < D ? kSCols : 0;
+    } else {
+      c = base + threadIdx.x;
+      n = c < D ? (int)min((int64_t)kSCols, (D - c + kSThreads - 1) / kSThreads) : 0;
+    }
+  }
+  __device__ void load(const float* row, float (&v)[kSCols]) const {
+    if constexpr (VEC) {
+      if (n) {
+        const float4 a = *reinterpret_cast<const float4*>(row + c);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kSCols; ++k)
+        if (k < n) v[k] = row[c + (int64_t)k * kSThreads];
+    }
+  }
+  // a row of pairs: D hi parts, then D lo parts
+  __device__ void load(const float* row, int64_t D, Pair (&v)[kSCols]) const {
+    float h[kSCols] = {}, l[kSCols] = {};
+    load(row, h);
+    load(row + D, l);
+#pragma unroll
+    for (int k = 0; k < kSCols; ++k) v[k] = Pair{h[k], l[k]};
+  }
+  __device__ void store(float* row, int64_t D, const Pair (&v)[kSCols]) const {
+    store(row, {v[0].h, v[1].h, v[2].h, v[3].h});
+    store(row + D, {v[0].l, v[1].l, v[2].l, v[3].l});
+  }
+  __device__ void store(float* row, const float (&v)[kSCols]) const {
+    if constexpr (VEC) {
+      if (n) *reinterpret_cast<float4*>(row + c) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kSCols; ++k)
+        if (k < n) row[c + (int64_t)k * kSThreads] = v[k];
+    }
+  }
+};
 
 // One stage's plan and batch, one launch. Every CTA takes the stage's
 // decision over its rows (at most 2048) with all of its warps, one 32-row chunk
@@ -132,9 +257,14 @@ __device__ __forceinline__ double block_sum(double v, double* s_w) {
 // tau_cache (Eq. 5); misses get ranks in row order (trajectory-major) from the
 // chunks' ballots and one scan of their miss counts. The
 // same inputs give the same plan in every CTA; CTA (0, 0) publishes it (ranks,
-// miss list, counters) and clears the distance set the coming apply adds into.
-// Then every CTA narrows its column range of the batch row whose rank is its
-// blockIdx.y, if that row holds a miss.
+// miss list, counters) and clears the distance set the coming apply adds into
+// (and, in an iteration's first coarse stage, the blocks' dist0).
+// Then every CTA copies (the hi parts, the rows rounded to fp32) its column range of the batch row whose rank is its
+// blockIdx.y, if that row holds a miss, kSUnroll pieces at a time with all
+// loads before the stores.
+constexpr int kSUnroll = 4;
+
+template <bool VEC>
 __global__ void __launch_bounds__(kSThreads) k_srds_plan_gather(SDev d, Stage st, int set) {
   pa::pdl_wait();     // everything read here comes from earlier kernels
   pa::pdl_trigger();  // the successor may now be scheduled
@@ -154,11 +284,12 @@ __global__ void __launch_bounds__(kSThreads) k_srds_plan_gather(SDev d, Stage st
     bool live = false, hit = false;
     if (r < rows) {
       int b, n, i;
-      double* x;
+      float* x;
       live = row_info(d, st, r, b, n, i, x);
       const bool has = i < d.T && d.has[(int64_t)b * d.T + i];
-      const double sv = d.sacc[((size_t)set * R + r) * pa::kAccStride];
-      hit = live && has && sv / (double)d.D < d.cache_thresh;
+      // the first fine rows are the boundaries: their sums were kept per block
+      const double sv = st.kind == kFine && st.j == 0 ? d.dist0[r] : d.sacc[((size_t)set * R + r) * pa::kAccStride];
+      hit = live && has && sv < d.thr_d;
     }
     const unsigned mm = __ballot_sync(0xffffffffu, live && !hit), hm = __ballot_sync(0xffffffffu, hit);
     if (lane == 0) {
@@ -194,7 +325,10 @@ __global__ void __launch_bounds__(kSThreads) k_srds_plan_gather(SDev d, Stage st
       }
     }
     if (publish)
-      for (int q = lane; q < R; q += 32) d.sacc[((size_t)(set ^ 1) * R + q) * pa::kAccStride] = 0.0;
+      for (int q = lane; q < R; q += 32) {
+        d.sacc[((size_t)(set ^ 1) * R + q) * pa::kAccStride] = 0.0;
+        if (st.kind != kFine && st.n == 0) d.dist0[q] = 0.0;
+      }
   }
   __syncthreads();
   // 3. ranks in row order; the row of this CTA's rank
@@ -209,7 +343,7 @@ __global__ void __launch_bounds__(kSThreads) k_srds_plan_gather(SDev d, Stage st
       d.rank[r] = miss ? rank : (((s_hm[c] >> lane) & 1u) ? -1 : -2);
       if (miss) {
         int b, n, i;
-        double* x;
+        float* x;
         row_info(d, st, r, b, n, i, x);
         d.miss_bt[2 * rank] = b;
         d.miss_bt[2 * rank + 1] = i;
@@ -220,148 +354,177 @@ __global__ void __launch_bounds__(kSThreads) k_srds_plan_gather(SDev d, Stage st
   const int m = blockIdx.y, r = s_row;
   if (m >= s_total || r < 0) return;
   int b, n, i;
-  double* x;
+  float* x;
   row_info(d, st, r, b, n, i, x);
   float* to = d.batch_x + (int64_t)m * d.D;
-  for (int64_t c = (int64_t)blockIdx.x * kSThreads + tid; c < d.D; c += (int64_t)gridDim.x * kSThreads)
-    to[c] = (float)x[c];
+  const int64_t npiece = (d.D + kSChunk - 1) / kSChunk;
+  for (int64_t q0 = blockIdx.x; q0 < npiece; q0 += (int64_t)gridDim.x * kSUnroll) {
+    float v[kSUnroll][kSCols];
+#pragma unroll
+    for (int u = 0; u < kSUnroll; ++u) {
+      const int64_t q = q0 + (int64_t)u * gridDim.x;
+      if (q < npiece) Piece<VEC>(q * kSChunk, d.D).load(x, v[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kSUnroll; ++u) {
+      const int64_t q = q0 + (int64_t)u * gridDim.x;
+      if (q < npiece) Piece<VEC>(q * kSChunk, d.D).store(to, v[u]);
+    }
+  }
 }
 
 // The step of every live row: eps from the batch (miss: the entry becomes
 // (x, eps), Eq. 7) or the cache (hit, Eq. 6); then a fine step
 // Y <- Y + (c_i - 1) Y + e_i eps, or a coarse jump g = x + (c - 1) x + e eps
-// with U_{n+1} = g (iteration 0) or g + F_n - G_n (later), G_n <- g.
-// The next stage's rows that this stage produced also get their Eq. 4
+// with U_{n+1} = g (iteration 0) or g + F_n - G_n (later), G_n <- g and, for
+// the next fine sweep, Y_n <- x.
+// The next stage's row that this row's value feeds also gets its Eq. 4
 // distance here, added into set `nset`: a fine step feeds the next fine step
-// of its block; the last fine step of block 0 feeds the first coarse block,
-// whose input U_0 does not change; a coarse block feeds the next one.
+// of its block, a coarse block the next one. (The first coarse block's input
+// U_0 never changes and equals its entry: its sum stays 0.) A coarse row's own
+// distance is that of the next fine sweep's first row of its block too, zero
+// once a miss has made the entry equal to the row (NaN if the row holds a
+// NaN or an infinity, which is never a hit); it goes to dist0.
+// grid: a CTA per kSChunk columns x rows. What earlier stages wrote (x, F, G,
+// the old boundary, the next entry's xhat, flags) is read before the
+// dependency wait; only the plan and eps, written by the two kernels before,
+// are read after it.
+template <bool VEC>
 __global__ void __launch_bounds__(kSThreads) k_srds_apply(SDev d, Stage st, const float* __restrict__ beps,
                                                          int nset) {
-  pa::pdl_wait();     // everything read here comes from earlier kernels
-  pa::pdl_trigger();  // the successor may now be scheduled
-  __shared__ double s_w[kSThreads / 32];
+  __shared__ double2 s_w[kSThreads / 32];
   const int r = blockIdx.y;
   int b, n, i;
-  double* x;
-  if (!row_info(d, st, r, b, n, i, x)) return;
-  const int rk = d.rank[r];
+  float* x;
+  const bool live = row_info(d, st, r, b, n, i, x);
+  if (!live) {  // every CTA passes the dependency wait before it exits
+    pa::pdl_wait();
+    return;
+  }
+  const bool fine = st.kind == kFine, corr = st.kind == kCoarse;
+  const Piece<VEC> pc((int64_t)blockIdx.x * kSChunk, d.D);
   const int64_t e_off = ((int64_t)b * d.T + i) * d.D;
-  const float* eps = rk >= 0 ? beps + (int64_t)rk * d.D : d.Eh + e_off;
-  if (rk >= 0 && blockIdx.x == 0 && threadIdx.x == 0) d.has[(int64_t)b * d.T + i] = 1;
-  const double cm1 = st.kind == kFine ? d.cm1[i] : d.cjm1[n];
-  const double ec = st.kind == kFine ? d.e1[i] : d.ej[n];
-  double* Un1 = d.U + ((int64_t)b * (d.N + 1) + n + 1) * d.D;
-  double* Gn = d.G + ((int64_t)b * d.N + n) * d.D;
-  const double* Fn = d.Y + ((int64_t)b * d.N + n) * d.D;
-  // the next stage's row fed by this one, if any: its row index, timestep and input
+  const float2 cm1 = fine ? d.cm1[i] : d.cjm1[n];
+  const float2 ec = fine ? d.e1[i] : d.ej[n];
+  float* Un1 = d.U + ((int64_t)b * (d.N + 1) + n + 1) * 2 * d.D;
+  float* Gn = d.G + ((int64_t)b * d.N + n) * 2 * d.D;
+  float* Yn = d.Y + ((int64_t)b * d.N + n) * 2 * d.D;
+  // the next stage's row fed by this one, if any: its row index and timestep
   int nrow = -1, i1 = 0;
-  const double* nx0 = nullptr;  // the next input when it is not the value computed here
-  if (st.kind == kFine) {
-    if (st.j + 1 < d.s) {
-      const int end = min((n + 1) * d.s, d.T);
-      if (i + 1 < end) { nrow = r; i1 = i + 1; }
-    } else if (n == 0) {
-      nrow = b; i1 = 0; nx0 = d.U + (int64_t)b * (d.N + 1) * d.D;
-    }
+  if (fine) {
+    if (st.j + 1 < d.s && i + 1 < min((n + 1) * d.s, d.T)) { nrow = r; i1 = i + 1; }
   } else if (n + 1 < d.N) {
     nrow = b; i1 = (n + 1) * d.s;
   }
-  // an entry for timestep i1 exists if an earlier stage made it, or this row
-  // (same timestep: one step per block) is a miss making it now
-  const bool nhas = nrow >= 0 && ((i1 == i && rk >= 0) || d.has[(int64_t)b * d.T + i1] != 0);
-  const double* xh1 = d.Xh + ((int64_t)b * d.T + i1) * d.D;
-  double dist = 0.0;
-  for (int64_t c = (int64_t)blockIdx.x * kSThreads + threadIdx.x; c < d.D; c += (int64_t)gridDim.x * kSThreads) {
-    const double xv = x[c];
-    const float ev = eps[c];
-    if (rk >= 0) {
-      d.Xh[e_off + c] = xv;
-      d.Eh[e_off + c] = ev;
-    }
-    const double g = xv + fma(cm1, xv, ec * (double)ev);
-    double nv;
-    if (st.kind == kFine) {
-      x[c] = g;
-      nv = g;
-    } else if (st.kind == kCoarseInit) {
-      Gn[c] = g;
-      Un1[c] = g;
-      nv = g;
-    } else {
-      nv = g + (Fn[c] - Gn[c]);
-      Un1[c] = nv;
-      Gn[c] = g;
-    }
-    if (nhas) dist += fabs((nx0 ? nx0[c] : nv) - xh1[c]);
+  const bool nhas = nrow >= 0 && d.has[(int64_t)b * d.T + i1] != 0;
+  Pair xv[kSCols] = {}, xh1[kSCols] = {}, fv[kSCols] = {}, gv[kSCols] = {}, uv[kSCols] = {};
+  pc.load(x, d.D, xv);
+  if (nhas) pc.load(d.Xh + ((int64_t)b * d.T + i1) * 2 * d.D, d.D, xh1);
+  if (corr) {
+    pc.load(Yn, d.D, fv);
+    pc.load(Gn, d.D, gv);
+    pc.load(Un1, d.D, uv);
   }
-  if (nhas) {
-    const double t = block_sum(dist, s_w);
-    if (threadIdx.x == 0) atomicAdd(d.sacc + ((size_t)nset * d.B * d.N + nrow) * pa::kAccStride, quantize_sum(t));
-  }
-}
-
-// End of an iteration: partial sums of (U_{n+1} - Up_{n+1})^2 per strip
-// (iterations >= 1), then Up <- U and Y_n <- U_n for the next fine sweep.
-// The next fine sweep starts from Y_n = U_n: the Eq. 4 distance of its first
-// stage's rows (timestep n s) is added into set `nset` here.
-__global__ void __launch_bounds__(kSThreads) k_srds_err(SDev d, int iter, int nset) {
-  pa::pdl_wait();     // everything read here comes from earlier kernels
+  float ev[kSCols] = {};
+  // a coarse stage is a chain of round trips: its entry is fetched before the
+  // plan is known (a fine stage would pay the bytes of every miss's)
+  if (!fine) pc.load(d.Eh + e_off, ev);
+  pa::pdl_wait();     // the plan and the batch's eps come from the kernels just before
   pa::pdl_trigger();  // the successor may now be scheduled
-  __shared__ double s_w[kSThreads / 32];
-  const int r = blockIdx.y, b = r / d.N, n = r % d.N;
-  if (!d.active[b]) return;
-  const int64_t c0 = (int64_t)blockIdx.x * kSStrip;
-  const int64_t c1 = (c0 + kSStrip < d.D) ? c0 + kSStrip : d.D;
-  double* u1 = d.U + ((int64_t)b * (d.N + 1) + n + 1) * d.D;
-  double* p1 = d.Up + ((int64_t)b * (d.N + 1) + n + 1) * d.D;
-  const double* u0 = d.U + ((int64_t)b * (d.N + 1) + n) * d.D;
-  double* y = d.Y + ((int64_t)b * d.N + n) * d.D;
-  const bool nhas = d.has[(int64_t)b * d.T + n * d.s] != 0;
-  const double* xh = d.Xh + ((int64_t)b * d.T + n * d.s) * d.D;
-  double acc = 0.0, dist = 0.0;
-  for (int64_t c = c0 + threadIdx.x; c < c1; c += kSThreads) {
-    const double df = u1[c] - p1[c];
-    acc = fma(df, df, acc);
-    p1[c] = u1[c];
-    const double v = u0[c];
-    y[c] = v;
-    if (nhas) dist += fabs(v - xh[c]);
+  const int rk = d.rank[r];
+  if (rk >= 0) {
+    pc.load(beps + (int64_t)rk * d.D, ev);
+  } else if (fine) {
+    pc.load(d.Eh + e_off, ev);
   }
-  const double t = block_sum(acc, s_w);
-  if (threadIdx.x == 0) d.part[(int64_t)r * d.nstrip + blockIdx.x] = iter > 0 ? t : 0.0;
-  if (nhas) {
-    __syncthreads();  // s_w is reused
-    const double t2 = block_sum(dist, s_w);
-    if (threadIdx.x == 0) atomicAdd(d.sacc + ((size_t)nset * d.B * d.N + r) * pa::kAccStride, quantize_sum(t2));
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (rk >= 0) d.has[(int64_t)b * d.T + i] = 1;
+    if (!fine && rk < 0)
+      atomicAdd(d.dist0 + (int64_t)b * d.N + n, d.sacc[((size_t)(nset ^ 1) * d.B * d.N + r) * pa::kAccStride]);
+  }
+  Pair nv[kSCols], g[kSCols], err = {0.f, 0.f}, dist = {0.f, 0.f};
+  float perr = 0.f, pdist = 0.f;  // the plain sums: what is left where the pairs are not finite
+#pragma unroll
+  for (int k = 0; k < kSCols; ++k) {
+    const Pair dr = pair_add(pair_mul(Pair{cm1.x, cm1.y}, xv[k]), pair_mul(Pair{ec.x, ec.y}, ev[k]));
+    g[k] = pair_or(pair_add(xv[k], dr), xv[k].h + fmaf(cm1.x, xv[k].h, ec.x * ev[k]));
+    nv[k] = corr ? pair_or(pair_add(g[k], pair_sub(fv[k], gv[k])), g[k].h + (fv[k].h - gv[k].h)) : g[k];
+    if (k < pc.n) {
+      if (nhas) {
+        const Pair df = pair_sub(nv[k], xh1[k]);
+        dist = pair_add(dist, df.h < 0.f ? Pair{-df.h, -df.l} : df);
+        pdist += fabsf(nv[k].h - xh1[k].h);
+      }
+      if (corr) {
+        const Pair df = pair_sub(nv[k], uv[k]);
+        err = pair_add(err, pair_mul(df, df));
+        const float q = nv[k].h - uv[k].h;
+        perr = fmaf(q, q, perr);
+      }
+    }
+  }
+  if (rk >= 0) {
+    pc.store(d.Xh + ((int64_t)b * d.T + i) * 2 * d.D, d.D, xv);
+    pc.store(d.Eh + e_off, ev);
+    if (!fine) {
+      float z = 0.f;
+#pragma unroll
+      for (int k = 0; k < kSCols; ++k) z += xv[k].h - xv[k].h;
+      if (!(z == 0.f)) atomicAdd(d.dist0 + (int64_t)b * d.N + n, (double)z);
+    }
+  }
+  if (fine) {
+    pc.store(x, d.D, g);
+  } else {
+    pc.store(Un1, d.D, nv);
+    pc.store(Gn, d.D, g);
+    pc.store(Yn, d.D, xv);
+  }
+  if (nhas || corr) {
+    const double2 t = block_sum2(pair_or(err, perr), corr, pair_or(dist, pdist), nhas, s_w);
+    if (threadIdx.x == 0) {
+      if (corr) d.part[((int64_t)b * d.N + n) * d.nstrip + blockIdx.x] = t.x;
+      if (nhas) atomicAdd(d.sacc + ((size_t)nset * d.B * d.N + nrow) * pa::kAccStride, quantize_sum(t.y));
+    }
   }
 }
 
-// Convergence of every trajectory after iteration `iter` (one CTA).
-__global__ void __launch_bounds__(kSThreads) k_srds_finish(SDev d, int iter, cudaGraphConditionalHandle next,
-                                                           int has_next) {
+// Convergence of every trajectory after iteration `iter` (one CTA, a warp per
+// trajectory at a time, a lane per boundary): the boundaries' Eq. 2 sums from
+// the apply CTAs' partials in order, then their maximum.
+constexpr int kSFinishThreads = 512;
+
+__global__ void __launch_bounds__(kSFinishThreads) k_srds_finish(SDev d, int iter, cudaGraphConditionalHandle next,
+                                                                 int has_next) {
   pa::pdl_wait();     // everything read here comes from earlier kernels
   pa::pdl_trigger();  // the successor may now be scheduled
   __shared__ int s_act;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_act = 0;
   __syncthreads();
-  for (int b = threadIdx.x; b < d.B; b += kSThreads) {
+  for (int b = warp; b < d.B; b += kSFinishThreads / 32) {
     if (!d.active[b]) continue;
+    bool more = true;
     if (iter > 0) {
       double err = 0.0;
-      for (int n = 0; n < d.N; ++n) {
+      for (int n = lane; n < d.N; n += 32) {
+        const double* pt = d.part + ((int64_t)b * d.N + n) * d.nstrip;
         double sum = 0.0;
-        const int r = b * d.N + n;
-        for (int k = 0; k < d.nstrip; ++k) sum += d.part[(int64_t)r * d.nstrip + k];
-        err = fmax(err, sum / (double)d.D);
+#pragma unroll 16
+        for (int k = 0; k < d.nstrip; ++k) sum += pt[k];
+        err = fmax(err, sum);
       }
-      d.iters[b] = iter;
-      d.err_log[(int64_t)(iter - 1) * d.B + b] = (float)err;
-      if (err <= d.tol || iter >= d.N) {
-        d.active[b] = 0;
-        continue;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
+      err /= (double)d.D;  // one division: the fp64 unit takes two operations per clock
+      more = !(err <= d.tol || iter >= d.N);
+      if (lane == 0) {
+        d.iters[b] = iter;
+        d.err_log[(int64_t)(iter - 1) * d.B + b] = (float)err;
+        if (!more) d.active[b] = 0;
       }
     }
-    atomicAdd(&s_act, 1);
+    if (more && lane == 0) atomicAdd(&s_act, 1);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -373,16 +536,33 @@ __global__ void __launch_bounds__(kSThreads) k_srds_finish(SDev d, int iter, cud
   }
 }
 
-// fp32 rows (pitch D) -> fp64 rows of the boundary array (pitch (N+1) D), and back.
-__global__ void k_srds_load(SDev d, const float* __restrict__ src, int slot) {
+// The start of a generation: the fp32 rows of x_init (pitch D) widened into
+// U_0, every flag, sum and counter cleared (grid x trajectories).
+__global__ void __launch_bounds__(kSThreads) k_srds_init(SDev d, const float* __restrict__ src) {
   pa::pdl_wait();     // everything read here comes from earlier kernels
   pa::pdl_trigger();  // the successor may now be scheduled
   const int b = blockIdx.y;
-  double* to = d.U + ((int64_t)b * (d.N + 1) + slot) * d.D;
-  double* to2 = d.Up + ((int64_t)b * (d.N + 1) + slot) * d.D;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < d.D; c += (int64_t)gridDim.x * blockDim.x) {
-    to[c] = (double)src[(int64_t)b * d.D + c];
-    to2[c] = to[c];
+  float* to = d.U + (int64_t)b * (d.N + 1) * 2 * d.D;
+  const int64_t first = (int64_t)blockIdx.x * kSThreads + threadIdx.x, step = (int64_t)gridDim.x * kSThreads;
+  for (int64_t c = first; c < d.D; c += step) {
+    to[c] = src[(int64_t)b * d.D + c];
+    to[d.D + c] = 0.f;
+  }
+  for (int64_t q = first; q < d.T; q += step) d.has[(int64_t)b * d.T + q] = 0;
+  for (int64_t q = first; q < d.N; q += step) {
+    const int64_t r = (int64_t)b * d.N + q, R = (int64_t)d.B * d.N;
+    d.dist0[r] = 0.0;
+    d.sacc[r * pa::kAccStride] = 0.0;
+    d.sacc[(R + r) * pa::kAccStride] = 0.0;
+  }
+  if (first == 0) {
+    d.active[b] = 1;
+    d.iters[b] = 0;
+    if (b == 0) {
+      SCtl c{};
+      c.n_active = d.B;
+      *d.ctl = c;
+    }
   }
 }
 
@@ -390,51 +570,36 @@ __global__ void k_srds_store(SDev d, float* __restrict__ dst, int slot) {
   pa::pdl_wait();     // everything read here comes from earlier kernels
   pa::pdl_trigger();  // the successor may now be scheduled
   const int b = blockIdx.y;
-  const double* from = d.U + ((int64_t)b * (d.N + 1) + slot) * d.D;
+  const float* from = d.U + ((int64_t)b * (d.N + 1) + slot) * 2 * d.D;  // the hi parts: rounded to fp32
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < d.D; c += (int64_t)gridDim.x * blockDim.x)
-    dst[(int64_t)b * d.D + c] = (float)from[c];
-}
-
-__global__ void k_srds_reset(SDev d) {
-  pa::pdl_wait();     // everything read here comes from earlier kernels
-  pa::pdl_trigger();  // the successor may now be scheduled
-  for (int b = threadIdx.x; b < d.B; b += blockDim.x) {
-    d.active[b] = 1;
-    d.iters[b] = 0;
-  }
-  for (int64_t q = threadIdx.x; q < (int64_t)d.B * d.T; q += blockDim.x) d.has[q] = 0;
-  if (threadIdx.x == 0) {
-    SCtl c{};
-    c.n_active = d.B;
-    *d.ctl = c;
-  }
+    dst[(int64_t)b * d.D + c] = from[c];
 }
 
 struct SLayout {
-  size_t U, Up, Y, G, Xh, Eh, has, batch_x, miss_bt, rank, part, sacc, active, iters, err_log, coef, ctl, total;
+  size_t U, Y, G, Xh, Eh, has, batch_x, miss_bt, rank, part, dist0, sacc, active, iters, err_log, coef, ctl, total;
 };
 
 SLayout s_layout(int T, int64_t D, int B, int N, int nstrip) {
   SLayout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = pa::align_up(o + bytes, pa::kAlign); return at; };
-  const size_t row = (size_t)D * sizeof(float), row64 = (size_t)D * sizeof(double);
-  L.U = take((size_t)B * (N + 1) * row64);
-  L.Up = take((size_t)B * (N + 1) * row64);
-  L.Y = take((size_t)B * N * row64);
-  L.G = take((size_t)B * N * row64);
-  L.Xh = take((size_t)B * T * row64);
+  const size_t row = (size_t)D * sizeof(float), row2 = 2 * row;  // rows of pairs
+  L.U = take((size_t)B * (N + 1) * row2);
+  L.Y = take((size_t)B * N * row2);
+  L.G = take((size_t)B * N * row2);
+  L.Xh = take((size_t)B * T * row2);
   L.Eh = take((size_t)B * T * row);
   L.has = take((size_t)B * T * sizeof(int32_t));
   L.batch_x = take((size_t)B * N * row);
   L.miss_bt = take((size_t)B * N * 2 * sizeof(int32_t));
   L.rank = take((size_t)B * N * sizeof(int32_t));
   L.part = take((size_t)B * N * nstrip * sizeof(double));
+  L.dist0 = take((size_t)B * N * sizeof(double));
   L.sacc = take((size_t)2 * B * N * pa::kAccStride * sizeof(double));  // one 128-byte line per sum
   L.active = take((size_t)B * sizeof(int32_t));
   L.iters = take((size_t)B * sizeof(int32_t));
   L.err_log = take((size_t)N * B * sizeof(float));
-  L.coef = take((size_t)(2 * T + 2 * N) * sizeof(double));
+  L.coef = take((size_t)(2 * T + 2 * N) * sizeof(float2));
   L.ctl = take(sizeof(SCtl));
   L.total = o;
   return L;
@@ -545,7 +710,7 @@ extern "C" size_t pa_srds_workspace_bytes(int T, int64_t D, int batch) {
   int s, N;
   s_blocks(T, &s, &N);
   if ((int64_t)batch * N > kSMaxRows) return 0;
-  return s_layout(T, D, batch, N, (int)((D + kSStrip - 1) / kSStrip)).total;
+  return s_layout(T, D, batch, N, (int)((D + kSChunk - 1) / kSChunk)).total;
 }
 
 extern "C" pa_status pa_srds_create(pa_srds** out, int T, const int64_t* latent_shape, int ndim,
@@ -568,7 +733,7 @@ extern "C" pa_status pa_srds_create(pa_srds** out, int T, const int64_t* latent_
   int s, N;
   s_blocks(T, &s, &N);
   if ((int64_t)batch * N > kSMaxRows) return s_fail("pa_srds_create: batch * blocks exceeds 2048", PA_ERR_ARG);
-  const int nstrip = (int)((D + kSStrip - 1) / kSStrip);
+  const int nstrip = (int)((D + kSChunk - 1) / kSChunk);
   const SLayout L = s_layout(T, D, batch, N, nstrip);
   if (!workspace_dev || (reinterpret_cast<uintptr_t>(workspace_dev) % pa::kAlign) != 0 || workspace_bytes < L.total)
     return s_fail("pa_srds_create: workspace NULL, not 256-byte aligned, or smaller than pa_srds_workspace_bytes()",
@@ -581,22 +746,22 @@ extern "C" pa_status pa_srds_create(pa_srds** out, int T, const int64_t* latent_
   char* w = h->ws;
   SDev& d = h->d;
   d.T = T; d.B = batch; d.N = N; d.s = s; d.nstrip = nstrip; d.D = D;
-  d.U = reinterpret_cast<double*>(w + L.U);
-  d.Up = reinterpret_cast<double*>(w + L.Up);
-  d.Y = reinterpret_cast<double*>(w + L.Y);
-  d.G = reinterpret_cast<double*>(w + L.G);
-  d.Xh = reinterpret_cast<double*>(w + L.Xh);
+  d.U = reinterpret_cast<float*>(w + L.U);
+  d.Y = reinterpret_cast<float*>(w + L.Y);
+  d.G = reinterpret_cast<float*>(w + L.G);
+  d.Xh = reinterpret_cast<float*>(w + L.Xh);
   d.Eh = reinterpret_cast<float*>(w + L.Eh);
   d.has = reinterpret_cast<int32_t*>(w + L.has);
   d.batch_x = reinterpret_cast<float*>(w + L.batch_x);
   d.miss_bt = reinterpret_cast<int32_t*>(w + L.miss_bt);
   d.rank = reinterpret_cast<int32_t*>(w + L.rank);
   d.part = reinterpret_cast<double*>(w + L.part);
+  d.dist0 = reinterpret_cast<double*>(w + L.dist0);
   d.sacc = reinterpret_cast<double*>(w + L.sacc);
   d.active = reinterpret_cast<int32_t*>(w + L.active);
   d.iters = reinterpret_cast<int32_t*>(w + L.iters);
   d.err_log = reinterpret_cast<float*>(w + L.err_log);
-  double* coef = reinterpret_cast<double*>(w + L.coef);
+  float2* coef = reinterpret_cast<float2*>(w + L.coef);
   d.cm1 = coef;
   d.e1 = coef + T;
   d.cjm1 = coef + 2 * T;
@@ -604,14 +769,20 @@ extern "C" pa_status pa_srds_create(pa_srds** out, int T, const int64_t* latent_
   d.ctl = reinterpret_cast<SCtl*>(w + L.ctl);
   d.tol = tol;
   d.cache_thresh = cache_thresh;
+  d.thr_d = cache_thresh * (double)D;
   // DDIM (eta = 0) jump from a to a2: x + (c - 1) x + e eps with c = sqrt(a2 / a),
   // e = sqrt(1 - a2) - sqrt(a2 (1 - a) / a); c - 1 formed without cancellation.
-  auto jump = [](double a, double a2, double* cm1, double* e) {
-    const double r = a2 / a, c = std::sqrt(r);
-    *cm1 = (r - 1.0) / (c + 1.0);
-    *e = std::sqrt(1.0 - a2) - std::sqrt(a2) * std::sqrt(1.0 - a) / std::sqrt(a);
+  // Each coefficient is handed over as a pair.
+  auto pair = [](double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
   };
-  std::vector<double> hc(2 * (size_t)T + 2 * (size_t)N);
+  auto jump = [&pair](double a, double a2, float2* cm1, float2* e) {
+    const double r = a2 / a, c = std::sqrt(r);
+    *cm1 = pair((r - 1.0) / (c + 1.0));
+    *e = pair(std::sqrt(1.0 - a2) - std::sqrt(a2) * std::sqrt(1.0 - a) / std::sqrt(a));
+  };
+  std::vector<float2> hc(2 * (size_t)T + 2 * (size_t)N);
   for (int i = 0; i < T; ++i) jump(alphas_cumprod[i], alphas_cumprod[i + 1], &hc[i], &hc[T + i]);
   for (int n = 0; n < N; ++n) {
     const int a0 = n * s, a1 = (n + 1) * s < T ? (n + 1) * s : T;
@@ -621,7 +792,7 @@ extern "C" pa_status pa_srds_create(pa_srds** out, int T, const int64_t* latent_
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&h->host_ctl), sizeof(SCtl), cudaHostAllocDefault);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(coef, hc.data(), hc.size() * sizeof(double), cudaMemcpyHostToDevice, h->st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(coef, hc.data(), hc.size() * sizeof(float2), cudaMemcpyHostToDevice, h->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.ctl, 0, sizeof(SCtl), h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
   if (e != cudaSuccess) {
@@ -637,13 +808,11 @@ extern "C" pa_status pa_srds_init(pa_srds* h, const float* x_init) {
   if (!h || !x_init) return s_fail("pa_srds_init: NULL argument", PA_ERR_ARG);
   if (h->loop_capturing) return s_fail("pa_srds_init: a generation is being captured", PA_ERR_STATE);
   const SDev& d = h->d;
-  // x_init (host or device) is staged in batch_x, then widened into U_0 and Up_0
+  // x_init (host or device) is staged in batch_x, then widened into U_0
   cudaError_t e = cudaMemcpyAsync(d.batch_x, x_init, (size_t)d.B * d.D * sizeof(float), cudaMemcpyDefault, h->st);
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_init: ") + cudaGetErrorString(e), PA_ERR_CUDA);
-  e = pa::launch_ex(k_srds_load, dim3(32, d.B), dim3(256), 0, h->st, 0, d, (const float*)d.batch_x, 0);
-  if (e == cudaSuccess) e = pa::launch_ex(k_srds_reset, dim3(1), dim3(256), 0, h->st, 0, d);
-  h->launches += 2;
-  if (e == cudaSuccess) e = cudaMemsetAsync(d.sacc, 0, (size_t)2 * d.B * d.N * pa::kAccStride * sizeof(double), h->st);
+  e = pa::launch_ex(k_srds_init, dim3(32, d.B), dim3(kSThreads), 0, h->st, 0, d, (const float*)d.batch_x);
+  h->launches += 1;
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_init: ") + cudaGetErrorString(e), PA_ERR_CUDA);
   h->iter = 0;
   h->stage = 0;
@@ -661,13 +830,13 @@ extern "C" pa_status pa_srds_step_async(pa_srds* h, const float** batch_x, const
   const Stage st = current_stage(h);
   const int rows = st.kind == kFine ? d.B * d.N : d.B;
   // every CTA plans: about two CTAs per SM in all, each narrowing a longer part of its row
-  int gx = (int)((d.D + kSThreads * 4 - 1) / (kSThreads * 4));
+  int gx = d.nstrip;
   const int gcap = (2 * h->nsm + rows - 1) / rows;
   if (gx > gcap) gx = gcap;
   if (gx > 32) gx = 32;
   if (gx < 1) gx = 1;
-  const cudaError_t e =
-      pa::launch_ex(k_srds_plan_gather, dim3(gx, rows), dim3(kSThreads), 0, h->st, 0, d, st, (int)(h->g & 1));
+  const cudaError_t e = pa::launch_ex(d.D % kSCols == 0 ? k_srds_plan_gather<true> : k_srds_plan_gather<false>,
+                                      dim3(gx, rows), dim3(kSThreads), 0, h->st, 0, d, st, (int)(h->g & 1));
   h->launches += 1;
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_step_async: ") + cudaGetErrorString(e), PA_ERR_CUDA);
   if (batch_x) *batch_x = d.batch_x;
@@ -707,27 +876,19 @@ extern "C" pa_status pa_srds_submit_eps(pa_srds* h, const float* batch_eps) {
   const SDev& d = h->d;
   const Stage st = current_stage(h);
   const int rows = st.kind == kFine ? d.B * d.N : d.B;
-  // column blocks per row: four columns per thread (at most 32 blocks), or
-  // more blocks when the stage has few rows (a coarse stage has only B), up to
-  // about two CTAs per SM in all and one column per thread
-  int gx = (int)((d.D + kSThreads * 4 - 1) / (kSThreads * 4));
-  if (gx > 32) gx = 32;
-  const int gsm = (2 * h->nsm + rows - 1) / rows;
-  const int gmax = (int)((d.D + kSThreads - 1) / kSThreads);
-  if (gsm > gx) gx = gsm < gmax ? gsm : gmax;
-  if (gx < 1) gx = 1;
   const int nset = (int)((h->g + 1) & 1);  // the next stage's distance set
-  cudaError_t e = pa::launch_ex(k_srds_apply, dim3(gx, rows), dim3(kSThreads), 0, h->st, 0, d, st, batch_eps, nset);
+  // 16-byte accesses need whole groups of four columns and aligned eps rows
+  const bool vec = d.D % kSCols == 0 && (reinterpret_cast<uintptr_t>(batch_eps) & 15) == 0;
+  cudaError_t e = pa::launch_ex(vec ? k_srds_apply<true> : k_srds_apply<false>, dim3(d.nstrip, rows), dim3(kSThreads),
+                                0, h->st, 0, d, st, batch_eps, nset);
   h->launches++;
   const int nstages = (h->iter == 0 ? 0 : d.s) + d.N;
   if (++h->stage == nstages) {  // the iteration is complete
     const bool next = h->loop_capturing && h->iter + 1 <= d.N;  // captured: set the next IF node's condition
     if (e == cudaSuccess)
-      e = pa::launch_ex(k_srds_err, dim3(d.nstrip, d.B * d.N), dim3(kSThreads), 0, h->st, 0, d, h->iter, nset);
-    if (e == cudaSuccess)
-      e = pa::launch_ex(k_srds_finish, dim3(1), dim3(kSThreads), 0, h->st, 0, d, h->iter,
+      e = pa::launch_ex(k_srds_finish, dim3(1), dim3(kSFinishThreads), 0, h->st, 0, d, h->iter,
                         next ? h->loop_cond[h->iter + 1] : (cudaGraphConditionalHandle)0, next ? 1 : 0);
-    h->launches += 2;
+    h->launches += 1;
     h->stage = 0;
     h->iter++;
     if (h->loop_capturing) {  // the iteration's body is complete: close it, open the next one's

@@ -140,6 +140,36 @@ def test_srds_edge_shapes(T, batch, shape, seed):
     assert g["stats"]["nfe"] == orc.nfe
 
 
+@pytest.mark.parametrize("shape", [(4, 16, 16), (4, 20, 20), (5, 41, 5), (3, 7, 9)])
+def test_srds_row_pieces(shape):
+    """The apply kernel's row pieces: exactly one piece of 1024 columns, a
+    second piece partly filled (1600), one column past a piece (1025, no
+    16-byte rows), a piece of 189 odd columns; and, for the same inputs, eps
+    rows that start 4 bytes past a 16-byte boundary (four-byte accesses)
+    give the aligned run's latents bit for bit."""
+    import torch
+    from paper_2609_36522_gb300.solver import SrdsSolver, GmmDenoiser
+    w = W.TINY.with_(T=20, latent_shape=shape, K=3, sampler="srds", batch=2, seed=33)
+    orc = oracle_srds(w)
+    assert srds_margin(orc, w.cache_thresh) > 1e-4
+    gpu = gpu_srds(w)
+    compare_srds(w, orc, gpu)
+    a, x0, mu = W.inputs(w)
+    s = SrdsSolver(w.T, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch)
+    g = GmmDenoiser(torch.from_numpy(mu).cuda(), w.gmm_std, a, s.max_rows)
+    eps = torch.empty(s.max_rows * w.D, dtype=torch.float32, device="cuda")
+    shifted = torch.empty(s.max_rows * w.D + 1, dtype=torch.float32, device="cuda")[1:]
+    s.init(torch.from_numpy(x0).cuda())
+    while (out := s.step()) is not None:
+        g.eps(out.batch_x_ptr, out.miss_bt_ptr, s.n_miss_dev(), eps)
+        shifted.copy_(eps)
+        s.submit_eps(shifted)
+    s.poll()
+    assert np.array_equal(s.result().cpu().numpy(), gpu["x_final"])
+    s.close()
+    g.close()
+
+
 @pytest.mark.parametrize("wname", ["srds", "srds_batched"])
 def test_srds_generation_graph_equals_host_driven(wname):
     """SrdsSolver.generate through the captured generation (IF nodes, one per
