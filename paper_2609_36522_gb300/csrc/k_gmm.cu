@@ -6,7 +6,11 @@
 //   r = softmax(logit)   (the common -||x||^2 / (2 v) term cancels)
 //   eps = sqrt(1 - a) / v * (x - sqrt(a) sum_k r_k mu_k)
 //
-// Two kernels per call:
+// Four ways to compute it, chosen per handle (pa_gmm_create):
+//   one kernel on thread-block clusters (k_gmm_cluster, form 2)
+//   three persistent tensor-core kernels (k_gmm_tc.cu, form 1, large problems)
+//   the tensor-core kernels below, a CTA per 64-column chunk (form 1, small
+//   problems), and CUDA-core kernels (form 0), two or three kernels per call:
 //   dot products   G = X M^T, split over column chunks of D, either on the
 //                  tensor cores (k_gmm_dots_tc: tcgen05, tf32 operands split
 //                  in two parts for fp32 accuracy) or on the CUDA cores
@@ -37,6 +41,7 @@
 
 #include "../../include/paraanya.h"
 #include "pa_bulk.cuh"
+#include "pa_gmm_tc.h"
 #include "pa_internal.h"
 #include "pa_tcgen05.cuh"
 
@@ -82,7 +87,18 @@ constexpr int kTcCols = 64;   // 8 MMA steps of 8 (98 KB of shared memory at K =
 constexpr int kTcThreads = 256;
 constexpr int kTcCluster = 8;            // column chunks per thread-block cluster ...
 constexpr int kTcClusterMinChunks = 256;  // ... when there are this many chunks (fewer atomics per accumulator)
-constexpr int kTcMinK = 16;               // tensor-core dot products by default above this many components
+constexpr int kTcMinK = 16;               // tensor cores by default above this many components ...
+constexpr int kTcMinRows = 768;           // ... or from this many rows on: at 4x64x64, 16 trajectories of a 100-point
+                                          // window and 16 components a generation takes 945 us, in form 2 1020 us
+// Whether form 1 runs as the persistent kernels of k_gmm_tc.cu: they fill the
+// GPU with one CTA per SM whatever the shape, which costs about 2 us more than
+// small CTAs that overlap where there is little to do. us per call, small CTAs
+// against persistent, at K components, D columns, a capacity of R rows:
+// K 20, D 16384, R 100: 13.6 / 16.1; K 24, D 4096, R 300: 14.9 / 17.5;
+// K 40, D 13056, R 100: 21.6 / 18.9; K 58, D 9216, R 138: 26.9 / 19.9;
+// K 96, D 16384, R 200: 104.5 / 37.5; K 64, D 65536, R 128: 72.7 / 46.6.
+// (They take any D and any alignment, the kernels here whole 16-byte rows.)
+constexpr int64_t kTcPersistentWork = 700 * 1000;
 
 // the MMA's N: K rounded up to 16, 32, 64 or 128 (padded means are zero)
 __host__ __device__ inline int tc_npad(int K) {
@@ -103,7 +119,13 @@ constexpr int kRespRows = 8;  // rows per k_gmm_resp CTA, a warp each
 __host__ __device__ inline size_t ot_img_floats(int K) { return (size_t)2 * kTcRows * tc_npad(K); }
 __host__ __device__ inline size_t ot_mut_floats(int K) { return (size_t)2 * kOtCols * tc_npad(K); }
 
+bool tc_persistent(int K, int64_t D, int max_rows) {
+  const int64_t blocks = ((int64_t)max_rows + kTcRows - 1) / kTcRows;
+  return (int64_t)(K <= 16 ? 16 : tc_npad(K)) * D * blocks >= kTcPersistentWork && (K > kTcMinK || max_rows >= kTcMinRows);
+}
+
 struct GmmLayout {
+  size_t tc;        // scratch of the persistent tensor-core kernels
   size_t coef, mnorm, gacc, epoch, status, mu_img, mut_img, r_img, rcoef, total;
   int tc_chunks;    // column chunks of the tensor-core dot products (whole clusters)
   int nchunk;       // D-chunks of the CUDA-core dots kernel
@@ -145,10 +167,12 @@ GmmLayout gmm_layout(int K, int64_t D, int max_rows, int T) {
   L.epoch = take(sizeof(GmmEpoch));
   L.status = take(sizeof(int32_t));
   L.tc_chunks = (int)((D + kTcCols - 1) / kTcCols + kTcCluster - 1) / kTcCluster * kTcCluster;  // whole clusters
-  L.mu_img = take((size_t)L.tc_chunks * tc_mu_chunk_floats(K) * sizeof(float));
+  const bool per = tc_persistent(K, D, max_rows);
+  L.tc = take(per ? pa::gmm_tc_layout(K, max_rows).total : 0);
+  L.mu_img = take(per ? 0 : (size_t)L.tc_chunks * tc_mu_chunk_floats(K) * sizeof(float));
   // the tensor-core output contraction (16 < K <= 64): the means' transposed
   // split image, the responsibilities' split image and the rows' scalars
-  const bool ot = K > kTcMinK && tc_npad(K) <= kOtMaxKp;
+  const bool ot = !per && K > kTcMinK && tc_npad(K) <= kOtMaxKp;
   L.mut_img = take(ot ? (size_t)((D + kOtCols - 1) / kOtCols) * ot_mut_floats(K) * sizeof(float) : 0);
   L.r_img = take(ot ? (size_t)((max_rows + kTcRows - 1) / kTcRows) * ot_img_floats(K) * sizeof(float) : 0);
   L.rcoef = take(ot ? (size_t)2 * max_rows * sizeof(float) : 0);
@@ -1177,6 +1201,7 @@ struct pa_gmm {
   bool tc_ok;   // the tensor-core dot products fit this device and these sizes
   bool use_tc;  // ... and are selected
   bool cl_ok;   // the single-kernel cluster form fits these sizes and this device
+  bool per;     // form 1 is the persistent kernels
   bool ot_ok;   // form 1 also takes the output contraction on the tensor cores (16 < K <= 64)
   int form;     // 0 CUDA-core dots + output kernel, 1 tensor-core dots + output kernel, 2 cluster form
 };
@@ -1248,7 +1273,11 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess && major == 10 && D % 4 == 0 && (reinterpret_cast<uintptr_t>(means_dev) & 15) == 0 &&
+  g->per = false;
+  if (e == cudaSuccess && tc_persistent(K, D, max_rows)) {
+    e = pa::gmm_tc_setup(K, &g->per);
+    g->tc_ok = g->per;
+  } else if (e == cudaSuccess && major == 10 && D % 4 == 0 && (reinterpret_cast<uintptr_t>(means_dev) & 15) == 0 &&
       tc_smem_bytes(K) + 2048 <= (size_t)optin) {
     e = cudaFuncSetAttribute(k_gmm_dots_tc<kTcCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tc_smem_bytes(K));
@@ -1264,7 +1293,7 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   // The tensor-core output contraction beside them: 16 < K <= 64 (padded
   // components fit one image of 128 rows x 64), whole kOtCols-column chunks.
   g->ot_ok = false;
-  if (e == cudaSuccess && g->tc_ok && K > kTcMinK && tc_npad(K) <= kOtMaxKp && D % kOtCols == 0 &&
+  if (e == cudaSuccess && g->tc_ok && !g->per && K > kTcMinK && tc_npad(K) <= kOtMaxKp && D % kOtCols == 0 &&
       ot_smem_bytes(K) + 4096 <= (size_t)optin) {
     e = cudaFuncSetAttribute(k_gmm_out_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ot_smem_bytes(K));
     if (e == cudaSuccess) {
@@ -1280,7 +1309,7 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   // shorter per-CTA chain wins (measured at 4x64x64: 30.1 vs 33.1 us per
   // Picard iteration); at K = 64 the tensor cores win (151.9 vs 170.4 us at
   // 4x128x128).
-  g->use_tc = g->tc_ok && K > kTcMinK;
+  g->use_tc = g->tc_ok && (K > kTcMinK || g->per);
   // The single-kernel cluster form for K <= 16 when D splits into kClSize
   // 16-byte-aligned column chunks whose tiles fit in shared memory and a
   // cluster of kClSize CTAs can be resident; then the default.
@@ -1317,7 +1346,7 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
         }
       }
     }
-    if (g->cl_ok) g->form = 2;
+    if (g->cl_ok && !g->use_tc) g->form = 2;
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);
   if (e != cudaSuccess) {
@@ -1348,6 +1377,18 @@ extern "C" pa_status pa_gmm_eps(pa_gmm* g, const float* batch_x_dev, const int32
   const size_t out_smem = (size_t)(g->K + kOutRows) * kOutCols * sizeof(float);
   const dim3 tc_grid(L.tc_chunks, (g->max_rows + kTcRows - 1) / kTcRows);
   cudaError_t e;
+  if (g->form == 1 && g->per) {  // any D, any alignment
+    const pa::GmmTcArgs a{batch_x_dev, g->means, coef, mnorm, miss_bt_dev, n_rows_dev, batch_eps_dev, g->ws + L.tc,
+                          status, g->K, g->T, g->max_rows, g->D};
+    e = pa::gmm_tc_launch(a, g->st);
+    g->launches += pa::kGmmTcLaunches;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      pa::set_error(std::string("pa_gmm_eps: ") + cudaGetErrorString(e));
+      return PA_ERR_CUDA;
+    }
+    return PA_OK;
+  }
   if (g->form == 2 && bulk && vec_out) {  // one kernel: cluster of kClSize CTAs per kClRows rows
     const int chunk = (int)(g->D / kClSize);
     e = pa::launch_ex(k_gmm_cluster<kClSize, kClRows>, dim3(kClSize, (g->max_rows + kClRows - 1) / kClRows),

@@ -296,6 +296,53 @@ def test_gmm_kernel_against_oracle(wname, n, max_rows, form):
     g.close()
 
 
+@pytest.mark.parametrize("K,D,n,cap,shift", [
+    (64, 65536, 118, 128, 0), (64, 65536, 1, 128, 0), (64, 32768, 128, 128, 0),  # one row block
+    (17, 40960, 129, 200, 0), (20, 16384, 257, 384, 0),   # row blocks with few rows, a block without rows
+    (65, 8192, 100, 100, 0), (128, 6000, 130, 260, 0),     # the means in two halves; a ragged last unit and tile
+    (33, 21846, 90, 100, 0), (40, 20001, 77, 130, 0),      # D % 4 != 0, odd: 4-byte copies
+    (64, 16400, 100, 128, 1),                              # rows 4 bytes past a 16-byte boundary
+    (16, 4096, 1500, 1600, 0), (5, 9000, 800, 800, 0),     # few components, many rows
+    (128, 64, 19590, 19600, 0),                            # more row blocks than CTAs
+    (100, 3000, 0, 256, 0)])                               # no rows
+def test_gmm_persistent_kernels(K, D, n, cap, shift):
+    """The persistent tensor-core denoiser (form 1 of a large problem) against
+    the fp64 oracle at the edges of its row blocks, column units and tiles,
+    twice in a row with bitwise equal results; rows past the count stay as
+    they were. Tolerance as for the other forms."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    w = W.SD15.with_(K=K, latent_shape=(1, 1, D))
+    a, mu, idx, x, miss = _gmm_rows(w, max(n, 1))
+    dev = torch.device("cuda")
+    g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
+    assert g.form() == 1
+    l0 = g.launches()
+    xd = torch.zeros(cap * D + shift, dtype=torch.float32, device=dev)[shift:].view(cap, D)
+    xd[:n] = torch.from_numpy(x[:n]).to(dev)
+    md = torch.zeros(cap, 2, dtype=torch.int32, device=dev)
+    md[:n] = torch.from_numpy(miss[:n]).to(dev)
+    nd = torch.tensor([n], dtype=torch.int32, device=dev)
+    outs = []
+    for _ in range(2):
+        out = torch.full((cap * D + shift,), float("nan"), device=dev)[shift:].view(cap, D)
+        g.eps(xd.data_ptr(), md.data_ptr(), nd.data_ptr(), out)
+        outs.append(out)
+    assert g.launches() - l0 == 6
+    torch.cuda.synchronize()
+    from paper_2609_36522_gb300 import abi
+    abi.pa_gmm_check(g.h)
+    some = np.unique(np.concatenate([np.arange(min(n, 40)), np.arange(max(0, n - 40), n)])).astype(int)
+    if n:
+        got = outs[0][torch.from_numpy(some).to(dev)].cpu().numpy().astype(np.float64)
+        want = gmm_eps(x[some].astype(np.float64), a[idx[some]], mu.astype(np.float64), w.gmm_std)
+        rel = np.abs(got - want).max(axis=1) / np.abs(want).max(axis=1)
+        assert rel.max() <= 2e-6, rel.max()
+    assert torch.equal(outs[1][:n], outs[0][:n])
+    assert torch.isfinite(outs[0][:n]).all() and torch.isnan(outs[0][n:]).all()
+    g.close()
+
+
 def test_gmm_in_cuda_graph():
     """The denoiser captured in a CUDA graph and replayed gives the eager
     result (bitwise), with a device row count that changes between replays."""
