@@ -57,12 +57,26 @@ __device__ __forceinline__ void copy_row(const Dev& d, int b, int src_state, int
   }
 }
 
-// The gather of a plan already in memory (copy par): after the first plan,
-// and after the one-CTA planner.
+// The gather of a plan already in memory (copy par), after the one-CTA planner.
+// Its CTAs also report the sums that the plan was made from (set par ^ 1,
+// divided by D) and clear the set that the planned iteration adds into: the
+// divisions by D are fp64, which one SM of this GPU does two per clock of.
 template <int VEC>
 __global__ void __launch_bounds__(kGatherThreads) k_gather(Dev d, int par) {
   pdl_wait();  // everything read here comes from the kernel that planned
   pdl_trigger();  // the successor may now run its prologue
+  {
+    const int npair = d.B * d.P, old = par ^ 1;
+    const int64_t step = (int64_t)gridDim.x * gridDim.y * kGatherThreads;
+    for (int64_t q = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kGatherThreads + threadIdx.x; q < npair; q += step) {
+      const double* e = d.acc + ((size_t)(old * 2 + 0) * npair + q) * kAccStride;
+      const double* dl = d.acc + ((size_t)(old * 2 + 1) * npair + q) * kAccStride;
+      d.red_err[q] = (float)(__ldcg(e) * d.inv_d);
+      d.red_del[q] = (float)(__ldcg(dl) * d.inv_d);
+      d.acc[((size_t)(par * 2 + 0) * npair + q) * kAccStride] = 0.0;
+      d.acc[((size_t)(par * 2 + 1) * npair + q) * kAccStride] = 0.0;
+    }
+  }
   const int n = d.ctl->n_miss;
   const Traj* tr = d.traj + par * d.B;
   for (int r = blockIdx.y; r < n; r += gridDim.y) {
@@ -322,15 +336,12 @@ constexpr int kFusedMaxPairs = 1024;  // B*P planned in every CTA at most; beyon
 constexpr int kFusedPreferPairs = 512;
 static_assert(kFusedMaxPairs <= 32 * 32, "decide_par keeps one miss mask per 32-position chunk, 32 of them");
 
-// The complete sums read from global memory (one-CTA planner).
-struct RedSums {
-  const double* e;
-  const double* dl;
-  double inv_d, tol_d, thr_d;
-  __device__ double err(int q) const { return __ldcg(e + (size_t)q * kAccStride) * inv_d; }
-  __device__ double del(int q) const { return __ldcg(dl + (size_t)q * kAccStride) * inv_d; }
-  __device__ bool conv(int q) const { return sum_le(__ldcg(e + (size_t)q * kAccStride), tol_d); }
-  __device__ bool near(int q) const { return sum_lt(__ldcg(dl + (size_t)q * kAccStride), thr_d); }
+// The decision's inputs as bits in shared memory (one-CTA planner).
+struct RedBits {
+  const unsigned* conv_w;
+  const unsigned* near_w;
+  __device__ bool conv(int q) const { return (conv_w[q >> 5] >> (q & 31)) & 1u; }
+  __device__ bool near(int q) const { return (near_w[q >> 5] >> (q & 31)) & 1u; }
 };
 
 // The miss of batch row r < ds.total from the decision's chunk bits: chunk c
@@ -386,26 +397,46 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanPerSm) k_plan_gather(Dev d,
 }
 
 // One-CTA planner for B*P beyond kFusedPreferPairs (without adaptation) or
-// kFusedMaxPairs: reads the sums from memory; a separate gather follows.
+// kFusedMaxPairs; a separate gather follows. The sums are read once, all loads
+// of a thread in flight together, and kept as the bits the decision needs: it
+// looks at each position several times, and a trip to memory every time (1,600
+// pairs) took 15 us a launch.
 constexpr int kPlanOneThreads = 1024;
+constexpr int kPlanOneWords = kMaxBatch * kMaxWindow / 32;
 
 __global__ void __launch_bounds__(kPlanOneThreads) k_plan_one(Dev d, int par) {
   __shared__ DecideShared ds;
-  const int npair = d.B * d.P;
+  __shared__ unsigned s_conv[kPlanOneWords], s_near[kPlanOneWords];
+  const int npair = d.B * d.P, lane = threadIdx.x & 31;
   decide_load<kPlanOneThreads>(d, ds, par);
   pdl_wait();  // the sums come from the update kernel
   pdl_trigger();  // the successor may now run its prologue
   const double* acc_e = d.acc + (size_t)(par * 2 + 0) * npair * kAccStride;
   const double* acc_d = d.acc + (size_t)(par * 2 + 1) * npair * kAccStride;
-  const RedSums red{acc_e, acc_d, d.inv_d, d.tol_d, d.thr_d};
-  decide_run<kPlanOneThreads>(d, ds, red, par, true, -1);
-  double* nxt = d.acc + (size_t)((par ^ 1) * 2) * npair * kAccStride;
-  for (int q = threadIdx.x; q < npair; q += kPlanOneThreads) {
-    d.red_err[q] = (float)red.err(q);
-    d.red_del[q] = (float)red.del(q);
-    nxt[(size_t)q * kAccStride] = 0.0;
-    nxt[((size_t)npair + q) * kAccStride] = 0.0;
+  constexpr int kAhead = 4;
+  for (int q0 = threadIdx.x; q0 - lane < npair; q0 += kAhead * kPlanOneThreads) {
+    double e[kAhead], dl[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int q = q0 + u * kPlanOneThreads;
+      e[u] = dl[u] = 0.0;
+      if (q < npair) {
+        e[u] = __ldcg(acc_e + (size_t)q * kAccStride);
+        dl[u] = __ldcg(acc_d + (size_t)q * kAccStride);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int q = q0 + u * kPlanOneThreads;
+      const unsigned cm = __ballot_sync(0xffffffffu, q < npair && sum_le(e[u], d.tol_d));
+      const unsigned nm = __ballot_sync(0xffffffffu, q < npair && sum_lt(dl[u], d.thr_d));
+      if (lane == 0 && q < npair) {
+        s_conv[q >> 5] = cm;
+        s_near[q >> 5] = nm;
+      }
+    }
   }
+  decide_run<kPlanOneThreads>(d, ds, RedBits{s_conv, s_near}, par, true, -1);  // starts with a barrier
 }
 
 }  // namespace

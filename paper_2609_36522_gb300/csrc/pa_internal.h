@@ -246,8 +246,12 @@ struct Bf16Row<1> {
 // up to 65536 values), far beyond any tolerance the decision compares it
 // with. Rounding up keeps a nonzero partial nonzero (tol = 0 stays exact) and
 // moves a sum by at most one 2^-32 per CTA.
+// In fp32, which is exact here: from 2^-9 on an fp32 value is a multiple of
+// 2^-32 already, and below it the scaled value and its ceiling are fp32 values.
+// (This GPU's fp64 unit takes two operations per clock and SM; only the
+// widening for the fp64 atomic is left to it.)
 __device__ __forceinline__ double quantize_partial(float v) {
-  return ceil((double)v * 4294967296.0) * (1.0 / 4294967296.0);
+  return (double)(fabsf(v) < 0.001953125f ? ceilf(v * 4294967296.f) * (1.f / 4294967296.f) : v);
 }
 
 // Eq. 2 / Eq. 5 tests on an accumulated (non-negative) sum, by bit pattern.

@@ -32,6 +32,21 @@ def test_rounding_is_up_by_less_than_one_step_and_keeps_nonzero():
     assert np.array_equal(q * SCALE, np.round(q * SCALE))   # multiples of 2^-32
 
 
+def test_fp32_form_of_the_rounding_is_the_same():
+    """The kernels round in fp32: values from 2^-9 on are multiples of 2^-32 as
+    they are, smaller ones are scaled, rounded up and scaled back exactly."""
+    rng = np.random.default_rng(4)
+    edge = np.float32(2.0 ** -9)
+    v = np.concatenate([_partials(rng, 20000), np.exp(rng.uniform(-100, 85, 20000)).astype(np.float32),
+                        np.array([0.0, 1e-45, 2.0 ** -33, 2.0 ** -32, edge, np.nextafter(edge, np.float32(0)),
+                                  np.nextafter(edge, np.float32(1)), 3e38, np.inf], np.float32)])
+    v = np.concatenate([v, -v])
+    with np.errstate(over="ignore"):
+        got = np.where(np.abs(v) < edge, np.ceil(v * np.float32(SCALE)) * np.float32(1 / SCALE), v)
+    assert got.dtype == np.float32
+    assert np.array_equal(got.astype(np.float64), quantize_up(v))
+
+
 def test_quantized_sums_are_exact_in_every_order():
     rng = np.random.default_rng(2)
     checked = 0
