@@ -127,8 +127,9 @@ PA_API pa_status pa_set_noise(pa_solver* s, double eta, const float* noise_dev);
  * direction is inferred from the address). All states of the first window are
  * x_init (Sec. 2.1 initial trajectory estimate); every first-window timestep is
  * a first entry, hence a miss (Sec. 2.2). Clears the cache and counters,
- * plans the first iteration and gathers its batch (two kernels), all
- * asynchronous on the solver's stream. May be called again at any time to
+ * plans the first iteration and gathers its batch (one kernel, which reads
+ * x_init itself where that is in the current device's memory; a copy comes
+ * first otherwise), all asynchronous on the solver's stream. May be called again at any time to
  * restart. */
 PA_API pa_status pa_init(pa_solver* s, const float* x_init);
 
@@ -217,15 +218,16 @@ PA_API pa_status pa_poll_end(pa_solver* s, int* n_active);
  * issues an even number n >= 2 of iterations (pa_step_async, its denoiser's
  * launches on the solver's stream reading the miss count on the device,
  * pa_submit_eps; an even number because the iterations alternate two plan
- * copies); pa_loop_capture_end appends a one-thread kernel that sets the
+ * copies); pa_loop_capture_end has the last iteration's planning kernel (or,
+ * where planning is not one launch, a one-thread kernel behind it) set the
  * node's condition (repeat while a trajectory is active, the device status is
- * clean and fewer than T / n + 2 passes have run: the window advances at
- * least one step per iteration, so T iterations always suffice, and the pass
+ * clean and fewer than T + 2 iterations have run: the window advances at
+ * least one step per iteration, so T iterations always suffice, and the
  * limit bounds the loop whatever the counters say; iterations after the end
  * do nothing), closes the capture and instantiates the graph. Nothing runs
  * during the capture, and the host state returns to what it was at
  * pa_loop_capture_begin. pa_loop_launch(s, x_init) is pa_init followed by the
- * whole loop: it enqueues the copy of x_init ([batch][D] fp32, HOST or
+ * whole loop: it enqueues x_init ([batch][D] fp32, HOST or
  * DEVICE) into state 0, pa_init's kernel (the first plan, its batch, cleared
  * sums and counters, the loop's pass counter among them) and one launch of
  * the graph, and returns; then

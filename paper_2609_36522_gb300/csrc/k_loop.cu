@@ -1,8 +1,9 @@
-// The device-side test of the generation loop (pa_loop_*): a CUDA graph whose
-// conditional WHILE node holds two Picard iterations (Sec. 2.1, Eq. 1: the
-// window slides until every trajectory has reached T, Eq. 2) and, last in its
-// body, this kernel. One thread reads the counters that the planning kernel
-// published and sets the node's condition: run the body again while a
+// The device-side test of the generation loop (pa_loop_*) where planning is not
+// one launch (k_solver.cu's planning kernel sets the condition itself): a CUDA
+// graph whose conditional WHILE node holds an even number of Picard iterations
+// (Sec. 2.1, Eq. 1: the window slides until every trajectory has reached T,
+// Eq. 2) and, last in its body, this kernel. One thread reads the counters that
+// the plan published and sets the node's condition: run the body again while a
 // trajectory is active, the device status is clean and fewer than `limit`
 // passes have run. The pass limit bounds the loop whatever the counters say.
 #include "pa_loop.h"

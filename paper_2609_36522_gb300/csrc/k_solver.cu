@@ -34,14 +34,17 @@ __device__ __forceinline__ void set_status(Ctl* c, int code) {
 constexpr int kGatherThreads = 256;
 constexpr int kGatherUnroll = 16;
 
+// This CTA's part (blockIdx.x of gridDim.x) of a row of D values, to one
+// place or two.
 template <int VEC>
-__device__ __forceinline__ void copy_row(const Dev& d, int b, int src_state, int r) {
+__device__ __forceinline__ void copy_part(int64_t D, const float* src, float* dst, float* dst2) {
   using T = typename std::conditional<VEC == 4, float4, float>::type;
-  const int64_t nvec = d.D / VEC;
+  const int64_t nvec = D / VEC;
   const int64_t stride = (int64_t)gridDim.x * kGatherThreads;
   const int64_t base = (int64_t)blockIdx.x * kGatherThreads + threadIdx.x;
-  const T* from = reinterpret_cast<const T*>(d.X + ((int64_t)b * (d.P + 1) + src_state % (d.P + 1)) * d.D);
-  T* to = reinterpret_cast<T*>(d.batch_x + (int64_t)r * d.D);
+  const T* from = reinterpret_cast<const T*>(src);
+  T* to = reinterpret_cast<T*>(dst);
+  T* to2 = reinterpret_cast<T*>(dst2);
   for (int64_t v0 = base; v0 < nvec; v0 += stride * kGatherUnroll) {
     T buf[kGatherUnroll];
 #pragma unroll
@@ -52,9 +55,17 @@ __device__ __forceinline__ void copy_row(const Dev& d, int b, int src_state, int
 #pragma unroll
     for (int u = 0; u < kGatherUnroll; ++u) {
       const int64_t v = v0 + u * stride;
-      if (v < nvec) to[v] = buf[u];
+      if (v < nvec) {
+        to[v] = buf[u];
+        if (to2) to2[v] = buf[u];
+      }
     }
   }
+}
+
+template <int VEC>
+__device__ __forceinline__ void copy_row(const Dev& d, int b, int src_state, int r) {
+  copy_part<VEC>(d.D, d.X + ((int64_t)b * (d.P + 1) + src_state % (d.P + 1)) * d.D, d.batch_x + (int64_t)r * d.D, nullptr);
 }
 
 // The gather of a plan already in memory (copy par), after the one-CTA planner.
@@ -86,8 +97,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(Dev d, int par) {
 }
 
 // ---------------------------------------------------------------------------
-// First iteration (after pa_init's copy of x_init into state 0): every
-// timestep of every first window enters for the first time, hence is a miss
+// First iteration. x: x_init in device memory, which this kernel also copies
+// into state 0; NULL: a copy has put it there. Every timestep of every first window enters for the first time, hence is a miss
 // (Sec. 2.2); states 1..p are lazy copies of state 0 = x_init, so the frontier
 // e starts at 0 and batch row r = b p0 + j is state 0 of trajectory b. One
 // launch on the planning kernel's grid: each CTA copies its part of its batch
@@ -97,8 +108,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(Dev d, int par) {
 // kAccStride-th) and the fused step's barrier counter; CTA (0, 0) writes the
 // trajectories, counters and the plan's counter copy 0.
 template <int VEC>
-__global__ void __launch_bounds__(kGatherThreads) k_init(Dev d) {
-  pdl_wait();  // x_init was copied into state 0 just before
+__global__ void __launch_bounds__(kGatherThreads) k_init(Dev d, const float* __restrict__ x) {
+  pdl_wait();  // the kernels and copies before are complete
   pdl_trigger();
   const int p0 = min(d.P, d.T);
   const int npair = d.B * d.P;
@@ -144,7 +155,28 @@ __global__ void __launch_bounds__(kGatherThreads) k_init(Dev d) {
       d.pc[0] = pc;
     }
   }
-  for (int r = blockIdx.y; r < d.B * p0; r += gridDim.y) copy_row<VEC>(d, r / p0, 0, r);
+  for (int r = blockIdx.y; r < d.B * p0; r += gridDim.y) {
+    const int b = r / p0;
+    float* state0 = d.X + (int64_t)b * (d.P + 1) * d.D;
+    copy_part<VEC>(d.D, x ? x + (int64_t)b * d.D : state0, d.batch_x + (int64_t)r * d.D,
+                   x && r == b * p0 ? state0 : nullptr);
+  }
+}
+
+// The poll of a generation whose x_T goes to device memory, in one launch in
+// place of two copies (the copy engine takes about 4 us for each, mostly
+// between them): the states in the slot of t = T to out [B][D], the counters to
+// pinned host memory.
+template <int VEC>
+__global__ void __launch_bounds__(kGatherThreads) k_poll(Dev d, float* __restrict__ out, Ctl* host) {
+  pdl_wait();  // the counters and states come from the kernels before
+  pdl_trigger();
+  const int b = blockIdx.y;
+  if (blockIdx.x == 0 && b == 0 && threadIdx.x == 0) {
+    *host = *d.ctl;
+    __threadfence_system();
+  }
+  copy_part<VEC>(d.D, d.X + ((int64_t)b * (d.P + 1) + d.T % (d.P + 1)) * d.D, out + (int64_t)b * d.D, nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -367,8 +399,16 @@ __device__ __forceinline__ bool row_miss(const DecideShared& ds, int B, int P, i
   return true;
 }
 
-template <int VEC>
-__global__ void __launch_bounds__(kPlanThreads, kPlanPerSm) k_plan_gather(Dev d, int par) {
+// COND: the planning kernel of the last iteration in a captured generation
+// loop's body, which also sets the condition of the loop's node (set_plan_cond;
+// in every iteration, or only as code not run, it cost each 0.5 us: the call
+// makes the decision spill): go on while a trajectory is active, the
+// device status is clean and fewer than lc.limit iterations have run (the
+// window advances at least one step in each, so T of them always suffice, and
+// the limit bounds the loop whatever the counters say).
+
+template <int VEC, bool COND>
+__global__ void __launch_bounds__(kPlanThreads, kPlanPerSm) k_plan_gather(Dev d, int par, LoopCond lc) {
   __shared__ DecideShared ds;
   const bool publish = blockIdx.x == 0 && blockIdx.y == 0;
   decide_load<kPlanThreads>(d, ds, par);
@@ -379,6 +419,15 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanPerSm) k_plan_gather(Dev d,
   const bool one_row = (int)gridDim.y >= d.B * d.P;  // every batch row has its own CTA
   decide_par(d, ds, par, publish ? 0 : -1, 1, one_row ? (int)blockIdx.y : -1);
   __syncthreads();  // the plan (the batch rows of this CTA) is known
+  if constexpr (COND) {
+    if (publish && threadIdx.x == 0) {
+      int act = 0;
+      if (ds.active != 0)
+        for (int b = 0; b < d.B; ++b) act += ds.pn[b] > 0;
+      const bool more = act > 0 && __ldcg(&d.ctl->status) == kDevOk && ds.iter + 1 < lc.limit;
+      cudaGraphSetConditional(lc.handle, more ? 1u : 0u);
+    }
+  }
   if (one_row) {
     if ((int)blockIdx.y < ds.total && ds.target_b >= 0) {
       const int b = ds.target_b;
@@ -499,15 +548,37 @@ cudaError_t split_grid(const Dev& d, int per_sm, dim3* out) {
 }
 }  // namespace
 
-cudaError_t launch_init(const Dev& d, cudaStream_t st) {
+cudaError_t launch_init(const Dev& d, const float* x, cudaStream_t st) {
   dim3 g;
   const cudaError_t e = split_grid(d, kPlanPerSm, &g);
   if (e != cudaSuccess) return e;
-  if (d.D % 4 == 0) return launch_ex(k_init<4>, g, dim3(kGatherThreads), 0, st, 0, d);
-  return launch_ex(k_init<1>, g, dim3(kGatherThreads), 0, st, 0, d);
+  if (d.D % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0)
+    return launch_ex(k_init<4>, g, dim3(kGatherThreads), 0, st, 0, d, x);
+  return launch_ex(k_init<1>, g, dim3(kGatherThreads), 0, st, 0, d, x);
+}
+
+cudaError_t launch_poll(const Dev& d, float* out, Ctl* host, cudaStream_t st) {
+  const bool vec = d.D % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  const int64_t nvec = d.D / (vec ? 4 : 1), want = (nvec + kGatherThreads * 4 - 1) / (kGatherThreads * 4);
+  const dim3 g((int)(want < 64 ? want : 64), d.B);
+  if (vec) return launch_ex(k_poll<4>, g, dim3(kGatherThreads), 0, st, 0, d, out, host);
+  return launch_ex(k_poll<1>, g, dim3(kGatherThreads), 0, st, 0, d, out, host);
+}
+
+cudaError_t set_plan_cond(cudaGraphNode_t node, const Dev& d, int par, LoopCond lc) {
+  cudaKernelNodeParams kp = {};
+  const cudaError_t e = cudaGraphKernelNodeGetParams(node, &kp);
+  if (e != cudaSuccess) return e;
+  Dev dev = d;
+  void* args[] = {&dev, &par, &lc};
+  kp.func = d.D % 4 == 0 ? reinterpret_cast<void*>(k_plan_gather<4, true>) : reinterpret_cast<void*>(k_plan_gather<1, true>);
+  kp.kernelParams = args;
+  kp.extra = nullptr;
+  return cudaGraphKernelNodeSetParams(node, &kp);
 }
 
 cudaError_t launch_plan(const Dev& d, int par, cudaStream_t st, int* launches) {
+  const LoopCond lc{};
   const int npair = d.B * d.P;
   if (npair <= kFusedPreferPairs || (d.adapt && npair <= kFusedMaxPairs)) {
     *launches = 1;
@@ -515,8 +586,8 @@ cudaError_t launch_plan(const Dev& d, int par, cudaStream_t st, int* launches) {
     dim3 g;
     const cudaError_t e = split_grid(d, kPlanPerSm, &g);
     if (e != cudaSuccess) return e;
-    if (d.D % 4 == 0) return launch_ex(k_plan_gather<4>, g, dim3(kPlanThreads), 0, st, 0, d, par);
-    return launch_ex(k_plan_gather<1>, g, dim3(kPlanThreads), 0, st, 0, d, par);
+    if (d.D % 4 == 0) return launch_ex(k_plan_gather<4, false>, g, dim3(kPlanThreads), 0, st, 0, d, par, lc);
+    return launch_ex(k_plan_gather<1, false>, g, dim3(kPlanThreads), 0, st, 0, d, par, lc);
   }
   *launches = 2;
   cudaError_t e = launch_ex(k_plan_one, dim3(1), dim3(kPlanOneThreads), 0, st, 0, d, par);

@@ -808,10 +808,13 @@ extern "C" pa_status pa_srds_init(pa_srds* h, const float* x_init) {
   if (!h || !x_init) return s_fail("pa_srds_init: NULL argument", PA_ERR_ARG);
   if (h->loop_capturing) return s_fail("pa_srds_init: a generation is being captured", PA_ERR_STATE);
   const SDev& d = h->d;
-  // x_init (host or device) is staged in batch_x, then widened into U_0
-  cudaError_t e = cudaMemcpyAsync(d.batch_x, x_init, (size_t)d.B * d.D * sizeof(float), cudaMemcpyDefault, h->st);
+  // x_init is widened into U_0 from where it lies, or, off this device's
+  // memory, staged in batch_x first
+  const bool here = pa::on_current_device(x_init);
+  cudaError_t e = cudaSuccess;
+  if (!here) e = cudaMemcpyAsync(d.batch_x, x_init, (size_t)d.B * d.D * sizeof(float), cudaMemcpyDefault, h->st);
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_init: ") + cudaGetErrorString(e), PA_ERR_CUDA);
-  e = pa::launch_ex(k_srds_init, dim3(32, d.B), dim3(kSThreads), 0, h->st, 0, d, (const float*)d.batch_x);
+  e = pa::launch_ex(k_srds_init, dim3(32, d.B), dim3(kSThreads), 0, h->st, 0, d, here ? x_init : (const float*)d.batch_x);
   h->launches += 1;
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_init: ") + cudaGetErrorString(e), PA_ERR_CUDA);
   h->iter = 0;
@@ -930,10 +933,12 @@ extern "C" pa_status pa_srds_result(pa_srds* h, float* x_out) {
   if (h->loop_capturing) return s_fail("pa_srds_result: synchronises; not inside a capture", PA_ERR_STATE);
   if (h->phase != 2) return s_fail("pa_srds_result: not finished", PA_ERR_STATE);
   const SDev& d = h->d;
-  // U_N narrowed to fp32 in batch_x (free once sampling is done), then copied out
-  cudaError_t e = pa::launch_ex(k_srds_store, dim3(32, d.B), dim3(256), 0, h->st, 0, d, d.batch_x, d.N);
+  // U_N narrowed to fp32 where it is wanted, or, off this device's memory, in
+  // batch_x (free once sampling is done) and then copied out
+  const bool here = pa::on_current_device(x_out);
+  cudaError_t e = pa::launch_ex(k_srds_store, dim3(32, d.B), dim3(256), 0, h->st, 0, d, here ? x_out : d.batch_x, d.N);
   h->launches++;
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !here)
     e = cudaMemcpyAsync(x_out, d.batch_x, (size_t)d.B * d.D * sizeof(float), cudaMemcpyDefault, h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_result: ") + cudaGetErrorString(e), PA_ERR_CUDA);

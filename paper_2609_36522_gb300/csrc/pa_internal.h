@@ -163,6 +163,7 @@ constexpr uint32_t kWaitLimit = 1u << 17;  // tries of an mbarrier wait (~1.3 s 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+bool on_current_device(const void* p);  // an address in the current device's memory (pa_solver.cpp)
 bool pdl_enabled();  // false when the environment sets PA_DISABLE_PDL=1
 
 // cudaLaunchKernelEx with the PDL attribute (when enabled), an optional
@@ -323,11 +324,23 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* ctr, unsigned long
 // Kernel launchers (k_solver.cu). Each returns the launch error. par = k mod 2
 // for iteration k: the copy of the plan the kernel reads (and the accumulator
 // set the update kernels add into).
-cudaError_t launch_init(const Dev& d, cudaStream_t st);  // first plan, its batch, cleared sums
+// first plan, its batch, cleared sums; x: x_init in device memory ([B][D]), or
+// NULL when it has been copied into state 0
+cudaError_t launch_init(const Dev& d, const float* x, cudaStream_t st);
+// x_T to out (device memory) and the counters to host (pinned memory)
+cudaError_t launch_poll(const Dev& d, float* out, Ctl* host, cudaStream_t st);
 cudaError_t launch_gather(const Dev& d, int par, cudaStream_t st);
 cudaError_t launch_update_plain(const Dev& d, const float* batch_eps, int par, cudaStream_t st);
+// The condition of a captured generation loop's node: limit = 0: none.
+struct LoopCond {
+  cudaGraphConditionalHandle handle;
+  int32_t limit;
+};
 // the decision after iteration k (par = k mod 2) and the gather of iteration k+1
+// (one launch or two)
 cudaError_t launch_plan(const Dev& d, int par, cudaStream_t st, int* launches);
+// Make a captured node of launch_plan's one-launch form set a loop's condition.
+cudaError_t set_plan_cond(cudaGraphNode_t node, const Dev& d, int par, LoopCond lc);
 // k_update_bulk.cu
 cudaError_t launch_update_bulk(const Dev& d, const float* batch_eps, int par, cudaStream_t st);
 bool update_bulk_supported(const Dev& d, const float* batch_eps);

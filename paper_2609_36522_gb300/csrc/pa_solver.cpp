@@ -19,6 +19,16 @@ namespace pa {
 static thread_local std::string g_err;
 void set_error(const std::string& msg) { g_err = msg; }
 
+bool on_current_device(const void* p) {
+  cudaPointerAttributes a = {};
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();  // not an address the runtime knows: the copies sort it out
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 bool pdl_enabled() {
   static const bool on = [] {
     const char* v = std::getenv("PA_DISABLE_PDL");
@@ -56,6 +66,8 @@ struct pa_solver {
   cudaGraphExec_t loop_exec;
   cudaGraphConditionalHandle loop_cond;
   bool loop_capturing;     // between pa_loop_capture_begin and _end
+  cudaGraphNode_t plan_node;  // the last captured iteration's planning kernel, if that is one launch
+  int plan_par;               // ... and the plan copy it reads
   bool looped;             // a loop was launched since pa_init: host-side stepping is closed
   int64_t loop_k0, loop_launches0;  // s->k and s->launches when the capture began
   std::vector<double> alphas;  // the schedule, kept for pa_set_noise
@@ -151,6 +163,19 @@ cudaError_t copy_xt(pa_solver* s, float* x_out) {
                            (size_t)d.D * sizeof(float), d.B, cudaMemcpyDefault, s->st);
 }
 
+// The node captured last on a stream under capture (NULL: not exactly one).
+cudaGraphNode_t last_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t n = 0;
+  if (cudaStreamGetCaptureInfo(st, &cs, nullptr, nullptr, &deps, &edges, &n) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  return cs == cudaStreamCaptureStatusActive && n == 1 ? deps[0] : nullptr;
+}
+
 // Let go of a loop graph whose capture the runtime invalidated, without
 // destroying it: destroying such a graph crashed the host process inside the
 // CUDA runtime. The graph leaks; the handle can capture again.
@@ -181,12 +206,27 @@ bool loop_busy(pa_solver* s, const char* where) {
   return true;
 }
 
-// Enqueue the copy of x_init ([batch][D], host or device) into state 0 of
-// every trajectory; the rest of the first window is lazy.
-cudaError_t copy_x_init(pa_solver* s, const float* x_init) {
+// Enqueue the start of a generation: x_init ([batch][D], host or device) into
+// state 0 of every trajectory (the rest of the first window is lazy), the first
+// plan (every timestep a first entry), its batch, both sets of the reductions'
+// (and the Anderson Gram sums') accumulators cleared: one kernel, which reads
+// x_init itself where that lies in this device's memory.
+cudaError_t begin_generation(pa_solver* s, const float* x_init) {
   const pa::Dev& d = s->d;
-  return cudaMemcpy2DAsync(d.X, (size_t)(d.P + 1) * d.D * sizeof(float), x_init, (size_t)d.D * sizeof(float),
-                           (size_t)d.D * sizeof(float), d.B, cudaMemcpyDefault, s->st);
+  if (pa::on_current_device(x_init)) return pa::launch_init(d, x_init, s->st);
+  const cudaError_t e = cudaMemcpy2DAsync(d.X, (size_t)(d.P + 1) * d.D * sizeof(float), x_init, (size_t)d.D * sizeof(float),
+                                          (size_t)d.D * sizeof(float), d.B, cudaMemcpyDefault, s->st);
+  return e == cudaSuccess ? pa::launch_init(d, nullptr, s->st) : e;
+}
+
+// Enqueue the copies of x_T into x_out (unless NULL) and of the counters into
+// `mirror` (pinned): one kernel for an x_out in this device's memory, else two
+// copies (a kernel's writes across to host memory are no quicker).
+cudaError_t copy_outcome(pa_solver* s, float* x_out, pa::Ctl* mirror) {
+  if (x_out && pa::on_current_device(x_out)) return pa::launch_poll(s->d, x_out, mirror, s->st);
+  cudaError_t e = x_out ? copy_xt(s, x_out) : cudaSuccess;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mirror, s->d.ctl, sizeof(pa::Ctl), cudaMemcpyDeviceToHost, s->st);
+  return e;
 }
 
 }  // namespace
@@ -310,6 +350,7 @@ pa_status pa_create(pa_solver** out, int T, int window, const int64_t* latent_sh
   s->loop_exec = nullptr;
   s->loop_cond = 0;
   s->loop_capturing = s->looped = false;
+  s->plan_node = nullptr;
   s->loop_k0 = s->loop_launches0 = 0;
   cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&s->host_ctl), 3 * sizeof(pa::Ctl), cudaHostAllocDefault);
   if (e != cudaSuccess) {
@@ -361,13 +402,9 @@ pa_status pa_set_noise(pa_solver* s, double eta, const float* noise_dev) {
 pa_status pa_init(pa_solver* s, const float* x_init) {
   if (!s) return arg_fail("pa_init: solver is NULL");
   if (!x_init) return arg_fail("pa_init: x_init is NULL");
-  cudaError_t e = copy_x_init(s, x_init);
-  if (e != cudaSuccess) return cuda_fail("pa_init: copy x_init", e);
-  // the first plan (every timestep a first entry), its batch, both sets of the
-  // reductions' (and the Anderson Gram sums') accumulators cleared: one kernel
-  e = pa::launch_init(s->d, s->st);
+  const cudaError_t e = begin_generation(s, x_init);
+  if (e != cudaSuccess) return cuda_fail("pa_init", e);
   s->launches += 1;
-  if (e != cudaSuccess) return cuda_fail("pa_init: launch", e);
   s->k = 0;
   s->looped = false;
   s->state = St::Ready;
@@ -475,6 +512,12 @@ pa_status pa_submit_eps(pa_solver* s, const float* batch_eps_dev) {
     e = pa::launch_plan(s->d, par, s->st, &nl);
     s->launches += nl;
     if (e != cudaSuccess) return cuda_fail("pa_submit_eps: plan", e);
+    if (s->loop_capturing) {
+      s->plan_node = nl == 1 ? last_captured(s->st) : nullptr;
+      s->plan_par = par;
+    }
+  } else {
+    s->plan_node = nullptr;
   }
   s->k++;
   s->state = St::Ready;
@@ -497,18 +540,20 @@ pa_status pa_result(pa_solver* s, float* x_out) {
   if (!s) return arg_fail("pa_result: solver is NULL");
   if (!x_out) return arg_fail("pa_result: x_out is NULL");
   if (s->state != St::Done) return state_fail("pa_result");
-  const cudaError_t e = copy_xt(s, x_out);
+  cudaError_t e = copy_outcome(s, x_out, s->host_ctl);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   if (e != cudaSuccess) return cuda_fail("pa_result", e);
-  return sync_ctl(s, "pa_result");
+  return check_ctl(*s->host_ctl, "pa_result");
 }
 
 pa_status pa_poll_result(pa_solver* s, float* x_out, int* n_active) {
   if (!s) return arg_fail("pa_poll_result: solver is NULL");
   if (!x_out) return arg_fail("pa_poll_result: x_out is NULL");
   if (s->state != St::Ready && s->state != St::Done) return state_fail("pa_poll_result");
-  cudaError_t e = copy_xt(s, x_out);
+  cudaError_t e = copy_outcome(s, x_out, s->host_ctl);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   if (e != cudaSuccess) return cuda_fail("pa_poll_result", e);
-  const pa_status r = sync_ctl(s, "pa_poll_result");
+  const pa_status r = check_ctl(*s->host_ctl, "pa_poll_result");
   if (r != PA_OK) return r;
   if (n_active) *n_active = s->host_ctl->n_active;
   if (s->host_ctl->n_active != 0) return PA_OK;
@@ -531,9 +576,7 @@ pa_status pa_poll_begin(pa_solver* s, float* x_out) {
     return PA_ERR_STATE;
   }
   const int slot = (s->poll_head + s->poll_count) & 1;
-  if (x_out) e = copy_xt(s, x_out);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&s->host_ring[slot], s->d.ctl, sizeof(pa::Ctl), cudaMemcpyDeviceToHost, s->st);
+  e = copy_outcome(s, x_out, &s->host_ring[slot]);
   if (e == cudaSuccess) e = cudaEventRecord(s->poll_ev[slot], s->st);
   if (e != cudaSuccess) return cuda_fail("pa_poll_begin", e);
   s->poll_count++;
@@ -603,6 +646,7 @@ pa_status pa_loop_capture_begin(pa_solver* s) {
     return cuda_fail("pa_loop_capture_begin", e);
   }
   s->loop_capturing = true;
+  s->plan_node = nullptr;
   s->loop_k0 = s->k;
   s->loop_launches0 = s->launches;
   return PA_OK;
@@ -617,9 +661,12 @@ pa_status pa_loop_capture_end(pa_solver* s) {
   const int64_t n_body = s->k - s->loop_k0;  // iterations in the body
   const bool two = s->state == St::Ready && n_body >= 2 && n_body % 2 == 0;
   cudaError_t e = cudaSuccess;
-  // at most T iterations reach t = T (the window advances by at least one
-  // step in each): T / n_body + 2 passes cover them
-  if (two) e = pa::launch_loop_cond(s->loop_cond, s->d.ctl, (int32_t)(s->d.T / n_body + 2), s->st);
+  // the last iteration's planning kernel sets the condition where it is one
+  // launch, else a kernel of its own that follows. At most T iterations reach
+  // t = T (the window advances by at least one step in each): T / n_body + 2
+  // passes cover them
+  const cudaGraphNode_t plan_node = two ? s->plan_node : nullptr;
+  if (two && !plan_node) e = pa::launch_loop_cond(s->loop_cond, s->d.ctl, (int32_t)(s->d.T / n_body + 2), s->st);
   cudaGraph_t body = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(s->st, &body);
   if (e == cudaSuccess) e = e2;
@@ -641,6 +688,8 @@ pa_status pa_loop_capture_end(pa_solver* s) {
                   "(pa_step_async, the denoiser, pa_submit_eps each)");
     return PA_ERR_STATE;
   }
+  if (e == cudaSuccess && plan_node)
+    e = pa::set_plan_cond(plan_node, s->d, s->plan_par, pa::LoopCond{s->loop_cond, s->d.T + 2});
   if (e == cudaSuccess) e = cudaGraphInstantiate(&s->loop_exec, s->loop_graph, 0);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
@@ -658,8 +707,7 @@ pa_status pa_loop_launch(pa_solver* s, const float* x_init) {
     return PA_ERR_STATE;
   }
   if (s->state == St::Stepped || s->loop_capturing) return state_fail("pa_loop_launch");
-  cudaError_t e = copy_x_init(s, x_init);
-  if (e == cudaSuccess) e = pa::launch_init(s->d, s->st);  // also clears the loop's pass counter
+  cudaError_t e = begin_generation(s, x_init);  // also clears the loop's pass counter
   if (e == cudaSuccess) e = cudaGraphLaunch(s->loop_exec, s->st);
   if (e != cudaSuccess) return cuda_fail("pa_loop_launch", e);
   s->k = 0;

@@ -148,8 +148,8 @@ class Solver:
         denoiser runs one host-driven generation of its x_init and takes its
         iteration count, rounded up to even, as the body (later generations
         that need more iterations simply take more passes). Each call then
-        enqueues ``pa_loop_launch`` (x_init copied in, pa_init's kernel, one
-        launch of the graph) and ``pa_poll_begin`` (x_T and the counters
+        enqueues ``pa_loop_launch`` (pa_init's kernel, which takes x_init in,
+        one launch of the graph) and ``pa_poll_begin`` (x_T and the counters
         copied out): no host round trip inside a generation. With ``wait``
         the call returns after that poll; without it, it returns at once with
         at most two generations in flight (a third call first waits for the
