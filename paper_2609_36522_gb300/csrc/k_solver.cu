@@ -68,6 +68,21 @@ __device__ __forceinline__ void copy_row(const Dev& d, int b, int src_state, int
   copy_part<VEC>(d.D, d.X + ((int64_t)b * (d.P + 1) + src_state % (d.P + 1)) * d.D, d.batch_x + (int64_t)r * d.D, nullptr);
 }
 
+// The sums of iteration par's decision (divided by D) for the host, and the
+// accumulator set that the next iteration adds into cleared: CTA `cta` of `ctas`
+// of kGatherThreads threads.
+__device__ __forceinline__ void report_sums(const Dev& d, int par, int64_t cta = 0, int64_t ctas = 1) {
+  const int npair = d.B * d.P;
+  for (int64_t q = cta * kGatherThreads + threadIdx.x; q < npair; q += ctas * kGatherThreads) {
+    const double* e = d.acc + ((size_t)(par * 2 + 0) * npair + q) * kAccStride;
+    const double* dl = d.acc + ((size_t)(par * 2 + 1) * npair + q) * kAccStride;
+    d.red_err[q] = (float)(__ldcg(e) * d.inv_d);
+    d.red_del[q] = (float)(__ldcg(dl) * d.inv_d);
+    d.acc[((size_t)((par ^ 1) * 2 + 0) * npair + q) * kAccStride] = 0.0;
+    d.acc[((size_t)((par ^ 1) * 2 + 1) * npair + q) * kAccStride] = 0.0;
+  }
+}
+
 // The gather of a plan already in memory (copy par), after the one-CTA planner.
 // Its CTAs also report the sums that the plan was made from (set par ^ 1,
 // divided by D) and clear the set that the planned iteration adds into: the
@@ -76,18 +91,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kGatherThreads) k_gather(Dev d, int par) {
   pdl_wait();  // everything read here comes from the kernel that planned
   pdl_trigger();  // the successor may now run its prologue
-  {
-    const int npair = d.B * d.P, old = par ^ 1;
-    const int64_t step = (int64_t)gridDim.x * gridDim.y * kGatherThreads;
-    for (int64_t q = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kGatherThreads + threadIdx.x; q < npair; q += step) {
-      const double* e = d.acc + ((size_t)(old * 2 + 0) * npair + q) * kAccStride;
-      const double* dl = d.acc + ((size_t)(old * 2 + 1) * npair + q) * kAccStride;
-      d.red_err[q] = (float)(__ldcg(e) * d.inv_d);
-      d.red_del[q] = (float)(__ldcg(dl) * d.inv_d);
-      d.acc[((size_t)(par * 2 + 0) * npair + q) * kAccStride] = 0.0;
-      d.acc[((size_t)(par * 2 + 1) * npair + q) * kAccStride] = 0.0;
-    }
-  }
+  report_sums(d, par ^ 1, (int64_t)blockIdx.y * gridDim.x + blockIdx.x, (int64_t)gridDim.x * gridDim.y);
   const int n = d.ctl->n_miss;
   const Traj* tr = d.traj + par * d.B;
   for (int r = blockIdx.y; r < n; r += gridDim.y) {
@@ -352,12 +356,14 @@ __global__ void __launch_bounds__(kPlainThreads) k_update_plain(Dev d, const flo
 // takes the whole decision in shared memory -- the same inputs and the same
 // arithmetic give the same plan in every CTA -- then copies the column range
 // blockIdx.x of batch rows blockIdx.y, blockIdx.y + gridDim.y, ... that hold
-// a miss (one row per CTA unless the rows outnumber one wave of CTAs). CTA (0, 0)
-// also publishes the plan (copy par ^ 1 of the trajectories and counters,
-// ranks, miss list, iteration log, the reductions for the host) and clears
-// the accumulator set of iteration k+1. Nobody waits for anybody: the other
+// a miss (one row per CTA unless the rows outnumber one wave of CTAs). A CTA of
+// the last row also publishes the plan (copy par ^ 1 of the trajectories and
+// counters, ranks, miss list, iteration log), one of the row before reports the
+// reductions for the host and clears the accumulator set of iteration k+1: they
+// seldom have a row to copy. Nobody waits for anybody: the other
 // CTAs read copy par of the plan, which no CTA writes in this launch.
 constexpr int kPlanThreads = 256;
+static_assert(kPlanThreads == kGatherThreads, "report_sums");
 constexpr int kPlanPerSm = 2;   // planning CTAs per SM (three: the launch bound makes the decision spill, slower)
 constexpr int kFusedMaxPairs = 1024;  // B*P planned in every CTA at most; beyond, one CTA plans
 // Beyond this many pairs one CTA plans and a separate gather follows unless
@@ -366,7 +372,7 @@ constexpr int kFusedMaxPairs = 1024;  // B*P planned in every CTA at most; beyon
 // step against 51.7 and 62.8 us, at 300 and 400 pairs 28.6 and 34.9 against
 // 27.9 and 34.4 us
 constexpr int kFusedPreferPairs = 512;
-static_assert(kFusedMaxPairs <= 32 * 32, "decide_par keeps one miss mask per 32-position chunk, 32 of them");
+static_assert(kFusedMaxPairs <= 32 * 32, "one miss mask per 32-position chunk, a lane each");
 
 // The decision's inputs as bits in shared memory (one-CTA planner).
 struct RedBits {
@@ -376,25 +382,154 @@ struct RedBits {
   __device__ bool near(int q) const { return (near_w[q >> 5] >> (q & 31)) & 1u; }
 };
 
-// The miss of batch row r < ds.total from the decision's chunk bits: chunk c
-// holds ranks cbase[c] .. cbase[c] + popc(cmiss[c]) - 1, in bit order. Every
-// lane of a warp calls it and gets the same answer; false if no chunk holds
-// row r (never expected).
-__device__ __forceinline__ bool row_miss(const DecideShared& ds, int B, int P, int r, int* b, int* i) {
+// Division of positions q < 2^16 by P: ceil(2^32 / P) is formed before the
+// dependency wait, each quotient is then one multiplication.
+struct Div {
+  uint32_t m;
+  __device__ explicit Div(int P) : m(P == 1 ? 0u : 0xffffffffu / (uint32_t)P + 1u) {}
+  __device__ int operator()(int q) const { return m ? (int)__umulhi((uint32_t)q, m) : q; }
+};
+
+// The decision over the grid: every CTA takes it whole, with all of its warps,
+// from the bits that stage_decision_bits left (the rules are decide_par's, which
+// takes it with one warp):
+//  1. every warp advances all trajectories, lane b the b-th and (b + 32)-th:
+//     a barrier less than one warp doing it for the others;
+//  2. warp w forms the miss bits of the next windows' 32-position chunks w,
+//     w + 8, ..., a trajectory's window by one shuffle of a packed word;
+//  3. after one barrier every warp scans the chunks' miss counts (lane c: chunk
+//     c), so ranks and rows need no further one.
+// One warp walking the chunks took about 250 cycles for each.
+struct GridPlan {
+  unsigned mm;   // lane c: miss bits of chunk c
+  int base;      // lane c: misses before chunk c
+  int total;
+};
+
+__device__ __forceinline__ GridPlan decide_grid(const Dev& d, DecideShared& sh, Div div) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int B = d.B, P = d.P, T = d.T, N = B * P, nchunk = (N + 31) / 32;
+  uint32_t packed[2] = {0u, 0u};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int b = lane + 32 * k;
+    if (b < B) {
+      const int t = sh.t[b], p = sh.p[b];
+      int stride = 0;
+      if (p > 0) {
+        int lead = 0;
+        while (lead < p) {
+          const unsigned w = bits32(sh.conv, b * P + lead);
+          const int ones = w == 0xffffffffu ? 32 : __ffs(~w) - 1;
+          lead += ones;
+          if (ones < 32) break;
+        }
+        stride = min(p, 1 + min(lead, p));
+      }
+      const int tn = t + stride, pn = p > 0 ? min(P, T - tn) : 0, nh = p > 0 ? p - stride : 0;
+      // window size (11 bits), positions with an entry (10), stride - 1 (10); B * P <= 1024
+      packed[k] = (uint32_t)pn | (uint32_t)nh << 11 | (uint32_t)max(stride - 1, 0) << 21;
+      if (warp == 0) {
+        sh.tn[b] = tn;
+        sh.pn[b] = pn;
+        sh.en[b] = p > 0 ? t + p : sh.e[b];
+        sh.stride[b] = stride;
+        sh.nh[b] = nh;
+        if (d.adapt) adapt_tau(d, sh, b, p, stride);
+      }
+    }
+  }
+  if (d.adapt) __syncthreads();  // the next hit test's bounds
+  for (int c = warp; c < nchunk; c += kPlanThreads / 32) {
+    const int q = c * 32 + lane;
+    const int b = min(div(q), B - 1), jn = q - b * P;
+    const uint32_t lo = __shfl_sync(0xffffffffu, packed[0], b & 31), hi = __shfl_sync(0xffffffffu, packed[1], b & 31);
+    const uint32_t w = b < 32 ? lo : hi;
+    const int pn = w & 0x7ff, nh = (w >> 11) & 0x3ff, back = w >> 21;  // stride - 1
+    const bool win = q < N && jn < pn;
+    bool hit = false;
+    if (win && jn < nh) {
+      const int qo = q + back;
+      hit = d.adapt ? sum_lt(sh.del[qo], sh.thr[b]) : ((sh.near[qo >> 5] >> (qo & 31)) & 1u);
+    }
+    const unsigned wm = __ballot_sync(0xffffffffu, win), mm = __ballot_sync(0xffffffffu, win && !hit);
+    if (lane == 0) {
+      sh.cwin[c] = wm;
+      sh.cmiss[c] = mm;
+    }
+  }
+  __syncthreads();
+  GridPlan g;
+  g.mm = lane < nchunk ? sh.cmiss[lane] : 0u;
+  const int cnt = __popc(g.mm);
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  g.base = incl - cnt;
+  g.total = __shfl_sync(0xffffffffu, incl, 31);
+  return g;
+}
+
+// The plan to memory, by one CTA: ranks and miss list (trajectory-major,
+// ascending t), trajectories, counters and iteration log of the next iteration.
+__device__ __forceinline__ void publish_plan(const Dev& d, DecideShared& sh, const GridPlan& g, int par, Div div) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int B = d.B, P = d.P, N = B * P, nchunk = (N + 31) / 32;
+  for (int c = warp; c < nchunk; c += kPlanThreads / 32) {
+    const int q = c * 32 + lane;
+    const unsigned mm = __shfl_sync(0xffffffffu, g.mm, c);
+    const int r = __shfl_sync(0xffffffffu, g.base, c) + __popc(mm & ((1u << lane) - 1u));
+    if (q >= N) continue;
+    if ((mm >> lane) & 1u) {
+      const int b = div(q);
+      d.rank[q] = r;
+      d.miss_bt[2 * r] = b;
+      d.miss_bt[2 * r + 1] = sh.tn[b] + (q - b * P);
+    } else {
+      d.rank[q] = -1;
+    }
+  }
+  const int win = __reduce_add_sync(0xffffffffu, lane < nchunk ? __popc(sh.cwin[lane]) : 0);
+  if (tid == 0) {
+    int act = 0;
+    for (int b = 0; b < B; ++b) act += (sh.pn[b] > 0);
+    PlanCtr c;
+    c.n_active = act;
+    c.iter = sh.iter + 1;
+    c.nfe = sh.nfe + g.total;
+    c.hits = sh.hits + (win - g.total);
+    d.pc[par ^ 1] = c;
+    d.ctl->n_miss = g.total;
+    d.ctl->n_active = act;
+    d.ctl->iter = c.iter;
+    d.ctl->nfe = c.nfe;
+    d.ctl->hits = c.hits;
+  }
+  for (int b = tid; b < B; b += kPlanThreads) {
+    publish_traj(d, sh, b, par);
+    log_traj(d, sh, b);
+  }
+}
+
+// The miss of batch row r < g.total: chunk c holds ranks base .. base +
+// popc(mm) - 1, in bit order. Every lane of a warp calls it and gets the same
+// answer; false if no chunk holds row r (never expected).
+__device__ __forceinline__ bool row_miss(const DecideShared& ds, const GridPlan& g, int N, int P, Div div, int r,
+                                         int* b, int* i) {
   const int lane = threadIdx.x & 31;
-  const int nchunk = (B * P + 31) / 32;  // <= 32 (kFusedMaxPairs)
-  const unsigned mm = lane < nchunk ? ds.cmiss[lane] : 0u;
-  const int base = lane < nchunk ? ds.cbase[lane] : 0;
-  const unsigned held = __ballot_sync(0xffffffffu, lane < nchunk && r >= base && r < base + __popc(mm));
+  const unsigned held = __ballot_sync(0xffffffffu, r >= g.base && r < g.base + __popc(g.mm));
   if (held == 0u) return false;
   const int c = __ffs(held) - 1;
-  const unsigned m = __shfl_sync(0xffffffffu, mm, c);
-  const int n = r - __shfl_sync(0xffffffffu, base, c);  // row r is the n-th miss of chunk c
+  const unsigned m = __shfl_sync(0xffffffffu, g.mm, c);
+  const int n = r - __shfl_sync(0xffffffffu, g.base, c);  // row r is the n-th miss of chunk c
   const unsigned at = __ballot_sync(0xffffffffu, ((m >> lane) & 1u) && __popc(m & ((1u << lane) - 1u)) == n);
   if (at == 0u) return false;
   const int q = c * 32 + __ffs(at) - 1;
-  if (q >= B * P) return false;
-  *b = q / P;
+  if (q >= N) return false;
+  *b = div(q);
   *i = ds.tn[*b] + (q - *b * P);
   return true;
 }
@@ -410,39 +545,42 @@ __device__ __forceinline__ bool row_miss(const DecideShared& ds, int B, int P, i
 template <int VEC, bool COND>
 __global__ void __launch_bounds__(kPlanThreads, kPlanPerSm) k_plan_gather(Dev d, int par, LoopCond lc) {
   __shared__ DecideShared ds;
-  const bool publish = blockIdx.x == 0 && blockIdx.y == 0;
+  // the last batch rows hold a miss only when everything misses: their CTAs
+  // publish the plan and report the sums
+  const bool publish = blockIdx.x == 0 && blockIdx.y == gridDim.y - 1;
+  const bool report = blockIdx.x == gridDim.x - 1 && (int)blockIdx.y == max((int)gridDim.y - 2, 0);
   decide_load<kPlanThreads>(d, ds, par);
+  const Div div(d.P);
   pdl_wait();  // the sums and the new states come from the update kernel
   pdl_trigger();  // the successor may now run its prologue
-  stage_decision_bits(d, ds, par, publish ? 0 : -1, 1);
+  stage_decision_bits(d, ds, par, -1, 1);
   __syncthreads();  // the decision's input bits and decide_load's state are staged
-  const bool one_row = (int)gridDim.y >= d.B * d.P;  // every batch row has its own CTA
-  decide_par(d, ds, par, publish ? 0 : -1, 1, one_row ? (int)blockIdx.y : -1);
-  __syncthreads();  // the plan (the batch rows of this CTA) is known
+  const bool active = ds.active != 0;
+  GridPlan g{0u, 0, 0};
+  if (active) {
+    g = decide_grid(d, ds, div);
+    if (publish) publish_plan(d, ds, g, par, div);
+  } else if (publish && threadIdx.x < 32) {
+    carry_plan(d, par);
+  }
   if constexpr (COND) {
     if (publish && threadIdx.x == 0) {
       int act = 0;
-      if (ds.active != 0)
+      if (active)
         for (int b = 0; b < d.B; ++b) act += ds.pn[b] > 0;
       const bool more = act > 0 && __ldcg(&d.ctl->status) == kDevOk && ds.iter + 1 < lc.limit;
       cudaGraphSetConditional(lc.handle, more ? 1u : 0u);
     }
   }
-  if (one_row) {
-    if ((int)blockIdx.y < ds.total && ds.target_b >= 0) {
-      const int b = ds.target_b;
-      copy_row<VEC>(d, b, min(ds.target_i, ds.en[b]), blockIdx.y);
-    }
-    return;
-  }
-  for (int r = blockIdx.y; r < ds.total; r += gridDim.y) {
+  for (int r = blockIdx.y; r < g.total; r += gridDim.y) {
     int b = 0, i = 0;
-    if (!row_miss(ds, d.B, d.P, r, &b, &i)) {
+    if (!row_miss(ds, g, d.B * d.P, d.P, div, r, &b, &i)) {
       if (threadIdx.x == 0) set_status(d.ctl, kDevBadRank);
       continue;
     }
     copy_row<VEC>(d, b, min(i, ds.en[b]), r);
   }
+  if (report) report_sums(d, par);
 }
 
 // One-CTA planner for B*P beyond kFusedPreferPairs (without adaptation) or

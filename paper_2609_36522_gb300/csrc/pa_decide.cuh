@@ -254,6 +254,65 @@ __device__ __forceinline__ unsigned bits32(const unsigned* w, int pos) {
   return v;
 }
 
+// Adaptation: tau_cache of trajectory b's next hit test, from the planned
+// iteration's hit rate among positions with an entry and its stride: below the
+// target rate tau rises by (1 + rate) if the window advanced beyond its first
+// position, else holds; at or above it falls by (1 + rate); kept within
+// [tau_min, tau_max]; no entries: tau holds.
+__device__ __forceinline__ void adapt_tau(const Dev& d, DecideShared& sh, int b, int p, int stride) {
+  double tau = sh.tau[b];
+  const int ne = sh.one[b], nh = sh.onh[b];
+  if (p > 0 && ne > 0) {
+    if ((double)nh / (double)ne < d.adapt_target) {
+      if (stride > 1) tau = fmin(tau * d.adapt_up, d.tau_max);
+    } else {
+      tau = fmax(tau / d.adapt_up, d.tau_min);
+    }
+  }
+  sh.tau[b] = tau;
+  sh.thr[b] = tau * (double)d.D;
+}
+
+// Trajectory b's entry of the iteration log.
+__device__ __forceinline__ void log_traj(const Dev& d, const DecideShared& sh, int b) {
+  int32_t* lg = d.iter_log + ((int64_t)sh.iter * d.B + b) * kLogFields;
+  if (sh.p[b] > 0) {
+    lg[0] = sh.t[b]; lg[1] = sh.p[b]; lg[2] = sh.om[b]; lg[3] = sh.stride[b];
+    lg[4] = sh.e[b]; lg[5] = sh.oh1[b]; lg[6] = sh.one[b]; lg[7] = sh.onh[b];
+  } else {
+    for (int f = 0; f < kLogFields; ++f) lg[f] = 0;
+    lg[0] = sh.t[b];
+  }
+}
+
+// Trajectory b of the next iteration (copy par ^ 1); its misses and its hits at
+// positions >= 1 come from the chunk bits.
+__device__ __forceinline__ void publish_traj(const Dev& d, const DecideShared& sh, int b, int par) {
+  const int P = d.P;
+  Traj tr{};
+  tr.t = sh.tn[b];
+  tr.p = sh.pn[b];
+  tr.e = sh.en[b];
+  tr.done = (sh.pn[b] == 0);
+  tr.m = range_popc(sh.cmiss, b * P, b * P + sh.pn[b]);
+  tr.h1 = sh.pn[b] > 1 ? (sh.pn[b] - 1) - range_popc(sh.cmiss, b * P + 1, b * P + sh.pn[b]) : 0;
+  tr.ne = sh.nh[b];
+  tr.nh = sh.nh[b] - range_popc(sh.cmiss, b * P, b * P + sh.nh[b]);
+  if (d.adapt) d.tau[(par ^ 1) * d.B + b] = sh.tau[b];
+  if (tr.t > d.T || tr.e < tr.t) atomicCAS(&d.ctl->status, kDevOk, kDevBadState);
+  d.traj[(par ^ 1) * d.B + b] = tr;
+}
+
+// Finished: iterating further changes nothing, the plan carries over (one warp).
+__device__ __forceinline__ void carry_plan(const Dev& d, int par) {
+  const int lane = threadIdx.x & 31;
+  for (int b = lane; b < d.B; b += 32) {
+    d.traj[(par ^ 1) * d.B + b] = d.traj[par * d.B + b];
+    if (d.adapt) d.tau[(par ^ 1) * d.B + b] = d.tau[par * d.B + b];
+  }
+  if (lane == 0) d.pc[par ^ 1] = d.pc[par];
+}
+
 // The decision that ends an iteration, for kernels in which every CTA decides
 // (B*P <= 32 * 32), from the bit strings that stage_decision_bits left in
 // sh.conv (bit b*P + j: the Eq. 2 error of window position j of trajectory b
@@ -277,22 +336,15 @@ __device__ __forceinline__ unsigned bits32(const unsigned* w, int pos) {
 // batch row `target` (target_b, target_i); the CTA with pub_id 0 also writes
 // the trajectories, counters and iteration log. Gives the same plan, ranks and
 // counters as decide_run. Every thread of the CTA calls it; the caller
-// synchronises the CTA afterwards.
+// synchronises the CTA afterwards. (The fused step's form; the planning
+// kernel's, which spreads it over the CTA's warps, is decide_grid.)
 __device__ inline void decide_par(const Dev& d, DecideShared& sh, int par, int pub_id, int pub_count, int target) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int B = d.B, P = d.P, T = d.T;
   const int N = B * P, nchunk = (N + 31) / 32;
-  Traj* out_traj = d.traj + (par ^ 1) * B;
   if (sh.active == 0) {  // finished: the plan carries over (uniform across the CTA)
     if (warp == 0) {
-      if (pub_id == 0) {
-        const Traj* in_traj = d.traj + par * B;
-        for (int b = lane; b < B; b += 32) {
-          out_traj[b] = in_traj[b];
-          if (d.adapt) d.tau[(par ^ 1) * B + b] = d.tau[par * B + b];
-        }
-        if (lane == 0) d.pc[par ^ 1] = d.pc[par];
-      }
+      if (pub_id == 0) carry_plan(d, par);
       for (int b = lane; b < B; b += 32) sh.en[b] = sh.e[b];
     }
     return;
@@ -318,34 +370,8 @@ __device__ inline void decide_par(const Dev& d, DecideShared& sh, int par, int p
       sh.en[b] = p > 0 ? t + p : sh.e[b];
       sh.stride[b] = stride;
       sh.nh[b] = p > 0 ? p - stride : 0;  // next-window positions with a cache entry
-      if (d.adapt) {
-        // tau_cache of the next hit test, from the planned iteration's hit
-        // rate among positions with an entry and its stride: below the
-        // target rate tau rises by (1 + rate) if the window advanced beyond
-        // its first position, else holds; at or above it falls by (1 + rate);
-        // kept within [tau_min, tau_max]; no entries: tau holds
-        double tau = sh.tau[b];
-        const int ne = sh.one[b], nh = sh.onh[b];
-        if (p > 0 && ne > 0) {
-          if ((double)nh / (double)ne < d.adapt_target) {
-            if (stride > 1) tau = fmin(tau * d.adapt_up, d.tau_max);
-          } else {
-            tau = fmax(tau / d.adapt_up, d.tau_min);
-          }
-        }
-        sh.tau[b] = tau;
-        sh.thr[b] = tau * (double)d.D;
-      }
-      if (pub_id == 0) {
-        int32_t* lg = d.iter_log + ((int64_t)iter * B + b) * kLogFields;
-        if (p > 0) {
-          lg[0] = t; lg[1] = p; lg[2] = sh.om[b]; lg[3] = stride;
-          lg[4] = sh.e[b]; lg[5] = sh.oh1[b]; lg[6] = sh.one[b]; lg[7] = sh.onh[b];
-        } else {
-          for (int f = 0; f < kLogFields; ++f) lg[f] = 0;
-          lg[0] = t;
-        }
-      }
+      if (d.adapt) adapt_tau(d, sh, b, p, stride);
+      if (pub_id == 0) log_traj(d, sh, b);
     }
     __syncwarp();
     // the next windows' bits, one 32-position chunk per ballot: position j'
@@ -415,20 +441,7 @@ __device__ inline void decide_par(const Dev& d, DecideShared& sh, int par, int p
   if (pub_id == 0) {
     // trajectories and counters of the next iteration; a trajectory's misses
     // and its hits at positions >= 1 come from the chunk bits
-    for (int b = tid; b < B; b += blockDim.x) {
-      Traj tr{};
-      tr.t = sh.tn[b];
-      tr.p = sh.pn[b];
-      tr.e = sh.en[b];
-      tr.done = (sh.pn[b] == 0);
-      tr.m = range_popc(sh.cmiss, b * P, b * P + sh.pn[b]);
-      tr.h1 = sh.pn[b] > 1 ? (sh.pn[b] - 1) - range_popc(sh.cmiss, b * P + 1, b * P + sh.pn[b]) : 0;
-      tr.ne = sh.nh[b];
-      tr.nh = sh.nh[b] - range_popc(sh.cmiss, b * P, b * P + sh.nh[b]);
-      if (d.adapt) d.tau[(par ^ 1) * B + b] = sh.tau[b];
-      if (tr.t > T || tr.e < tr.t) atomicCAS(&d.ctl->status, kDevOk, kDevBadState);
-      out_traj[b] = tr;
-    }
+    for (int b = tid; b < B; b += blockDim.x) publish_traj(d, sh, b, par);
     if (tid == 0) {
       int act = 0;
       for (int b = 0; b < B; ++b) act += (sh.pn[b] > 0);
