@@ -153,8 +153,10 @@ PA_API pa_status pa_step_async(pa_solver* s, const float** batch_x_dev,
 PA_API const int32_t* pa_n_miss_dev(const pa_solver* s);
 
 /* Hand back eps_theta for the planned misses: batch_eps_dev [M][D] fp32,
- * DEVICE pointer, 16-byte aligned for the fused, lean and bulk update forms
- * (otherwise the plain-load kernel runs). Runs Eq. 6 (assembly), Eq. 7 (cache update),
+ * DEVICE pointer, 16-byte aligned for the fused and bulk update forms and the
+ * lean form's 16-byte accesses (otherwise the lean form's 4-byte accesses or,
+ * where it does not hold the window or with stochastic steps, the plain-load
+ * kernel). Runs Eq. 6 (assembly), Eq. 7 (cache update),
  * the drift and the Picard prefix sum (Eq. 1), the errors of Eq. 2 and the
  * cache distances of the next iteration (Eq. 4), then the window advance
  * (Sec. 2.1), the hit-miss plan of the next iteration (Eq. 5) and the gather
@@ -288,11 +290,12 @@ PA_API pa_status pa_last_reductions(pa_solver* s, float* err_out, float* delta_o
  *   0       plain loads (one thread per column; any D);
  *   1       the bulk forms: register-resident rows, or rows staged in shared
  *           memory by bulk copies for windows the registers cannot hold;
- *   2       the lean register form followed by the planning kernel (default
- *           when D % 4 == 0): 16-byte rows
- *           straight into registers, plain fp32 prefix sums, coefficients and
- *           ranks staged in shared memory; windows up to 112 points with
- *           deterministic steps, else it falls back to 1;
+ *   2       the lean register form followed by the planning kernel (default):
+ *           16-byte rows straight into registers, plain fp32 prefix sums,
+ *           coefficients and ranks staged in shared memory; windows up to 112
+ *           points with deterministic steps, else it falls back to 1. Where
+ *           D % 4 != 0 or batch_eps is not 16-byte aligned: 4-byte accesses
+ *           and compensated sums (not with a launch shape 200 + n);
  *   100 + n bulk forms with launch shape n (0..12; columns per lane, warps per
  *           CTA, pipeline depth; 112 = the register-resident form);
  *   200 + n lean form with launch shape n: 0 by window, 1 = 16 warps x 7
@@ -301,8 +304,8 @@ PA_API pa_status pa_last_reductions(pa_solver* s, float* err_out, float* delta_o
  *           210 + n (n <= 4) the same with compensated (TwoSum) sums,
  *           deterministic steps only. Shapes 5 and 6 take deterministic steps
  *           only. A shape that cannot hold the window falls back to 1.
- * Forms 1 and 2 fall back to plain loads for a batch_eps pointer that is not
- * 16-byte aligned. A tuning aid; returns PA_ERR_ARG for an unknown value. */
+ * Form 1 falls back to plain loads where D % 4 != 0 or for a batch_eps pointer
+ * that is not 16-byte aligned. A tuning aid; returns PA_ERR_ARG for an unknown value. */
 PA_API pa_status pa_set_update_kernel(pa_solver* s, int kind);
 
 /* ---- triangular Anderson mixing (ParaTAA-style update) ------------------

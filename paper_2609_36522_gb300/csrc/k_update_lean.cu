@@ -61,6 +61,33 @@ __device__ __forceinline__ Q ldq(const float* p) {
 __device__ __forceinline__ void stq(float* p, const Q& q) {
   *reinterpret_cast<float4*>(p) = make_float4(q.l.x, q.l.y, q.h.x, q.h.y);
 }
+// The lane's four columns of a row: adjacent ones (VEC), or every 32nd of the
+// strip, so that a warp's 4-byte accesses are still adjacent; of those the
+// first nl lie inside the row, the others read as 0 and are not written.
+template <bool VEC>
+__device__ __forceinline__ Q ld_cols(const float* p, int nl) {
+  if constexpr (VEC) {
+    return ldq(p);
+  } else {
+    Q q = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    if (nl > 0) q.l.x = p[0];
+    if (nl > 1) q.l.y = p[32];
+    if (nl > 2) q.h.x = p[64];
+    if (nl > 3) q.h.y = p[96];
+    return q;
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void st_cols(float* p, const Q& q, int nl) {
+  if constexpr (VEC) {
+    stq(p, q);
+  } else {
+    if (nl > 0) p[0] = q.l.x;
+    if (nl > 1) p[32] = q.l.y;
+    if (nl > 2) p[64] = q.h.x;
+    if (nl > 3) p[96] = q.h.y;
+  }
+}
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return __ffma2_rn(b, make_float2(-1.f, -1.f), a);  // -b exact, one rounding: a - b
 }
@@ -71,23 +98,37 @@ __device__ __forceinline__ Q qsub(const Q& a, const Q& b) { return {sub2(a.l, b.
 // bfloat16 when CB (rounded to nearest even when written, widened exactly when
 // read). The trajectory's rows start where its fp32 rows would; within them
 // the row pitch is D entries.
-template <bool CB>
-__device__ __forceinline__ Q ld_ent(const float* traj_base, int off) {
-  if constexpr (CB) {
+template <bool CB, bool VEC>
+__device__ __forceinline__ Q ld_ent(const float* traj_base, int off, int nl) {
+  if constexpr (CB && VEC) {
     float a[4];
     Bf16Row<4>::load(reinterpret_cast<const uint16_t*>(traj_base) + off, a);
     return {make_float2(a[0], a[1]), make_float2(a[2], a[3])};
+  } else if constexpr (CB) {
+    const uint16_t* p = reinterpret_cast<const uint16_t*>(traj_base) + off;
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (k < nl) Bf16Row<1>::load(p + 32 * k, a + k);
+    return {make_float2(a[0], a[1]), make_float2(a[2], a[3])};
   } else {
-    return ldq(traj_base + off);
+    return ld_cols<VEC>(traj_base + off, nl);
   }
 }
-template <bool CB>
-__device__ __forceinline__ void st_ent(float* traj_base, int off, const Q& q) {
+template <bool CB, bool VEC>
+__device__ __forceinline__ void st_ent(float* traj_base, int off, const Q& q, int nl) {
   if constexpr (CB) {
     const float a[4] = {q.l.x, q.l.y, q.h.x, q.h.y};
-    Bf16Row<4>::store(reinterpret_cast<uint16_t*>(traj_base) + off, a);
+    uint16_t* p = reinterpret_cast<uint16_t*>(traj_base) + off;
+    if constexpr (VEC) {
+      Bf16Row<4>::store(p, a);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k < nl) Bf16Row<1>::store(p + 32 * k, a + k);
+    }
   } else {
-    stq(traj_base + off, q);
+    st_cols<VEC>(traj_base + off, q, nl);
   }
 }
 // The value an fp32 row piece takes once stored as an entry.
@@ -196,9 +237,11 @@ __device__ __forceinline__ void step_tail(const Dev& d, DecideShared& ds, int pa
   }
 }
 
-template <int NW, int LMAX, int MINB, bool NOISE, bool COMP, bool CB = false, bool FUSE = false, bool TAA = false>
+template <int NW, int LMAX, int MINB, bool NOISE, bool COMP, bool CB = false, bool FUSE = false, bool TAA = false,
+          bool VEC = true>
 __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const float* __restrict__ beps, int par) {
   static_assert(!(FUSE && TAA), "the fused step and the Anderson mixing are separate forms");
+  static_assert(VEC || (!FUSE && !TAA && !NOISE), "4-byte accesses: the plain form's deterministic steps");
   using Sh = LeanShape<NW, NOISE>;
   using CT = typename Coef<NOISE>::T;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -248,8 +291,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
   __syncthreads();
 
   const int t = tr.t, p = tr.p, e = tr.e;
-  const int mycol = blockIdx.x * 128 + lane * 4;
+  const int mycol = blockIdx.x * 128 + (VEC ? lane * 4 : lane);
   const bool live = mycol < D;
+  const int nl = VEC ? 4 : max(0, min(4, (D - mycol + 31) / 32));
   const float* Xr = d.X + (int64_t)b * (P + 1) * D + mycol;  // this lane's column of each ring
   float* Xw = d.X + (int64_t)b * (P + 1) * D + mycol;
   float* Xh = d.Xhat + (int64_t)b * P * D;  // entries: column mycol of row slot s at s * D + mycol
@@ -296,12 +340,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
 #pragma unroll
     for (int g = 0; g <= LMAX; ++g) {
       if (g > nj) break;
-      x[g] = ldq(Xr + xslot(g) * D);
+      x[g] = ld_cols<VEC>(Xr + xslot(g) * D, nl);
     }
 #pragma unroll
     for (int g = 0; g < LMAX; ++g) {
       if (g >= nj) break;
-      if (!(miss >> g & 1)) ep[g] = ld_ent<CB>(Eh, cslot(g) * D + mycol);
+      if (!(miss >> g & 1)) ep[g] = ld_ent<CB, VEC>(Eh, cslot(g) * D + mycol, nl);
       if constexpr (TAA) {
         // the previous iteration's residual of state t + j0 + g + 1, which it
         // has iff that state was computed then (state <= e)
@@ -311,7 +355,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
           xh[g] = ldq(Rp + sr * D);
         }
       } else {
-        if (!(miss >> (g + 1) & 1)) xh[g] = ld_ent<CB>(Xh, cslot(g + 1) * D + mycol);
+        if (!(miss >> (g + 1) & 1)) xh[g] = ld_ent<CB, VEC>(Xh, cslot(g + 1) * D + mycol, nl);
       }
       if constexpr (NOISE) z[g] = ldq(Zr + (t + j0 + g) * D);
     }
@@ -322,7 +366,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
 #pragma unroll
     for (int g = 0; g < LMAX; ++g) {
       if (g >= nj) break;
-      if (miss >> g & 1) ep[g] = ldq(Br + s_rank[j0 + g] * D);
+      if (miss >> g & 1) ep[g] = ld_cols<VEC>(Br + s_rank[j0 + g] * D, nl);
     }
   }
 
@@ -345,8 +389,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
       if (g >= nj) break;
       if (miss >> g & 1) {
         const int o = cslot(g) * D + mycol;
-        st_ent<CB>(Eh, o, ep[g]);
-        st_ent<CB>(Xh, o, x[g]);
+        st_ent<CB, VEC>(Eh, o, ep[g], nl);
+        st_ent<CB, VEC>(Xh, o, x[g], nl);
       }
       const CT c = s_coef[t + j0 + g];
       const float2 cm = make_float2(c.x, c.x), ec = make_float2(c.y, c.y);
@@ -430,7 +474,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
             dv = dd.x + dd.y;
           }
         } else {
-          stq(Xw + so * D, n);
+          st_cols<VEC>(Xw + so * D, n, nl);
           Q df = qsub(n, x[g + 1]);  // against the old state i+1 (lazy-resolved)
           if constexpr (FUSE) ep[g] = n;  // the drift is spent: keep the new state for the next batch
           const float2 e2 = __ffma2_rn(df.h, df.h, __fmul2_rn(df.l, df.l));
@@ -474,12 +518,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_update_lean(Dev d, const floa
   if constexpr (FUSE) step_tail<NW, LMAX>(d, ds, par, tr, ep, j0, nj, mycol, D, live);
 }
 
-template <int NW, int LMAX, int MINB, bool NOISE, bool COMP, bool CB = false, bool FUSE = false, bool TAA = false>
+template <int NW, int LMAX, int MINB, bool NOISE, bool COMP, bool CB = false, bool FUSE = false, bool TAA = false,
+          bool VEC = true>
 cudaError_t launch_lean(const Dev& d, const float* beps, int par, cudaStream_t st) {
   using Sh = LeanShape<NW, NOISE>;
   const int nstrip = (int)((d.D + 127) / 128);
   const size_t smem = Sh::smem_bytes(d.T, d.P, COMP);
-  auto kern = k_update_lean<NW, LMAX, MINB, NOISE, COMP, CB, FUSE, TAA>;
+  auto kern = k_update_lean<NW, LMAX, MINB, NOISE, COMP, CB, FUSE, TAA, VEC>;
   static size_t configured[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -493,6 +538,11 @@ cudaError_t launch_lean(const Dev& d, const float* beps, int par, cudaStream_t s
 }
 
 constexpr size_t kLeanSmemMax = 200 * 1024;
+
+// Rows, eps and draws that start on 16-byte boundaries.
+bool lean_vec(const Dev& d, const float* batch_eps) {
+  return d.D % 4 == 0 && ((reinterpret_cast<uintptr_t>(batch_eps) | reinterpret_cast<uintptr_t>(d.noise)) & 15) == 0;
+}
 
 // The fused step: launched cooperatively, so only when every CTA of the grid
 // (a strip of 128 columns of each trajectory) can be resident at once;
@@ -541,6 +591,21 @@ cudaError_t launch_fused(const Dev& d, const float* beps, int par, cudaStream_t 
 cudaError_t launch_update_lean(const Dev& d, const float* batch_eps, int par, int shape, cudaStream_t st) {
   const bool comp = shape >= 10;
   int s = shape % 10;
+  if (!lean_vec(d, batch_eps)) {
+    // 4-byte accesses (rows of any length, eps of any alignment), by window
+    // only, with the compensated sums of the plain-load kernel, which walks the
+    // window one position after the other (a generation of T 50 at 3x37x53,
+    // window 24, two trajectories: 235 us with that one, 157 with this)
+    if (shape != 0 || d.noise) return cudaErrorNotSupported;
+    if (d.cache_bf16) {
+      if (d.P <= 32) return launch_lean<8, 4, 2, false, true, true, false, false, false>(d, batch_eps, par, st);
+      if (d.P <= 64) return launch_lean<16, 4, 1, false, true, true, false, false, false>(d, batch_eps, par, st);
+      return launch_lean<16, 7, 1, false, true, true, false, false, false>(d, batch_eps, par, st);
+    }
+    if (d.P <= 32) return launch_lean<8, 4, 2, false, true, false, false, false, false>(d, batch_eps, par, st);
+    if (d.P <= 64) return launch_lean<16, 4, 1, false, true, false, false, false, false>(d, batch_eps, par, st);
+    return launch_lean<16, 7, 1, false, true, false, false, false, false>(d, batch_eps, par, st);
+  }
   if (s == 0) {
     // by window: as many CTAs per SM as the registers allow without spilling
     // (three of 8 x 4, two of 8 x 8), else 16 warps of at most 7 positions
@@ -614,7 +679,8 @@ cudaError_t launch_step_fused(const Dev& d, const float* batch_eps, int par, int
 // 8 x 8 or 8 x 4 warps x positions; with draws 16 x 7 or 8 x 4 at two CTAs per
 // SM), fp32 cache entries.
 cudaError_t launch_update_taa(const Dev& d, const float* batch_eps, int par, cudaStream_t st) {
-  if (!update_lean_supported(d, batch_eps) || d.cache_bf16 || !d.taa_g) return cudaErrorNotSupported;
+  if (!update_lean_supported(d, batch_eps) || !lean_vec(d, batch_eps) || d.cache_bf16 || !d.taa_g)
+    return cudaErrorNotSupported;
   if (d.noise) {
     if (d.P <= 32) return launch_lean<8, 4, 2, true, false, false, false, true>(d, batch_eps, par, st);
     return launch_lean<16, 7, 1, true, false, false, false, true>(d, batch_eps, par, st);
@@ -627,13 +693,11 @@ cudaError_t launch_update_taa(const Dev& d, const float* batch_eps, int par, cud
 bool step_fused_supported(const Dev& d, const float* batch_eps, int shape) {
   // every CTA decides in shared memory from one miss mask per 32-position chunk
   if (shape >= 10 || (int64_t)d.B * d.P > 32 * 32) return false;
-  return update_lean_supported(d, batch_eps);
+  return lean_vec(d, batch_eps) && update_lean_supported(d, batch_eps);
 }
 
 bool update_lean_supported(const Dev& d, const float* batch_eps) {
-  if (d.D % 4 != 0 || (d.cache_bf16 && d.noise)) return false;
-  if ((reinterpret_cast<uintptr_t>(batch_eps) & 15) != 0) return false;
-  if (d.noise && (reinterpret_cast<uintptr_t>(d.noise) & 15) != 0) return false;
+  if (d.noise && (d.cache_bf16 || !lean_vec(d, batch_eps))) return false;
   if (d.P > 16 * 7) return false;
   if ((int64_t)(d.P + 1) * d.D > INT32_MAX || (int64_t)d.T * d.D > INT32_MAX) return false;
   if ((int64_t)d.B * d.P * d.D > INT32_MAX) return false;  // batch rank * D

@@ -336,12 +336,12 @@ pa_status pa_create(pa_solver** out, int T, int window, const int64_t* latent_sh
   d.inv_d = 1.0 / (double)D;
   d.wait_limit = pa::kWaitLimit;
   d.cache_bf16 = 0;
-  // the lean register form and the planning kernel, else the bulk forms, else
-  // plain loads; the fused step (3) is an option: at the 4x64x64 shape it
+  // the lean register form and the planning kernel, else (windows and steps it
+  // does not hold) the bulk forms, else plain loads; the fused step (3) is an option: at the 4x64x64 shape it
   // takes as long per solver step as the pair and a generation with the
   // denoiser is slower with it (its 16-warp CTAs hold every SM's register
   // file through the grid barrier, so nothing overlaps their tail)
-  s->update_kind = (D % 4 == 0) ? 2 : 0;
+  s->update_kind = 2;
 
   const std::vector<float> hc = step_coefficients(s->alphas, 0.0);  // DDIM (eta = 0)
   s->poll_ev[0] = s->poll_ev[1] = nullptr;

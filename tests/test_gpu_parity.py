@@ -453,6 +453,49 @@ def test_lean_update(kind, T, window, eta):
     assert np.abs(ref["x_final"] - got["x_final"]).max() <= 1e-5 * scale
 
 
+def _steps_with_eps_at(w, offset, update_kernel):
+    """One generation by steps, the eps rows written `offset` floats into their
+    allocation: (final latents, iteration log, update form that ran)."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser, Solver
+    a, x0, mu = W.inputs(w)
+    s = Solver(w.T, w.window, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch)
+    if update_kernel is not None:
+        s.set_update_kernel(update_kernel)
+    rows = w.batch * s.window
+    g = GmmDenoiser(torch.from_numpy(mu).cuda(), w.gmm_std, a, rows)
+    eps = torch.empty(rows, w.D, dtype=torch.float32, device="cuda")
+    moved = torch.empty(rows * w.D + offset, dtype=torch.float32, device="cuda")[offset:].view(rows, w.D)
+    s.init(torch.from_numpy(x0).cuda())
+    while (out := s.step()) is not None:
+        g.eps(out.batch_x_ptr, out.miss_bt_ptr, s.n_miss_dev(), eps)
+        moved.copy_(eps)
+        s.submit_eps(moved)
+    res = s.result().cpu().numpy(), s.iter_log(), s.stats()["update_kernel"]
+    s.close()
+    g.close()
+    return res
+
+
+@pytest.mark.parametrize("shape,T,window,offset", [
+    ((3, 5, 7), 40, 32, 0), ((3, 37, 53), 40, 33, 0),       # 105 and 5883 columns: one strip, and 123 in the last
+    ((1, 1, 1), 20, 6, 0), ((1, 3, 43), 150, 112, 0),       # one column; one past a strip
+    ((3, 9, 14), 150, 113, 0),                              # one past the largest window: the plain kernel
+    ((4, 20, 20), 40, 24, 1), ((4, 8, 8), 70, 64, 2), ((4, 8, 4), 100, 100, 3)])  # eps off its 16 bytes
+def test_lean_update_any_alignment(shape, T, window, offset):
+    """Rows or eps off the 16-byte boundaries: the lean update's 4-byte
+    accesses against the plain-load kernel. Both keep compensated sums of the
+    same fp32 steps, so a state differs by a few of its own roundings per
+    iteration: 1e-6 of the latents' scale, as between the other forms."""
+    w = W.Workload("alignment", T=T, window=window, batch=2, latent_shape=shape, K=3,
+                   tol=1e-3, cache_thresh=0.05, seed=23)
+    x_ref, log_ref, kind_ref = _steps_with_eps_at(w, offset, 0)
+    x, log, kind = _steps_with_eps_at(w, offset, None)
+    assert kind_ref == 0 and kind == (2 if min(window, T) <= 112 else 0)
+    assert np.array_equal(log, log_ref)
+    assert np.abs(x - x_ref).max() <= 1e-6 * np.abs(x_ref).max()
+
+
 @pytest.mark.parametrize("kind,eta", [(200, 0.0), (204, 0.0), (201, 1.0), (204, 1.0)])
 def test_lean_update_long_schedule(kind, eta):
     """A 1000-step schedule: every CTA stages 1000 coefficient sets (two per
@@ -615,7 +658,7 @@ def test_bf16_cache_entries(w):
     a neighbouring bfloat16 value when the GPU's fp32 value and the oracle's
     fp64 value straddle a rounding boundary), final latents within the bound of
     bf16_tolerance (about 1.6e-3 at T = 100). The lean register form runs where
-    it applies, the plain-load kernel elsewhere (odd D, window 128, stochastic
+    it applies, the plain-load kernel elsewhere (window 128, stochastic
     steps)."""
     from oracle.storage import round_bf16
     orc = oracle_run(w, cache_store=round_bf16)
