@@ -79,6 +79,7 @@ constexpr int kDotRows = 16;     // rows per dots CTA (two per warp)
 constexpr int kOutRows = 16;     // rows per output CTA
 constexpr int kOutCols = 256;    // columns per output CTA (four per thread)
 constexpr size_t kDotSmemBudget = 96 * 1024;
+constexpr int kDotCtas = 120;    // CTAs that a dots launch should have (of 152 SMs)
 constexpr float kDotScale = 4294967296.f;  // 2^32: fixed-point scale of the dot-product accumulators
 
 // tensor-core dot products: rows per CTA (the MMA's M), columns per CTA
@@ -147,11 +148,15 @@ size_t dots_smem_bytes(int K, int chunk) {
   return tiles > red ? tiles : red;
 }
 
-int dots_chunk(int K, int64_t D) {
+int dots_chunk(int K, int64_t D, int max_rows) {
   // largest of 512/256/128/64 columns whose (rows + K) row segments fit the budget
   int c = 512;
   while (c > 64 && (size_t)(kDotRows + K) * (c + 4) * sizeof(float) > kDotSmemBudget) c /= 2;
   while (c > 64 && (int64_t)c >= 2 * D) c /= 2;
+  // down to 128 while the chunks leave SMs without a CTA (48 rows of 5883
+  // columns: 36 CTAs of 512, 138 of 128)
+  const int64_t blocks = (max_rows + kDotRows - 1) / kDotRows;
+  while (c > 128 && (D + c - 1) / c * blocks < kDotCtas) c /= 2;
   return c;
 }
 
@@ -159,7 +164,7 @@ GmmLayout gmm_layout(int K, int64_t D, int max_rows, int T) {
   GmmLayout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = pa::align_up(o + bytes, pa::kAlign); return at; };
-  L.chunk = dots_chunk(K, D);
+  L.chunk = dots_chunk(K, D, max_rows);
   L.nchunk = (int)((D + L.chunk - 1) / L.chunk);
   L.coef = take((size_t)3 * T * sizeof(float));
   L.mnorm = take((size_t)K * sizeof(float));
@@ -206,7 +211,9 @@ __global__ void __launch_bounds__(256) k_gmm_norms(const float* __restrict__ mu,
 // Stage `nrows` row segments [c0, c0 + ncol) of a row-major matrix with row
 // length D into shared rows of stride `ld` floats: bulk copies counted on
 // `bar`, issued by the lanes of warp 0 (after the caller announced the bytes),
-// or plain loads by every thread when `bulk` is false.
+// or, when `bulk` is false (rows that start on no 16-byte boundary), 4-byte
+// asynchronous copies by every warp: no register waits for them, so a thread
+// has all of its copies in flight together.
 __device__ __forceinline__ void stage_rows(float* dst, int ld, const float* src, int64_t D, int64_t c0,
                                            int ncol, int nrows, bool bulk, uint64_t* bar) {
   if (bulk) {
@@ -217,16 +224,24 @@ __device__ __forceinline__ void stage_rows(float* dst, int ld, const float* src,
     }
     return;
   }
-  for (int q = threadIdx.x; q < nrows * ncol; q += blockDim.x) {
-    const int r = q / ncol, c = q % ncol;
-    dst[(size_t)r * ld + c] = src[(int64_t)r * D + c0 + c];
+  const int lane = threadIdx.x & 31;
+  for (int r = threadIdx.x >> 5; r < nrows; r += blockDim.x >> 5) {
+    const float* sr = src + (int64_t)r * D + c0;
+    const uint32_t dr = smem_u32(dst + (size_t)r * ld);
+    for (int c = lane; c < ncol; c += 32)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dr + 4 * c), "l"(sr + c) : "memory");
   }
 }
 
-// Wait for the bulk copies of a single-phase kernel. On a timeout: record it,
-// let the copies already issued land (bounded), and report false.
+// Wait for the bulk copies of a single-phase kernel (without them, for the
+// calling thread's own copies; the caller's barrier makes the others' visible).
+// On a timeout: record it, let the copies already issued land (bounded), and
+// report false.
 __device__ __forceinline__ bool wait_staged(bool bulk, uint64_t* bar, int32_t* status) {
-  if (!bulk) return true;
+  if (!bulk) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return true;
+  }
   if (mbar_wait_bounded(bar, 0, pa::kWaitLimit)) return true;
   atomicCAS(status, 0, pa::kDevTimeout);
   mbar_wait_bounded(bar, 0, pa::kDrainLimit);
@@ -1566,7 +1581,7 @@ extern "C" pa_status pa_gmm_eps_noalloc(const float* means_dev, int K, int64_t D
   if (n_rows == 0) return PA_OK;
   // scratch layout: coef[3T] | mnorm[K] | gacc[2][n_rows][K] (int64) | epoch |
   //                 n_rows | status   (256-byte aligned pieces)
-  const int chunk = dots_chunk(K, D);
+  const int chunk = dots_chunk(K, D, n_rows);
   const int nchunk = (int)((D + chunk - 1) / chunk);
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = pa::align_up(o + bytes, pa::kAlign); return at; };

@@ -343,6 +343,34 @@ def test_gmm_persistent_kernels(K, D, n, cap, shift):
     g.close()
 
 
+@pytest.mark.parametrize("K,D,n,cap,shift", [
+    (8, 5883, 48, 48, 0), (8, 129, 5, 8, 0), (3, 513, 33, 40, 0),   # rows on no 16-byte boundary: 4-byte copies
+    (16, 1001, 1, 16, 0), (40, 127, 17, 40, 0), (8, 1, 3, 4, 0),
+    (8, 4096, 30, 48, 1), (8, 2048, 640, 640, 0), (8, 2048, 100, 160, 0)])  # chunks of 512 and of 128 columns
+def test_gmm_cuda_core_form(K, D, n, cap, shift):
+    """The CUDA-core denoiser (form 0) against the fp64 oracle over its column
+    chunks and both ways of staging rows; tolerance as for the other forms."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    w = W.SD15.with_(K=K, latent_shape=(1, 1, D))
+    a, mu, idx, x, miss = _gmm_rows(w, n)
+    dev = torch.device("cuda")
+    g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
+    g.set_form(0)
+    xd = torch.zeros(cap * D + shift, dtype=torch.float32, device=dev)[shift:].view(cap, D)
+    xd[:n] = torch.from_numpy(x).to(dev)
+    md = torch.zeros(cap, 2, dtype=torch.int32, device=dev)
+    md[:n] = torch.from_numpy(miss).to(dev)
+    nd = torch.tensor([n], dtype=torch.int32, device=dev)
+    out = torch.full((cap, D), float("nan"), device=dev)
+    g.eps(xd.data_ptr(), md.data_ptr(), nd.data_ptr(), out)
+    want = gmm_eps(x.astype(np.float64), a[idx], mu.astype(np.float64), w.gmm_std)
+    rel = np.abs(out[:n].cpu().numpy() - want).max(axis=1) / np.abs(want).max(axis=1)
+    assert rel.max() <= 2e-6, rel.max()
+    assert torch.isnan(out[n:]).all()
+    g.close()
+
+
 def test_gmm_in_cuda_graph():
     """The denoiser captured in a CUDA graph and replayed gives the eager
     result (bitwise), with a device row count that changes between replays."""
