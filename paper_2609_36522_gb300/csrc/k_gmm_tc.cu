@@ -1,4 +1,4 @@
-// Mixture denoiser on the tensor cores (tcgen05, kind::tf32), three kernels:
+// Mixture denoiser on the tensor cores (tcgen05), three kernels:
 //
 //   k_gmm_dots_tc   partial dot products x . mu_k over a CTA's share of the
 //                   columns, accumulated in TMEM
@@ -7,13 +7,15 @@
 //   k_gmm_out_tc    eps = a x - a sqrt(a) R M, tiles of 128 columns x up to
 //                   128 rows
 //
-// fp32 accuracy from tf32 operands: every value is split as v = hi + lo with
-// hi = tf32(v), lo = tf32(v - hi); the products hi hi + hi lo + lo hi (and, where
-// it costs nothing, lo lo) are accumulated in fp32.
+// fp32 accuracy from shorter operands: the dot products split every value in
+// two tf32 parts, v = hi + lo with hi = tf32(v), lo = tf32(v - hi), and add up
+// the products hi hi + hi lo + lo hi (and, where it costs nothing, lo lo) in
+// fp32; the output splits it in three bfloat16 parts.
 //
 // What bounds it: at 118 rows of 4x128x128 and 64 components a call reads the
-// rows twice and the means twice and writes eps once, 126 MB. The two
-// contractions are 6 GFLOP of tf32 each, 3 to 4 us on all SMs, so both large
+// rows twice and the means twice and writes eps once, 126 MB (19 us at the copy
+// rate, less for what the 126 MB L2 still holds). The two contractions are three
+// times 1 GFLOP of tf32 each, 3 to 4 us on all SMs, so both large
 // kernels are one CTA per SM that keeps copies in flight while the tensor core
 // works: asynchronous copies into a ring of shared-memory stages, warps that
 // split what has landed, one thread that issues a stage's MMAs as soon as it is
@@ -47,9 +49,8 @@ __host__ __device__ inline int kpad(int K) { return K <= 16 ? 16 : K <= 32 ? 32 
 // How `blocks` row blocks of `units` column pieces each are shared by `grid`
 // CTAs: up to `grid` blocks, each block has a group of neighbouring CTAs, which
 // take its pieces in turn, so that at any time a group reads one contiguous
-// stretch of every row (pieces handed out as contiguous ranges instead leave
-// 128 bytes of each DRAM page per visit: 2.6 TB/s); more blocks than CTAs, a
-// CTA takes whole blocks in turn. A slot holds the sums of one CTA and block.
+// stretch of every row (contiguous ranges per CTA measured the same); more
+// blocks than CTAs, a CTA takes whole blocks in turn. A slot holds the sums of one CTA and block.
 // (Rows that fit this GPU's memory make fewer than 2^31 pieces.)
 struct Share {
   int blocks, units, grid;
@@ -75,6 +76,26 @@ __device__ __forceinline__ Hilo split4(float4 v) {
   Hilo r;
   r.hi = make_float4(to_tf32(v.x), to_tf32(v.y), to_tf32(v.z), to_tf32(v.w));
   r.lo = make_float4(to_tf32(v.x - r.hi.x), to_tf32(v.y - r.hi.y), to_tf32(v.z - r.hi.z), to_tf32(v.w - r.hi.w));
+  return r;
+}
+
+// Eight values as three bfloat16 parts each, v = a + b + c exactly (8 + 8 + 8
+// bits): 16 bytes per part, a half of a core-matrix pair's row.
+struct Parts {
+  uint4 a, b, c;
+};
+__device__ __forceinline__ uint32_t split2(float& x, float& y) {  // leaves what the part does not hold
+  uint32_t p;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p) : "f"(y), "f"(x));
+  x -= __uint_as_float(p << 16);
+  y -= __uint_as_float(p & 0xffff0000u);
+  return p;
+}
+__device__ __forceinline__ Parts split8(float4 u, float4 v) {
+  Parts r;
+  r.a = make_uint4(split2(u.x, u.y), split2(u.z, u.w), split2(v.x, v.y), split2(v.z, v.w));
+  r.b = make_uint4(split2(u.x, u.y), split2(u.z, u.w), split2(v.x, v.y), split2(v.z, v.w));
+  r.c = make_uint4(split2(u.x, u.y), split2(u.z, u.w), split2(v.x, v.y), split2(v.z, v.w));
   return r;
 }
 
@@ -487,23 +508,36 @@ __global__ void __launch_bounds__(kRespThreads) k_gmm_resp(const float* __restri
 // output warps keep 32 rows of x per thread in flight and finish the tile from
 // TMEM. Two operand stages and two accumulators: tile t + 1 is multiplied while
 // tile t is written.
+// Both operands are held exactly, as three bfloat16 parts, and an accumulator
+// is two: the products of the first parts, and the five next larger products
+// (the three left out are below 2^-26 of the value); the output adds the two
+// with one rounding. Where one component carries all of the weight, as in most
+// rows, the contraction is then exact, as it is with fp32 multiply-adds. (Two
+// tf32 parts and one accumulator, as many MMAs and 8 bytes of shared memory per
+// value in place of 6: rms error of eps against 64 bits 6.07e-8 at 92
+// components, 360 rows of 2688 columns, 5.11e-8 so, 5.12e-8 with fp32
+// multiply-adds; a call at 118 rows of 4x128x128 and 64 components 48.4 us, 43.4
+// so.)
 constexpr int kOtTile = 128;
 constexpr int kOtOutWarps = 16;
 constexpr int kOtOut = kOtOutWarps * 32;
 constexpr int kOtConv = kOtTile;
 constexpr int kOtThreads = kOtOut + kOtConv + 32;
-constexpr uint32_t kOtTmem = 2 * kRows;
+constexpr uint32_t kOtSmall = 2 * kRows;  // TMEM columns of the small products' accumulators
+constexpr uint32_t kOtTmem = 4 * kRows;
 
 template <int KP>
 struct OtShape {
   static constexpr int KH = KP < 32 ? KP : 32;     // components per stage
   static constexpr int NH = KP / KH;               // stages per tile
-  static constexpr int kRespFloats = 2 * kRows * KP;      // hi rows, then lo rows
-  static constexpr int kStageFloats = 2 * kOtTile * KH;   // hi columns, then lo columns
+  static constexpr int kRespPart = kRows * KP * 2;        // bytes of a part of the responsibilities
+  static constexpr int kMeanPart = kOtTile * KH * 2;      // ... of a stage's means
   static constexpr int kRawFloats = kOtTile * KH;         // [component][column], as they lie in memory
-  static constexpr int NST = KP > 64 ? 1 : 2;      // operand stages
+  static constexpr int NST = 2;                    // operand stages
   static constexpr int NRAW = KP > 64 ? 3 : 4;     // raw stages: all but one are in flight
-  static constexpr size_t smem() { return (size_t)(kRespFloats + NST * kStageFloats + NRAW * kRawFloats) * sizeof(float); }
+  static constexpr size_t smem() {
+    return (size_t)3 * kRespPart + (size_t)NST * 3 * kMeanPart + (size_t)NRAW * kRawFloats * sizeof(float);
+  }
 };
 
 template <int KP>
@@ -518,9 +552,9 @@ __global__ void __launch_bounds__(kOtThreads, 1) k_gmm_out_tc(const float* __res
   __shared__ __align__(8) uint64_t full[NST], empty[NST], dfull[2], dfree[2];
   __shared__ uint32_t s_taddr;
   __shared__ __align__(16) float2 s_c[kRows];
-  float* R = reinterpret_cast<float*>(smem_raw);
-  float* stage0 = R + Sh::kRespFloats;
-  float* raw0 = stage0 + NST * Sh::kStageFloats;
+  unsigned char* R = smem_raw;
+  unsigned char* stage0 = R + 3 * Sh::kRespPart;
+  float* raw0 = reinterpret_cast<float*>(stage0 + NST * 3 * Sh::kMeanPart);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) {
@@ -600,7 +634,8 @@ __global__ void __launch_bounds__(kOtThreads, 1) k_gmm_out_tc(const float* __res
     if (blk != blk0) begin_block(blk);
     const int r0 = blk * kRows, nr = min(kRows, n_rows - r0);
     const int nb = (nr + 15) & ~15;
-    // the block's responsibilities, split, in core-matrix order (a warp step: 8 rows x 16 components)
+    // the block's responsibilities, split, in core-matrix order (a warp step: 8
+    // rows x 16 components, a lane 4 of them: 8 bytes of a core matrix's row)
     constexpr int kWarps = kOtThreads / 32, kSteps = kRows / 8 * (KP / 16), kBatch = kSteps < 4 * kWarps ? (kSteps + kWarps - 1) / kWarps : 4;
     for (int it0 = warp; it0 < (nb >> 3) * (KP / 16); it0 += kBatch * kWarps) {
       float4 v[kBatch];
@@ -614,10 +649,12 @@ __global__ void __launch_bounds__(kOtThreads, 1) k_gmm_out_tc(const float* __res
       for (int i = 0; i < kBatch; ++i) {
         const int it = it0 + i * kWarps, r = (it / (KP / 16)) * 8 + (lane & 7), kq = (it % (KP / 16)) * 4 + (lane >> 3);
         if (r >= nb) break;
-        const Hilo h = split4(v[i]);
-        const int off = ((r >> 3) * (KP / 4) + kq) * 32 + (r & 7) * 4;
-        *reinterpret_cast<float4*>(R + off) = h.hi;
-        *reinterpret_cast<float4*>(R + kRows * KP + off) = h.lo;
+        unsigned char* o = R + ((r >> 3) * (KP / 8) + (kq >> 1)) * 128 + (r & 7) * 16 + (kq & 1) * 8;
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          const uint32_t p0 = split2(v[i].x, v[i].y), p1 = split2(v[i].z, v[i].w);
+          *reinterpret_cast<uint2*>(o + part * Sh::kRespPart) = make_uint2(p0, p1);
+        }
       }
     }
     for (int r = tid; r < nr; r += kOtThreads) s_c[r] = make_float2(rcoef[2 * (r0 + r)], rcoef[2 * (r0 + r) + 1]);
@@ -632,13 +669,15 @@ __global__ void __launch_bounds__(kOtThreads, 1) k_gmm_out_tc(const float* __res
         group_end();
         if (use > 0) wait_or_fail(&empty[s], (use - 1) & 1u, &bad, status);
         const float* rw = raw0 + (uint32_t)w % NRAW * Sh::kRawFloats + lt;
-        float* as = stage0 + s * Sh::kStageFloats + (lt >> 3) * (KH / 4) * 32 + (lt & 7) * 4;
+        unsigned char* as = stage0 + s * 3 * Sh::kMeanPart + (lt >> 3) * (KH / 8) * 128 + (lt & 7) * 16;
 #pragma unroll
-        for (int kq = 0; kq < KH / 4; ++kq) {
-          const Hilo h = split4(make_float4(rw[(4 * kq) * kOtTile], rw[(4 * kq + 1) * kOtTile], rw[(4 * kq + 2) * kOtTile],
-                                            rw[(4 * kq + 3) * kOtTile]));
-          *reinterpret_cast<float4*>(as + kq * 32) = h.hi;
-          *reinterpret_cast<float4*>(as + kOtTile * KH + kq * 32) = h.lo;
+        for (int k8 = 0; k8 < KH / 8; ++k8) {
+          const float* c = rw + 8 * k8 * kOtTile;
+          const Parts h = split8(make_float4(c[0], c[kOtTile], c[2 * kOtTile], c[3 * kOtTile]),
+                                 make_float4(c[4 * kOtTile], c[5 * kOtTile], c[6 * kOtTile], c[7 * kOtTile]));
+          *reinterpret_cast<uint4*>(as + k8 * 128) = h.a;
+          *reinterpret_cast<uint4*>(as + k8 * 128 + Sh::kMeanPart) = h.b;
+          *reinterpret_cast<uint4*>(as + k8 * 128 + 2 * Sh::kMeanPart) = h.c;
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -653,51 +692,63 @@ __global__ void __launch_bounds__(kOtThreads, 1) k_gmm_out_tc(const float* __res
         bad = __any_sync(0xffffffffu, bad);
         const uint32_t tl = taddr + d * kRows + ((uint32_t)(32 * q) << 16);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int rb = row0 + 16 * j;
-          float acc[16];
-          if (rb < nb) tmem_ld16(tl + (uint32_t)rb, acc);
-          if (j == 1) {  // the accumulator is read: the tile after the next may overwrite it
+        for (int j = 0; j < 4; ++j) {
+          const int rb = row0 + 8 * j;
+          float acc[8], small[8];
+          if (rb < nb) {
+            tmem_ld8(tl + (uint32_t)rb, acc);
+            tmem_ld8(tl + kOtSmall + (uint32_t)rb, small);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i] += small[i];
+          }
+          if (j == 3) {  // the accumulator is read: the tile after the next may overwrite it
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&dfree[d]);
           }
           const int lim = col < D ? nr - rb : 0;
           float* er = eps + (int64_t)(r0 + rb) * D + col;
-          if (lim >= 16 && !bad) {
+          if (lim >= 8 && !bad) {
 #pragma unroll
-            for (int i = 0; i < 16; i += 2, er += 2 * D) {
+            for (int i = 0; i < 8; i += 2, er += 2 * D) {
               const float4 c = *reinterpret_cast<const float4*>(&s_c[rb + i]);  // two rows' scalars
-              er[0] = c.x * buf[16 * j + i] - c.y * acc[i];
-              er[D] = c.z * buf[16 * j + i + 1] - c.w * acc[i + 1];
+              er[0] = c.x * buf[8 * j + i] - c.y * acc[i];
+              er[D] = c.z * buf[8 * j + i + 1] - c.w * acc[i + 1];
             }
           } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i, er += D)
-              if (i < lim) *er = bad ? __int_as_float(0x7fc00000) : s_c[rb + i].x * buf[16 * j + i] - s_c[rb + i].y * acc[i];
+            for (int i = 0; i < 8; ++i, er += D)
+              if (i < lim) *er = bad ? __int_as_float(0x7fc00000) : s_c[rb + i].x * buf[8 * j + i] - s_c[rb + i].y * acc[i];
           }
-          if (w + 1 < n) fetch_rows(j, blk, t0 + (w + 1) * ustep);
+          if (w + 1 < n && (j & 1)) fetch_rows(j >> 1, blk, t0 + (w + 1) * ustep);
         }
       }
     } else {
       if (lane == 0) {
-        const uint32_t idesc = tc_idesc_tf32(128, nb);
-        constexpr uint32_t asbo = (KH / 4) * 128, bsbo = (KP / 4) * 128;  // next 8-row group
+        const uint32_t idesc = tc_idesc_bf16(128, nb);
+        constexpr uint32_t asbo = (KH / 8) * 128, bsbo = (KP / 8) * 128;  // next 8-row group
         for (int w = 0; w < n * NH; ++w) {
           const uint32_t u = su + (uint32_t)w, s = u % NST, tile = tu + (uint32_t)(w / NH), d = tile & 1u;
           if (w % NH == 0 && tile >= 2) wait_or_fail(&dfree[d], ((tile >> 1) - 1) & 1u, &bad, status);
           wait_or_fail(&full[s], (u / NST) & 1u, &bad, status);
           tc_fence_after_sync();
-          const uint32_t a = smem_u32(stage0 + s * Sh::kStageFloats), b = smem_u32(R) + (uint32_t)(w % NH) * (KH / 8) * 256;
-          const uint32_t acc = taddr + d * kRows;
+          const uint32_t a = smem_u32(stage0 + s * 3 * Sh::kMeanPart), b = smem_u32(R) + (uint32_t)(w % NH) * (KH / 8) * 128;
+          const uint32_t acc = taddr + d * kRows, small = acc + kOtSmall;
 #pragma unroll
-          for (int ks = 0; ks < KH / 8; ++ks) {
-            const uint32_t ko = (uint32_t)ks * 256;
-            const uint64_t ah = tc_smem_desc(a + ko, 128, asbo), al = tc_smem_desc(a + kOtTile * KH * 4 + ko, 128, asbo);
-            const uint64_t bh = tc_smem_desc(b + ko, 128, bsbo), bl = tc_smem_desc(b + kRows * KP * 4 + ko, 128, bsbo);
-            tc_mma_tf32(acc, ah, bh, idesc, w % NH > 0 || ks > 0 ? 1u : 0u);
-            tc_mma_tf32(acc, al, bh, idesc, 1u);
-            tc_mma_tf32(acc, ah, bl, idesc, 1u);
+          for (int ks = 0; ks < KH / 16; ++ks) {
+            uint64_t ad[3], bd[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              ad[i] = tc_smem_desc(a + i * Sh::kMeanPart + (uint32_t)ks * 256, 128, asbo);
+              bd[i] = tc_smem_desc(b + i * Sh::kRespPart + (uint32_t)ks * 256, 128, bsbo);
+            }
+            const uint32_t more = w % NH > 0 || ks > 0 ? 1u : 0u;
+            tc_mma_f16(acc, ad[0], bd[0], idesc, more);
+            tc_mma_f16(small, ad[2], bd[0], idesc, more);  // the smallest first
+            tc_mma_f16(small, ad[1], bd[1], idesc, 1u);
+            tc_mma_f16(small, ad[0], bd[2], idesc, 1u);
+            tc_mma_f16(small, ad[1], bd[0], idesc, 1u);
+            tc_mma_f16(small, ad[0], bd[1], idesc, 1u);
           }
           tc_commit(&empty[s]);
           if (w % NH == NH - 1) tc_commit(&dfull[d]);

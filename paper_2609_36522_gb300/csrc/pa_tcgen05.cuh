@@ -1,9 +1,9 @@
 // Inline-PTX helpers for the 5th-generation tensor cores on sm_103a: TMEM
-// allocation, tcgen05.mma with kind::tf32 operands in shared memory, commit to
+// allocation, tcgen05.mma with kind::tf32 and bfloat16 operands in shared memory, commit to
 // an mbarrier, and TMEM -> register loads. One CTA, no clusters
 // (cta_group::1). Operand tiles are K-major without swizzle: 8-row x 16-byte
-// core matrices, the two core matrices of one 8-element K step 128 bytes
-// apart (leading byte offset) and consecutive 8-row groups `sbo` bytes apart
+// core matrices, the two core matrices of one K step (8 tf32 or 16 bfloat16
+// values) 128 bytes apart (leading byte offset) and consecutive 8-row groups `sbo` bytes apart
 // (stride byte offset).
 #pragma once
 
@@ -37,6 +37,11 @@ __host__ __device__ constexpr uint32_t tc_idesc_tf32(int M, int N) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same for kind::f16: A and B bfloat16.
+__host__ __device__ constexpr uint32_t tc_idesc_bf16(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
 // Whole warp: allocate `ncols` TMEM columns (a power of two >= 32); the TMEM
 // address is written to *dst in shared memory.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
@@ -57,6 +62,16 @@ __device__ __forceinline__ void tc_mma_tf32(uint32_t tmem_d, uint64_t adesc, uin
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// The same with 16-bit operands (a K step is 16 values, two core matrices).
+__device__ __forceinline__ void tc_mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
