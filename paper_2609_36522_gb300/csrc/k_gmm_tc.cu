@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
 // block summed in CTA order (each thread a fixed share, as an error-free pair,
 // so that the number of CTAs costs no precision), logits, softmax, and the
 // row's two scalars for the output.
-constexpr int kRespThreads = 256;
+constexpr int kRespThreads = 512;
 constexpr int kBatch = 20;       // partial sums in flight per thread: at 64 components 152 of them in two trips
 constexpr int kRespGrid = 4096;  // rows beyond it are taken in turn
 
