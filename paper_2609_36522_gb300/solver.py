@@ -27,6 +27,21 @@ def _stream_ptr(stream):
     return int(stream.cuda_stream), stream
 
 
+# A step hands its batch out between two host waits, so the views of it are on
+# the critical path of a loop driven from Python: the whole workspace is viewed
+# in both element types once, a step takes rows of that. One generation of T 100
+# at 4x64x64 with a PyTorch denoiser, four iterations: 811 us with the bytes
+# sliced and re-typed at each step, 604 so.
+def _typed(workspace):
+    return {t: workspace.view(t) for t in (torch.float32, torch.int32)}
+
+
+def _rows_at(elements, ptr, rows, cols):
+    """The [rows][cols] elements of a workspace from address ``ptr`` on."""
+    first = (int(ptr) - elements.data_ptr()) // 4
+    return elements[first:first + rows * cols].view(rows, cols)
+
+
 class Solver:
     """Cached sliding-window Picard DDIM solver of ``batch`` trajectories."""
 
@@ -43,15 +58,14 @@ class Solver:
         if nbytes == 0:
             raise abi.PaError("pa_workspace_bytes", abi.PA_ERR_ARG, "unsupported sizes")
         self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        self._ws_as = _typed(self.workspace)
         self.h = abi.pa_create(self.T, int(window), self.latent_shape, list(alphas_cumprod),
                                tol, cache_thresh, self.batch, self.workspace.data_ptr(),
                                nbytes, self.stream_ptr)
 
     # -- views into the workspace -------------------------------------------
-    def _view(self, ptr, n, dtype, shape):
-        off = int(ptr) - self.workspace.data_ptr()
-        nb = int(np.prod(shape)) * torch.tensor([], dtype=dtype).element_size()
-        return self.workspace[off: off + nb].view(dtype).view(*shape)
+    def _view(self, ptr, dtype, rows, cols):
+        return _rows_at(self._ws_as[dtype], ptr, rows, cols)
 
     def set_noise(self, eta, noise=None):
         """Stochastic steps: noise is a CUDA float32 [batch][T][D] tensor of
@@ -83,8 +97,7 @@ class Solver:
         st, n, bx, mb = abi.pa_step(self.h)
         if st == abi.PA_DONE:
             return None
-        return Plan(n, self._view(bx, n, torch.float32, (n, self.D)),
-                    self._view(mb, n, torch.int32, (n, 2)), bx, mb)
+        return Plan(n, self._view(bx, torch.float32, n, self.D), self._view(mb, torch.int32, n, 2), bx, mb)
 
     def step_async(self):
         """-> (batch_x_ptr, miss_bt_ptr, n_miss_dev_ptr), no host synchronisation."""
@@ -409,6 +422,7 @@ class SrdsSolver:
             raise ValueError("unsupported sizes for the Parareal sampler")
         dev = torch.device("cuda", torch.cuda.current_device())
         self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+        self._ws_as = _typed(self.workspace)
         self.h = abi.pa_srds_create(self.T, self.latent_shape, list(alphas_cumprod), tol, cache_thresh,
                                     self.batch, self.workspace.data_ptr(), nbytes, self.stream_ptr)
         st = abi.pa_srds_stats(self.h)
@@ -422,17 +436,15 @@ class SrdsSolver:
         self._x_init_keepalive = x
         abi.pa_srds_init(self.h, x.data_ptr())
 
-    def _view(self, ptr, dtype, shape):
-        off = int(ptr) - self.workspace.data_ptr()
-        nb = int(np.prod(shape)) * torch.tensor([], dtype=dtype).element_size()
-        return self.workspace[off: off + nb].view(dtype).view(*shape)
+    def _view(self, ptr, dtype, rows, cols):
+        return _rows_at(self._ws_as[dtype], ptr, rows, cols)
 
     def step(self):
         """-> None when done, else a Plan of the next evaluation stage."""
         st, n, bx, mb = abi.pa_srds_step(self.h)
         if st == abi.PA_DONE:
             return None
-        return Plan(n, self._view(bx, torch.float32, (n, self.D)), self._view(mb, torch.int32, (n, 2)), bx, mb)
+        return Plan(n, self._view(bx, torch.float32, n, self.D), self._view(mb, torch.int32, n, 2), bx, mb)
 
     def n_miss_dev(self):
         return abi.pa_srds_n_miss_dev(self.h)
