@@ -561,25 +561,24 @@ PA_API pa_status pa_gmm_check(pa_gmm* g);
 PA_API int64_t pa_gmm_launches(const pa_gmm* g);
 
 /* How pa_gmm_eps computes (a choice of this library; the paper has no
- * counterpart). form 2 (the default for K <= 16 when D is a multiple of 64 and
- * max_rows < 768): one kernel -- a thread-block cluster of 16 CTAs per block of
- * 8 rows, each CTA one sixteenth of the columns; the partial dot products
- * x . mu_k are summed across the cluster through distributed shared memory and
- * every CTA writes its columns of eps from the row and mean tiles it staged
- * once. form 1: both contractions on the tensor cores (tcgen05, kind::tf32,
- * every operand split into two tf32 parts and the products summed, which keeps
- * fp32 accuracy). A handle for large problems (K rounded up to a power of two,
- * at least 16, times D times 128-row blocks of max_rows is 700,000 or more,
- * and K > 16 or max_rows >= 768) runs three persistent kernels, one CTA per SM,
- * for any D and alignment; smaller ones a CTA per 64 columns x 128 rows, then
- * an output kernel -- for 16 < K <= 64 and D % 64 == 0 the output contraction
- * on the tensor cores as well -- and need D % 4 == 0 and 16-byte aligned means.
- * Form 1 needs a GPU of the sm_100 family; it is the default when K > 16, and
- * when max_rows >= 768 for such large problems. form 0: fp32 FMA dot products
- * on the CUDA cores, then the output kernel. A call whose batch_x or batch_eps
- * is not 16-byte aligned uses form 0 in place of form 2 and of the smaller
- * problems' form 1. The forms agree to fp32 rounding; each is bitwise
- * reproducible. Returns PA_ERR_ARG for a form that is not available. */
+ * counterpart). form 2: one kernel -- a thread-block cluster of 16 CTAs per
+ * block of 8 rows, each CTA one sixteenth of the columns; the partial dot
+ * products x . mu_k are summed across the cluster through distributed shared
+ * memory and every CTA writes its columns of eps from the row and mean tiles it
+ * staged once; for K <= 16 and D a multiple of 64. form 1: both contractions on
+ * the tensor cores (tcgen05), three persistent kernels, one CTA per SM, for any
+ * D and alignment; operands split into parts so that the result keeps fp32
+ * accuracy. form 0: fp32 multiply-adds on the CUDA cores, two kernels.
+ * The default goes by sizes: for K > 16 form 1 where K D max_rows is 40e6 or
+ * more (12e6 for K > 64), else form 0; for K <= 16 form 2 where it is available,
+ * except form 0 for max_rows >= 200 with D <= 10000 and D <= 25 max_rows, and
+ * form 1 where K D max_rows is 250e6 or more with max_rows >= 512; where form 2 is not available form 0, except form
+ * 1 for K > 8, D % 4 == 0, aligned means and K D max_rows of 100e6 or more.
+ * A call whose batch_x or batch_eps is not 16-byte aligned uses form 0 in place
+ * of form 2. Forms 1 and 2 need a GPU of the sm_100 family, and to be set here
+ * D % 4 == 0 and 16-byte aligned means. The forms agree to fp32 rounding; each
+ * is bitwise reproducible. Returns PA_ERR_ARG for a form that is not
+ * available. */
 PA_API pa_status pa_gmm_set_form(pa_gmm* g, int form);
 
 /* The form pa_gmm_eps uses: 2, 1 or 0, -1 for NULL. */

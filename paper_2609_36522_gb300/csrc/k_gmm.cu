@@ -6,22 +6,19 @@
 //   r = softmax(logit)   (the common -||x||^2 / (2 v) term cancels)
 //   eps = sqrt(1 - a) / v * (x - sqrt(a) sum_k r_k mu_k)
 //
-// Four ways to compute it, chosen per handle (pa_gmm_create):
+// Three ways to compute it, chosen per handle (pa_gmm_create):
 //   one kernel on thread-block clusters (k_gmm_cluster, form 2)
-//   three persistent tensor-core kernels (k_gmm_tc.cu, form 1, large problems)
-//   the tensor-core kernels below, a CTA per 64-column chunk (form 1, small
-//   problems), and CUDA-core kernels (form 0), two or three kernels per call:
-//   dot products   G = X M^T, split over column chunks of D, either on the
-//                  tensor cores (k_gmm_dots_tc: tcgen05, tf32 operands split
-//                  in two parts for fp32 accuracy) or on the CUDA cores
-//                  (k_gmm_dots: bulk-staged 16-row tiles, 4 rows x 8
+//   three persistent tensor-core kernels (k_gmm_tc.cu, form 1)
+//   two CUDA-core kernels (form 0):
+//   k_gmm_dots     dot products G = X M^T, split over column chunks of D
+//                  (16-row tiles staged in shared memory, 4 rows x 8
 //                  components per thread); each CTA adds its chunk sums, in
 //                  2^-32 fixed point, into int64 accumulators with integer
 //                  atomics (exact: the order of arrival does not matter)
 //   k_gmm_out      per 16-row block: logits and max-subtracted softmax of its
 //                  rows from the accumulators, then eps = a x - a sqrt(a) R M
-//                  over bulk-staged 16-row x 256-column tiles (4 x 4 outputs
-//                  per thread)
+//                  over staged 16-row x 256-column tiles (4 x 4 outputs per
+//                  thread)
 // The accumulators come in two sets used in turn. A call's dot-product kernel
 // reads the handle's epoch e, accumulates into set e mod 2, clears the other
 // set (read by the previous call's output kernel, which has completed) and
@@ -43,7 +40,6 @@
 #include "pa_bulk.cuh"
 #include "pa_gmm_tc.h"
 #include "pa_internal.h"
-#include "pa_tcgen05.cuh"
 
 namespace pa {
 void set_error(const std::string& msg);  // pa_solver.cpp
@@ -61,17 +57,6 @@ using pa::mbar_arrive_expect_tx;
 using pa::mbar_init;
 using pa::mbar_wait_bounded;
 using pa::smem_u32;
-using pa::tc_commit;
-using pa::tc_fence_after_sync;
-using pa::tc_fence_before_sync;
-using pa::tc_idesc_tf32;
-using pa::tc_mma_tf32;
-using pa::tc_smem_desc;
-using pa::tmem_alloc;
-using pa::tmem_dealloc;
-using pa::tmem_ld16;
-using pa::to_tf32;
-using pa::fence_proxy_async_smem;
 
 constexpr int kMaxK = 128;
 constexpr int kThreads = 256;
@@ -82,53 +67,38 @@ constexpr size_t kDotSmemBudget = 96 * 1024;
 constexpr int kDotCtas = 120;    // CTAs that a dots launch should have (of 152 SMs)
 constexpr float kDotScale = 4294967296.f;  // 2^32: fixed-point scale of the dot-product accumulators
 
-// tensor-core dot products: rows per CTA (the MMA's M), columns per CTA
-constexpr int kTcRows = 128;
-constexpr int kTcCols = 64;   // 8 MMA steps of 8 (98 KB of shared memory at K = 64: two CTAs per SM)
-constexpr int kTcThreads = 256;
-constexpr int kTcCluster = 8;            // column chunks per thread-block cluster ...
-constexpr int kTcClusterMinChunks = 256;  // ... when there are this many chunks (fewer atomics per accumulator)
-constexpr int kTcMinK = 16;               // tensor cores by default above this many components ...
-constexpr int kTcMinRows = 768;           // ... or from this many rows on: at 4x64x64, 16 trajectories of a 100-point
-                                          // window and 16 components a generation takes 945 us, in form 2 1020 us
-// Whether form 1 runs as the persistent kernels of k_gmm_tc.cu: they fill the
-// GPU with one CTA per SM whatever the shape, which costs about 2 us more than
-// small CTAs that overlap where there is little to do. us per call, small CTAs
-// against persistent, at K components, D columns, a capacity of R rows:
-// K 20, D 16384, R 100: 13.6 / 16.1; K 24, D 4096, R 300: 14.9 / 17.5;
-// K 40, D 13056, R 100: 21.6 / 18.9; K 58, D 9216, R 138: 26.9 / 19.9;
-// K 96, D 16384, R 200: 104.5 / 37.5; K 64, D 65536, R 128: 72.7 / 46.6.
-// (They take any D and any alignment, the kernels here whole 16-byte rows.)
-constexpr int64_t kTcPersistentWork = 700 * 1000;
-
-// the MMA's N: K rounded up to 16, 32, 64 or 128 (padded means are zero)
-__host__ __device__ inline int tc_npad(int K) {
-  int n = 16;
-  while (n < K) n <<= 1;
-  return n;
-}
-// floats of one column chunk's means image: hi and lo, Kp rows each
-__host__ __device__ inline size_t tc_mu_chunk_floats(int K) { return (size_t)2 * tc_npad(K) * kTcCols; }
-// The tensor-core output contraction: kOtCols columns per CTA (two CTAs per
-// SM), up to 64 (padded) components; its operand images hold hi rows, then lo
-// rows, of tc_npad(K) values in core-matrix order: 2 x 128 rows of
-// responsibilities, 2 x kOtCols rows (columns of D) of means.
-constexpr int kOtCols = 64;
-constexpr int kOtThreads = 256;
-constexpr int kOtMaxKp = 64;
-constexpr int kRespRows = 8;  // rows per k_gmm_resp CTA, a warp each
-__host__ __device__ inline size_t ot_img_floats(int K) { return (size_t)2 * kTcRows * tc_npad(K); }
-__host__ __device__ inline size_t ot_mut_floats(int K) { return (size_t)2 * kOtCols * tc_npad(K); }
-
-bool tc_persistent(int K, int64_t D, int max_rows) {
-  const int64_t blocks = ((int64_t)max_rows + kTcRows - 1) / kTcRows;
-  return (int64_t)(K <= 16 ? 16 : tc_npad(K)) * D * blocks >= kTcPersistentWork && (K > kTcMinK || max_rows >= kTcMinRows);
-}
+// Default form by sizes (pa_gmm_create). K components, D columns, a capacity of R
+// rows; the figures are us per call on a batch filled to 4/5.
+// Above 16 components the persistent tensor-core kernels (form 1) cost 12 us
+// before they do anything, the CUDA-core kernels (form 0) 6, and those take time
+// with K: form 1 from K D R = kTcWork on, above 64 components from kTcWideWork.
+// Form 0 / 1: K 32, D 8192, R 64 (17e6) 10.5 / 13.7; K 32, D 16384, R 64 (34e6)
+// 13.3 / 15.6; K 64, D 8192, R 128 (67e6) 20.1 / 16.5; K 64, D 65536, R 128
+// (537e6) 145 / 41; K 90, D 8192, R 16 (12e6) 16.0 / 17.4; K 128, D 4096, R 64
+// (34e6) 23.2 / 17.9; a generation at K 95, D 784, R 306 (23e6) 278 / 226.
+// Up to 16 components the cluster kernel (form 2) is the shortest chain, but its
+// time goes with the rows, eight to a cluster of 16 CTAs, however few columns
+// they have: form 0 for many short rows. Form 0 / 2: K 8, D 4096, R 256 7.9 / 9.8,
+// R 100 8.6 / 5.2; K 8, D 8192, R 256 10.2 / 10.8, R 400 14.7 / 16.9; K 16,
+// D 16384, R 400 30.1 / 24.9; a generation at K 4, D 4224, R 256 815 / 910.
+// Where the work is large form 1 wins here too: form 0 / 1 / 2 at K 16, D 16384,
+// R 1000 (262e6) 63.1 / 56.4 / 58.6, R 1600 86.8 / 73.2 / 81.1; without the
+// cluster kernel form 0 / 1 at K 16, D 40000, R 256 (164e6) 42.4 / 38.1, at K 8,
+// R 1000 (320e6) 110 / 122, and with D % 4 != 0, where form 1 copies four bytes at
+// a time, at K 16, D 40001, R 1000 170 / 188.
+constexpr int64_t kTcWork = 40 * 1000 * 1000;
+constexpr int64_t kTcWideWork = 12 * 1000 * 1000;
+constexpr int kManyRows = 200;        // many short rows: R >= kManyRows, D <= kShortRow,
+constexpr int64_t kShortRow = 10000;  // and D <= kShortPerRow R
+constexpr int64_t kShortPerRow = 25;
+constexpr int64_t kTcFewWork = 250 * 1000 * 1000;   // up to 16 components, against form 2 ...
+constexpr int kTcFewRows = 512;
+constexpr int64_t kTcFewWork0 = 100 * 1000 * 1000;  // ... and against form 0
+constexpr int kTcFewMinK = 9;
 
 struct GmmLayout {
   size_t tc;        // scratch of the persistent tensor-core kernels
-  size_t coef, mnorm, gacc, epoch, status, mu_img, mut_img, r_img, rcoef, total;
-  int tc_chunks;    // column chunks of the tensor-core dot products (whole clusters)
+  size_t coef, mnorm, gacc, epoch, status, total;
   int nchunk;       // D-chunks of the CUDA-core dots kernel
   int chunk;        // columns per chunk
 };
@@ -171,16 +141,7 @@ GmmLayout gmm_layout(int K, int64_t D, int max_rows, int T) {
   L.gacc = take((size_t)2 * max_rows * K * sizeof(long long));  // two sets, used in turn
   L.epoch = take(sizeof(GmmEpoch));
   L.status = take(sizeof(int32_t));
-  L.tc_chunks = (int)((D + kTcCols - 1) / kTcCols + kTcCluster - 1) / kTcCluster * kTcCluster;  // whole clusters
-  const bool per = tc_persistent(K, D, max_rows);
-  L.tc = take(per ? pa::gmm_tc_layout(K, max_rows).total : 0);
-  L.mu_img = take(per ? 0 : (size_t)L.tc_chunks * tc_mu_chunk_floats(K) * sizeof(float));
-  // the tensor-core output contraction (16 < K <= 64): the means' transposed
-  // split image, the responsibilities' split image and the rows' scalars
-  const bool ot = !per && K > kTcMinK && tc_npad(K) <= kOtMaxKp;
-  L.mut_img = take(ot ? (size_t)((D + kOtCols - 1) / kOtCols) * ot_mut_floats(K) * sizeof(float) : 0);
-  L.r_img = take(ot ? (size_t)((max_rows + kTcRows - 1) / kTcRows) * ot_img_floats(K) * sizeof(float) : 0);
-  L.rcoef = take(ot ? (size_t)2 * max_rows * sizeof(float) : 0);
+  L.tc = take(pa::gmm_tc_layout(K, max_rows).total);
   L.total = o;
   return L;
 }
@@ -501,443 +462,6 @@ __global__ void __launch_bounds__(kThreads) k_gmm_out(const float* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// Tensor-core form of the dot products (tcgen05, kind::tf32). G = X M^T is a
-// dense contraction over D: a CTA takes a block of 128 rows (M = 128, rows past
-// the count are zero) and a chunk of kTcCols columns, and computes the
-// 128 x Kp partial product (Kp = K rounded up to 16, 32, 64 or 128; padded
-// means are zero) in TMEM with single-thread tcgen05.mma issue. fp32 accuracy
-// from tf32 operands: every value is split as v = hi + lo with
-// hi = tf32(v), lo = tf32(v - hi), and the product summed as
-// hi*hi + hi*lo + lo*hi (the lo*lo term is below fp32 resolution). The rows are
-// split by the CTA's threads into core-matrix order in shared memory; the
-// means' split image is prepared once per handle (k_gmm_mu_image) and arrives
-// by one bulk copy. Chunk sums go into the fixed-point accumulators as in
-// k_gmm_dots (with a thread-block cluster of kTcCluster chunks, the cluster's
-// partial sums are first added through distributed shared memory, which cuts
-// the atomics on each accumulator by that factor).
-__host__ inline size_t tc_smem_bytes(int K) {
-  return ((size_t)2 * kTcRows * kTcCols + tc_mu_chunk_floats(K)) * sizeof(float);
-}
-// element (r, c) of a K-major tile with kTcCols columns, in core-matrix order:
-// 8-row groups of (kTcCols / 4) core matrices of 8 rows x 4 values
-__host__ __device__ inline int tc_off(int r, int c) {
-  return ((r >> 3) * (kTcCols / 4) + (c >> 2)) * 32 + (r & 7) * 4 + (c & 3);
-}
-
-// The means' split image, once per handle: chunk ch, part (0 hi, 1 lo), in
-// core-matrix order with Kp rows.
-__global__ void __launch_bounds__(256) k_gmm_mu_image(const float* __restrict__ mu, int K, int64_t D,
-                                                      float* __restrict__ img) {
-  const int Kp = tc_npad(K);
-  const int64_t ch = blockIdx.x;
-  float* out = img + ch * tc_mu_chunk_floats(K);
-  for (int q = threadIdx.x; q < Kp * kTcCols; q += 256) {
-    const int k = q / kTcCols, c = q % kTcCols;
-    const int64_t col = ch * kTcCols + c;
-    const float v = (k < K && col < D) ? mu[(int64_t)k * D + col] : 0.f;
-    const float hi = to_tf32(v);
-    out[tc_off(k, c)] = hi;
-    out[(size_t)Kp * kTcCols + tc_off(k, c)] = to_tf32(v - hi);
-  }
-}
-
-template <int CL>
-__global__ void __launch_bounds__(kTcThreads) k_gmm_dots_tc(const float* __restrict__ X,
-                                                            const float* __restrict__ mu_img,
-                                                            const int32_t* __restrict__ n_rows_dev, int K,
-                                                            int64_t D, int max_rows,
-                                                            long long* __restrict__ gacc2, GmmEpoch* ep,
-                                                            int32_t* status) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bar_mu;
-  __shared__ __align__(8) uint64_t bar_mma;
-  __shared__ uint32_t s_taddr;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  long long* gacc = begin_dots(gacc2, ep, (int64_t)max_rows * K);
-  const int r0 = blockIdx.y * kTcRows;
-  const int Kp = tc_npad(K);
-  const uint32_t ncols = 2 * Kp < 32 ? 32u : (uint32_t)(2 * Kp);  // TMEM columns: a power of two >= 32
-  const int64_t c0 = (int64_t)blockIdx.x * kTcCols;
-  float* A_hi = reinterpret_cast<float*>(smem_raw);
-  float* A_lo = A_hi + kTcRows * kTcCols;
-  float* B_img = A_lo + kTcRows * kTcCols;  // hi then lo, Kp rows each
-  if (tid == 0) {
-    mbar_init(&bar_mu, 1);
-    mbar_init(&bar_mma, 1);
-    fence_barrier_init();
-  }
-  if (warp == 0) {
-    tmem_alloc(&s_taddr, ncols);
-    tc_fence_before_sync();
-  }
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t taddr = s_taddr;
-  if (tid == 0) {  // the means image does not depend on the predecessor
-    const uint32_t bytes = (uint32_t)(tc_mu_chunk_floats(K) * sizeof(float));
-    mbar_arrive_expect_tx(&bar_mu, bytes);
-    bulk_g2s(B_img, mu_img + (size_t)blockIdx.x * tc_mu_chunk_floats(K), bytes, &bar_mu);
-  }
-  pdl_wait();  // the rows and their count come from the kernel just before
-  pdl_trigger();  // the successor may now run its prologue
-  const int n_rows = min(*n_rows_dev, max_rows);
-  const int nr = min(kTcRows, n_rows - r0);
-  if (nr <= 0) {  // no rows for this block (the whole cluster alike): the means copy
-                  // lands and TMEM is freed before the CTA exits
-    if (!mbar_wait_bounded(&bar_mu, 0, pa::kDrainLimit) && tid == 0) atomicCAS(status, 0, pa::kDevTimeout);
-    tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(taddr, ncols);
-    return;
-  }
-
-  // rows -> (hi, lo) in core-matrix order: a warp step covers 8 rows x 16
-  // columns; lanes 8q..8q+7 write one 128-byte core matrix (conflict-free).
-  // All of a thread's loads are issued before the first conversion.
-  {
-    constexpr int kSteps = (kTcRows / 8) * (kTcCols / 16);
-    constexpr int kPer = kSteps / (kTcThreads / 32);
-    const int rin = lane & 7, kq = lane >> 3;
-    float4 v[kPer];
-#pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int it = warp + u * (kTcThreads / 32);
-      const int g = it / (kTcCols / 16), kb = (it % (kTcCols / 16)) * 4 + kq;
-      const int r = g * 8 + rin, c = kb * 4;
-      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (r < nr && c0 + c < D) v[u] = __ldg(reinterpret_cast<const float4*>(X + (int64_t)(r0 + r) * D + c0 + c));
-    }
-#pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int it = warp + u * (kTcThreads / 32);
-      const int g = it / (kTcCols / 16), kb = (it % (kTcCols / 16)) * 4 + kq;
-      const int r = g * 8 + rin, c = kb * 4;
-      float4 hi, lo;
-      hi.x = to_tf32(v[u].x); lo.x = to_tf32(v[u].x - hi.x);
-      hi.y = to_tf32(v[u].y); lo.y = to_tf32(v[u].y - hi.y);
-      hi.z = to_tf32(v[u].z); lo.z = to_tf32(v[u].z - hi.z);
-      hi.w = to_tf32(v[u].w); lo.w = to_tf32(v[u].w - hi.w);
-      const int off = tc_off(r, c);
-      *reinterpret_cast<float4*>(A_hi + off) = hi;
-      *reinterpret_cast<float4*>(A_lo + off) = lo;
-    }
-  }
-  fence_proxy_async_smem();  // the tensor core reads what the threads wrote
-  // every decision below is taken by the whole CTA (__syncthreads_and)
-  bool ok = __syncthreads_and(mbar_wait_bounded(&bar_mu, 0, pa::kWaitLimit));
-  if (!ok) {
-    if (tid == 0) atomicCAS(status, 0, pa::kDevTimeout);
-    mbar_wait_bounded(&bar_mu, 0, pa::kDrainLimit);  // the copy lands before the CTA moves on
-  }
-  if (tid == 0 && ok) {
-    tc_fence_after_sync();
-    // The means image's hi rows are directly followed by its lo rows, so one
-    // N = 2 Kp product gives hi*hi in columns [0, Kp) and hi*lo in [Kp, 2 Kp);
-    // lo*hi then accumulates into [0, Kp): two MMAs per k-step.
-    const uint32_t idesc2 = tc_idesc_tf32(kTcRows, 2 * Kp), idesc1 = tc_idesc_tf32(kTcRows, Kp);
-    const uint32_t a_hi = smem_u32(A_hi), a_lo = smem_u32(A_lo);
-    const uint32_t b_hi = smem_u32(B_img);
-    const uint32_t sbo = (kTcCols / 4) * 128;  // next 8-row group
-    for (int ks = 0; ks < kTcCols / 8; ++ks) {
-      const uint32_t ko = (uint32_t)ks * 256;  // two core matrices along K per step
-      const uint64_t dah = tc_smem_desc(a_hi + ko, 128, sbo), dal = tc_smem_desc(a_lo + ko, 128, sbo);
-      const uint64_t db = tc_smem_desc(b_hi + ko, 128, sbo);
-      tc_mma_tf32(taddr, dah, db, idesc2, ks > 0 ? 1u : 0u);
-      tc_mma_tf32(taddr, dal, db, idesc1, 1u);
-    }
-    tc_commit(&bar_mma);
-  }
-  if (ok && !__syncthreads_and(mbar_wait_bounded(&bar_mma, 0, pa::kWaitLimit))) {
-    if (tid == 0) atomicCAS(status, 0, pa::kDevTimeout);
-    mbar_wait_bounded(&bar_mma, 0, pa::kDrainLimit);  // let the MMAs finish before TMEM is freed
-    ok = false;
-  }
-  tc_fence_after_sync();
-  float* part = A_hi;  // [kTcRows][Kp]: this CTA's partial sums (the operands are consumed)
-  if (warp < 4 && ok) {  // warp w reads TMEM lanes (rows) 32w .. 32w + 31
-    const int row = warp * 32 + lane;
-    for (int cb = 0; cb < Kp; cb += 16) {
-      float v[16], w[16];
-      tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)cb, v);
-      tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)(Kp + cb), w);
-#pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] += w[u];  // (hi*hi + lo*hi) + hi*lo
-      if constexpr (CL > 1) {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) part[row * Kp + cb + u] = v[u];
-      } else if (row < nr) {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int k = cb + u;
-          if (k < K)
-            atomicAdd(reinterpret_cast<unsigned long long*>(gacc + (int64_t)(r0 + row) * K + k),
-                      static_cast<unsigned long long>(__float2ll_rn(v[u] * kDotScale)));
-        }
-      }
-    }
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(taddr, ncols);
-  if constexpr (CL > 1) {
-    // the CL column chunks of a cluster are added through distributed shared
-    // memory in rank order; rank q then adds rows [q R, (q+1) R) to gacc
-    cg::cluster_group cluster = cg::this_cluster();
-    if (!ok)
-      for (int q = tid; q < kTcRows * Kp; q += kTcThreads) part[q] = 0.f;
-    cluster.sync();
-    const int rank = (int)cluster.block_rank();
-    constexpr int kRowsPer = kTcRows / CL;
-    for (int o = tid; o < kRowsPer * K; o += kTcThreads) {
-      const int rr = rank * kRowsPer + o / K, k = o % K;
-      if (rr < nr) {
-        float sum = 0.f;
-        for (int q = 0; q < CL; ++q) sum += cluster.map_shared_rank(part, q)[rr * Kp + k];
-        atomicAdd(reinterpret_cast<unsigned long long*>(gacc + (int64_t)(r0 + rr) * K + k),
-                  static_cast<unsigned long long>(__float2ll_rn(sum * kDotScale)));
-      }
-    }
-    cluster.sync();  // peers read this CTA's partial sums until here
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Tensor-core form of the output contraction, for 16 < K <= 64 (with the
-// tensor-core dot products, form 1). eps = a x - a sqrt(a) R M, and R M is a
-// dense contraction over the components: rows x K times K x D.
-// k_gmm_resp forms each row's responsibilities once -- the same logits and
-// max-subtracted softmax as k_gmm_out -- and writes them as a split image
-// (hi = tf32(R), lo = tf32(R - hi), in core-matrix order, K-major); then
-// k_gmm_out_tc takes a block of 128 rows (M = 128; rows past the count are
-// zero) and kOtCols columns: one bulk copy brings the responsibilities'
-// image, another the means' transposed split image of its columns (built once
-// per handle, k_gmm_mut_image: the hi rows of the kOtCols columns followed by
-// their lo rows), one thread issues R_hi [M_hi; M_lo]^T (N = 2 kOtCols,
-// columns [0, kOtCols) hi*hi and [kOtCols, 2 kOtCols) hi*lo) and R_lo M_hi^T
-// (accumulated into [0, kOtCols)) per 8-component step into TMEM, and every
-// thread reads its row's
-// accumulators back (tcgen05.ld, one row per TMEM lane) and writes its
-// columns of eps from the row values it loaded before the dependency wait.
-
-// element (r, c) of a K-major tile with Kp columns, in core-matrix order
-__host__ __device__ inline int ot_off(int r, int c, int Kp) {
-  return ((r >> 3) * (Kp >> 2) + (c >> 2)) * 32 + (r & 7) * 4 + (c & 3);
-}
-
-// The means' transposed split image, once per handle: chunk ch of kOtCols
-// columns, rows n (column ch * kOtCols + n; n >= kOtCols: the lo parts) x
-// components.
-__global__ void __launch_bounds__(256) k_gmm_mut_image(const float* __restrict__ mu, int K, int64_t D,
-                                                       float* __restrict__ img) {
-  const int Kp = tc_npad(K);
-  const int64_t ch = blockIdx.x;
-  float* out = img + ch * ot_mut_floats(K);
-  for (int q = threadIdx.x; q < Kp * kOtCols; q += 256) {
-    const int k = q / kOtCols, n = q % kOtCols;  // consecutive threads read consecutive columns
-    const int64_t col = ch * kOtCols + n;
-    const float v = (k < K && col < D) ? mu[(int64_t)k * D + col] : 0.f;
-    const float hi = to_tf32(v);
-    out[ot_off(n, k, Kp)] = hi;
-    out[ot_off(n + kOtCols, k, Kp)] = to_tf32(v - hi);
-  }
-}
-
-// The responsibilities of every row (a warp per row) as the split image of
-// its 128-row block, and the row's scalars (a, a sqrt(a)) for the epilogue;
-// rows past the count (up to the end of their block) are zero. Advances the
-// accumulator epoch as k_gmm_out does.
-__global__ void __launch_bounds__(kRespRows * 32) k_gmm_resp(const long long* __restrict__ gacc2, GmmEpoch* ep,
-                                                             const float* __restrict__ coef, int T,
-                                                             const int32_t* __restrict__ miss_bt,
-                                                             const float* __restrict__ mnorm,
-                                                             const int32_t* __restrict__ n_rows_dev, int K,
-                                                             int max_rows, float* __restrict__ rimg,
-                                                             float* __restrict__ rcoef) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * kRespRows + warp;
-  const int Kp = tc_npad(K);
-  const int n_rows = min(*n_rows_dev, max_rows);  // written two kernels back
-  float sa = 0.f, q = 0.f, c = 0.f;
-  if (r < n_rows) {
-    const int i = miss_bt[2 * r + 1];
-    sa = coef[i];
-    q = coef[T + i];
-    c = coef[2 * T + i];
-  }
-  pdl_wait();     // the dot products come from the kernel just before
-  pdl_trigger();  // the successor may now run its prologue
-  const uint32_t cur = ep->cur;
-  float* blk = rimg + (size_t)(r / kTcRows) * ot_img_floats(K);
-  const int rr = r % kTcRows;
-  float rv[2] = {0.f, 0.f};  // components lane and lane + 32
-  if (r < n_rows) {
-    const long long* g = gacc2 + (int64_t)(cur & 1u) * max_rows * K + (int64_t)r * K;
-    float l[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int k = lane + 32 * u;
-      if (k < K) {
-        const float dot = __ll2float_rn(__ldcg(g + k)) * (1.f / kDotScale);  // exact scale
-        l[u] = (2.f * sa * dot - sa * sa * mnorm[k]) * q;
-      }
-    }
-    float mx = fmaxf(l[0], l[1]);  // the order of k_gmm_out's loop: k = lane, then lane + 32
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float sum = 0.f;
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (lane + 32 * u < K) sum += expf(l[u] - mx);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    const float inv = 1.f / sum;
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (lane + 32 * u < K) rv[u] = expf(l[u] - mx) * inv;
-    if (lane == 0) {
-      rcoef[2 * r] = c;
-      rcoef[2 * r + 1] = c * sa;
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int k = lane + 32 * u;
-    if (k < Kp) {
-      const float hi = to_tf32(rv[u]);
-      blk[ot_off(rr, k, Kp)] = hi;
-      blk[ot_off(rr + kTcRows, k, Kp)] = to_tf32(rv[u] - hi);
-    }
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) ep->epoch = cur + 1u;  // the next call's set
-}
-
-__host__ inline size_t ot_smem_bytes(int K) {
-  // both split images; at least 60 KB so that at most three CTAs (3 x 128 TMEM columns) share an SM
-  const size_t b = (ot_img_floats(K) + ot_mut_floats(K)) * sizeof(float);
-  return b < 60 * 1024 ? 60 * 1024 : b;
-}
-
-__global__ void __launch_bounds__(kOtThreads, 2) k_gmm_out_tc(const float* __restrict__ X,
-                                                              const float* __restrict__ mut_img,
-                                                              const float* __restrict__ rimg,
-                                                              const float* __restrict__ rcoef,
-                                                              const int32_t* __restrict__ n_rows_dev, int K,
-                                                              int64_t D, int max_rows, float* __restrict__ eps,
-                                                              int32_t* status) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bar_b, bar_a, bar_mma;
-  __shared__ uint32_t s_taddr;
-  constexpr uint32_t kTmemCols = 2 * kOtCols;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int Kp = tc_npad(K);
-  const size_t img = ot_img_floats(K), mimg = ot_mut_floats(K);
-  float* A = reinterpret_cast<float*>(smem_raw);  // responsibilities: hi rows, then lo rows
-  float* B = A + img;                              // means of the columns: hi rows, then lo rows
-  const int64_t c0 = (int64_t)blockIdx.x * kOtCols;
-  const int r0 = blockIdx.y * kTcRows;
-  if (tid == 0) {
-    mbar_init(&bar_b, 1);
-    mbar_init(&bar_a, 1);
-    mbar_init(&bar_mma, 1);
-    fence_barrier_init();
-  }
-  if (warp == 0) {
-    tmem_alloc(&s_taddr, kTmemCols);
-    tc_fence_before_sync();
-  }
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t taddr = s_taddr;
-  const uint32_t img_bytes = (uint32_t)(img * sizeof(float)), mimg_bytes = (uint32_t)(mimg * sizeof(float));
-  if (tid == 0) {  // the means image does not change
-    mbar_arrive_expect_tx(&bar_b, mimg_bytes);
-    bulk_g2s(B, mut_img + (size_t)blockIdx.x * mimg, mimg_bytes, &bar_b);
-  }
-  // the rows and their count were written three kernels back: thread (warp,
-  // lane) takes row 32 (warp % 4) + lane (its TMEM lane) and the 64 columns
-  // of half warp / 4
-  const int n_rows = min(*n_rows_dev, max_rows);
-  const int nr = min(kTcRows, n_rows - r0);
-  const int row = 32 * (warp & 3) + lane, half = warp >> 2;
-  const int64_t cb0 = c0 + half * (kOtCols / 2);
-  float4 xv[kOtCols / 8];
-  if (row < nr) {
-    const float4* xr = reinterpret_cast<const float4*>(X + (int64_t)(r0 + row) * D + cb0);
-#pragma unroll
-    for (int u = 0; u < kOtCols / 8; ++u) xv[u] = __ldg(xr + u);
-  }
-  pdl_wait();     // the responsibilities and the row scalars come from the kernel just before
-  pdl_trigger();  // the successor may now run its prologue
-  if (nr <= 0) {  // no rows in this block: the means copy lands and TMEM is freed
-    if (!mbar_wait_bounded(&bar_b, 0, pa::kDrainLimit) && tid == 0) atomicCAS(status, 0, pa::kDevTimeout);
-    tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(taddr, kTmemCols);
-    return;
-  }
-  if (tid == 0) {
-    mbar_arrive_expect_tx(&bar_a, img_bytes);
-    bulk_g2s(A, rimg + (size_t)blockIdx.y * img, img_bytes, &bar_a);
-  }
-  const bool dots_bad = __ldcg(status) != 0;  // a dot-product wait ran out: the sums are incomplete
-  bool ok = __syncthreads_and(mbar_wait_bounded(&bar_b, 0, pa::kWaitLimit) &&
-                              mbar_wait_bounded(&bar_a, 0, pa::kWaitLimit));
-  if (!ok) {
-    if (tid == 0) atomicCAS(status, 0, pa::kDevTimeout);
-    mbar_wait_bounded(&bar_b, 0, pa::kDrainLimit);  // the copies land before the CTA moves on
-    mbar_wait_bounded(&bar_a, 0, pa::kDrainLimit);
-  }
-  if (tid == 0 && ok) {
-    tc_fence_after_sync();
-    const uint32_t idesc2 = tc_idesc_tf32(kTcRows, 2 * kOtCols), idesc1 = tc_idesc_tf32(kTcRows, kOtCols);
-    const uint32_t a_hi = smem_u32(A), a_lo = smem_u32(A + (size_t)kTcRows * Kp), b = smem_u32(B);
-    const uint32_t sbo = (uint32_t)(Kp / 4) * 128;  // next 8-row group
-    for (int ks = 0; ks < Kp / 8; ++ks) {
-      const uint32_t ko = (uint32_t)ks * 256;  // two core matrices along K per step
-      tc_mma_tf32(taddr, tc_smem_desc(a_hi + ko, 128, sbo), tc_smem_desc(b + ko, 128, sbo), idesc2,
-                  ks > 0 ? 1u : 0u);
-      tc_mma_tf32(taddr, tc_smem_desc(a_lo + ko, 128, sbo), tc_smem_desc(b + ko, 128, sbo), idesc1, 1u);
-    }
-    tc_commit(&bar_mma);
-  }
-  if (ok && !__syncthreads_and(mbar_wait_bounded(&bar_mma, 0, pa::kWaitLimit))) {
-    if (tid == 0) atomicCAS(status, 0, pa::kDevTimeout);
-    mbar_wait_bounded(&bar_mma, 0, pa::kDrainLimit);  // the MMAs finish before TMEM is freed
-    ok = false;
-  }
-  tc_fence_after_sync();
-  const bool live = row < nr;
-  const float ac = live ? rcoef[2 * (r0 + row)] : 0.f, acs = live ? rcoef[2 * (r0 + row) + 1] : 0.f;
-  float* er = eps + (int64_t)(r0 + row) * D + cb0;
-  const uint32_t tl = taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(half * (kOtCols / 2));
-#pragma unroll
-  for (int cb = 0; cb < kOtCols / 2; cb += 16) {
-    float v[16], w[16];
-    if (ok) {  // uniform across the CTA: every lane of the warp takes part in the loads
-      tmem_ld16(tl + (uint32_t)cb, v);
-      tmem_ld16(tl + (uint32_t)(kOtCols + cb), w);
-    }
-    if (!live) continue;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const float4 x = xv[cb / 4 + g];
-      float4 o;
-      if (ok && !dots_bad) {
-        o = make_float4(ac * x.x - acs * (v[4 * g] + w[4 * g]), ac * x.y - acs * (v[4 * g + 1] + w[4 * g + 1]),
-                        ac * x.z - acs * (v[4 * g + 2] + w[4 * g + 2]), ac * x.w - acs * (v[4 * g + 3] + w[4 * g + 3]));
-      } else {  // a bounded wait ran out here or before: the tile shows it
-        const float nan = __int_as_float(0x7fc00000);
-        o = make_float4(nan, nan, nan, nan);
-      }
-      *reinterpret_cast<float4*>(er + cb + 4 * g) = o;
-    }
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(taddr, kTmemCols);
-}
-
-// ---------------------------------------------------------------------------
 // Single-kernel form for up to 16 components (form 2): a thread-block cluster
 // of CL CTAs takes a block of RB rows; CTA q of the cluster owns columns
 // [q * chunk, (q + 1) * chunk) with chunk = D / CL. Each CTA stages its chunk of
@@ -1213,17 +737,24 @@ struct pa_gmm {
   GmmLayout L;
   cudaStream_t st;
   int64_t launches;
-  bool tc_ok;   // the tensor-core dot products fit this device and these sizes
-  bool use_tc;  // ... and are selected
+  bool per;     // the tensor-core kernels fit this device
+  bool tc_ok;   // ... and pa_gmm_set_form gives them for these sizes and means
   bool cl_ok;   // the single-kernel cluster form fits these sizes and this device
-  bool per;     // form 1 is the persistent kernels
-  bool ot_ok;   // form 1 also takes the output contraction on the tensor cores (16 < K <= 64)
-  int form;     // 0 CUDA-core dots + output kernel, 1 tensor-core dots + output kernel, 2 cluster form
+  int form;     // 0 CUDA cores, 1 tensor cores, 2 cluster form
 };
 
 namespace {
 constexpr int kClSize = 16;   // CTAs per cluster (non-portable size, opted into)
 constexpr int kClRows = 8;    // rows per cluster
+
+// See the constants above. (`rows16`: the means' rows start on 16-byte boundaries.)
+int default_form(const pa_gmm& g, bool rows16) {
+  const double work = (double)g.K * (double)g.D * g.max_rows;
+  if (g.K > kClMaxK) return g.per && work >= (g.K > 64 ? kTcWideWork : kTcWork) ? 1 : 0;
+  if (!g.cl_ok) return g.per && rows16 && g.K >= kTcFewMinK && work >= kTcFewWork0 ? 1 : 0;
+  if (g.max_rows >= kManyRows && g.D <= kShortRow && g.D <= kShortPerRow * g.max_rows) return 0;
+  return g.per && g.max_rows >= kTcFewRows && work >= kTcFewWork ? 1 : 2;
+}
 }  // namespace
 
 extern "C" size_t pa_gmm_workspace_bytes(int K, int64_t D, int max_rows, int T) {
@@ -1281,57 +812,19 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
     e = cudaFuncSetAttribute(k_gmm_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_gmm_out, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out_smem);
-  // tensor-core dot products: sm_100-family tensor cores, 16-byte rows, and
-  // shared memory for the split rows and the means image of one chunk
   int dev = 0, major = 0, optin = 0;
-  g->tc_ok = false;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const bool rows16 = D % 4 == 0 && (reinterpret_cast<uintptr_t>(means_dev) & 15) == 0;
   g->per = false;
-  if (e == cudaSuccess && tc_persistent(K, D, max_rows)) {
-    e = pa::gmm_tc_setup(K, &g->per);
-    g->tc_ok = g->per;
-  } else if (e == cudaSuccess && major == 10 && D % 4 == 0 && (reinterpret_cast<uintptr_t>(means_dev) & 15) == 0 &&
-      tc_smem_bytes(K) + 2048 <= (size_t)optin) {
-    e = cudaFuncSetAttribute(k_gmm_dots_tc<kTcCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tc_smem_bytes(K));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_gmm_dots_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(K));
-    if (e == cudaSuccess) {
-      k_gmm_mu_image<<<L.tc_chunks, 256, 0, g->st>>>(means_dev, K, D, reinterpret_cast<float*>(g->ws + L.mu_img));
-      g->launches++;
-      e = cudaGetLastError();
-      g->tc_ok = e == cudaSuccess;
-    }
-  }
-  // The tensor-core output contraction beside them: 16 < K <= 64 (padded
-  // components fit one image of 128 rows x 64), whole kOtCols-column chunks.
-  g->ot_ok = false;
-  if (e == cudaSuccess && g->tc_ok && !g->per && K > kTcMinK && tc_npad(K) <= kOtMaxKp && D % kOtCols == 0 &&
-      ot_smem_bytes(K) + 4096 <= (size_t)optin) {
-    e = cudaFuncSetAttribute(k_gmm_out_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ot_smem_bytes(K));
-    if (e == cudaSuccess) {
-      k_gmm_mut_image<<<(unsigned)(D / kOtCols), 256, 0, g->st>>>(means_dev, K, D,
-                                                                    reinterpret_cast<float*>(g->ws + L.mut_img));
-      g->launches++;
-      e = cudaGetLastError();
-      g->ot_ok = e == cudaSuccess;
-    }
-  }
-  // Default: the tensor cores for K > 16. At K <= 16 the contraction is under
-  // a microsecond of CUDA-core FMA work per call and the CUDA-core kernel's
-  // shorter per-CTA chain wins (measured at 4x64x64: 30.1 vs 33.1 us per
-  // Picard iteration); at K = 64 the tensor cores win (151.9 vs 170.4 us at
-  // 4x128x128).
-  g->use_tc = g->tc_ok && (K > kTcMinK || g->per);
+  if (e == cudaSuccess) e = pa::gmm_tc_setup(K, &g->per);
+  g->tc_ok = g->per && rows16;
   // The single-kernel cluster form for K <= 16 when D splits into kClSize
   // 16-byte-aligned column chunks whose tiles fit in shared memory and a
-  // cluster of kClSize CTAs can be resident; then the default.
+  // cluster of kClSize CTAs can be resident.
   g->cl_ok = false;
-  g->form = g->use_tc ? 1 : 0;
-  if (e == cudaSuccess && major == 10 && K <= kClMaxK && D % (4 * kClSize) == 0 &&
-      (reinterpret_cast<uintptr_t>(means_dev) & 15) == 0) {
+  if (e == cudaSuccess && major == 10 && K <= kClMaxK && D % (4 * kClSize) == 0 && rows16) {
     const int chunk = (int)(D / kClSize);
     const size_t smem = ClShape<kClSize, kClRows>::smem_bytes(chunk, T);
     auto kern = k_gmm_cluster<kClSize, kClRows>;
@@ -1356,13 +849,13 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
         e = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg);
         g->cl_ok = e == cudaSuccess && nclusters > 0;
         if (e != cudaSuccess) {
-          (void)cudaGetLastError();  // the size is not supported here: keep the two-kernel forms
+          (void)cudaGetLastError();  // the size is not supported here: keep the other forms
           e = cudaSuccess;
         }
       }
     }
-    if (g->cl_ok && !g->use_tc) g->form = 2;
   }
+  g->form = default_form(*g, rows16);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);
   if (e != cudaSuccess) {
     pa::set_error(std::string("pa_gmm_create: ") + cudaGetErrorString(e));
@@ -1390,9 +883,8 @@ extern "C" pa_status pa_gmm_eps(pa_gmm* g, const float* batch_x_dev, const int32
                                        reinterpret_cast<uintptr_t>(g->means)) & 15) == 0;
   const bool vec_out = g->D % 4 == 0 && (reinterpret_cast<uintptr_t>(batch_eps_dev) & 15) == 0;
   const size_t out_smem = (size_t)(g->K + kOutRows) * kOutCols * sizeof(float);
-  const dim3 tc_grid(L.tc_chunks, (g->max_rows + kTcRows - 1) / kTcRows);
   cudaError_t e;
-  if (g->form == 1 && g->per) {  // any D, any alignment
+  if (g->form == 1) {  // any D, any alignment
     const pa::GmmTcArgs a{batch_x_dev, g->means, coef, mnorm, miss_bt_dev, n_rows_dev, batch_eps_dev, g->ws + L.tc,
                           status, g->K, g->T, g->max_rows, g->D};
     e = pa::gmm_tc_launch(a, g->st);
@@ -1418,38 +910,9 @@ extern "C" pa_status pa_gmm_eps(pa_gmm* g, const float* batch_x_dev, const int32
     }
     return PA_OK;
   }
-  if (g->use_tc && bulk && L.tc_chunks >= kTcClusterMinChunks)
-    e = pa::launch_ex(k_gmm_dots_tc<kTcCluster>, tc_grid, dim3(kTcThreads), tc_smem_bytes(g->K), g->st,
-                      kTcCluster, batch_x_dev, (const float*)(g->ws + L.mu_img), n_rows_dev, g->K, g->D,
-                      g->max_rows, gacc2, ep, status);
-  else if (g->use_tc && bulk)
-    e = pa::launch_ex(k_gmm_dots_tc<1>, tc_grid, dim3(kTcThreads), tc_smem_bytes(g->K), g->st, 0, batch_x_dev,
-                      (const float*)(g->ws + L.mu_img), n_rows_dev, g->K, g->D, g->max_rows, gacc2, ep, status);
-  else
-    e = pa::launch_ex(k_gmm_dots, dim3(L.nchunk, (g->max_rows + kDotRows - 1) / kDotRows), dim3(kThreads),
-                      dots_smem_bytes(g->K, L.chunk), g->st, 0, batch_x_dev, g->means, n_rows_dev, g->K, g->D,
-                      L.chunk, L.nchunk, g->max_rows, bulk, gacc2, ep, status);
-  if (g->use_tc && g->ot_ok && bulk && vec_out) {  // responsibilities, then the contraction on the tensor cores
-    const int blocks = (g->max_rows + kTcRows - 1) / kTcRows;
-    float* rimg = reinterpret_cast<float*>(g->ws + L.r_img);
-    float* rcoef = reinterpret_cast<float*>(g->ws + L.rcoef);
-    if (e == cudaSuccess)
-      e = pa::launch_ex(k_gmm_resp, dim3(blocks * (kTcRows / kRespRows)), dim3(kRespRows * 32), 0, g->st, 0,
-                        (const long long*)gacc2, ep, coef, g->T, miss_bt_dev, mnorm, n_rows_dev, g->K, g->max_rows,
-                        rimg, rcoef);
-    if (e == cudaSuccess)
-      e = pa::launch_ex(k_gmm_out_tc, dim3((unsigned)(g->D / kOtCols), blocks), dim3(kOtThreads),
-                        ot_smem_bytes(g->K), g->st, 0, batch_x_dev, (const float*)(g->ws + L.mut_img),
-                        (const float*)rimg, (const float*)rcoef, n_rows_dev, g->K, g->D, g->max_rows,
-                        batch_eps_dev, status);
-    g->launches += 3;
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      pa::set_error(std::string("pa_gmm_eps: ") + cudaGetErrorString(e));
-      return PA_ERR_CUDA;
-    }
-    return PA_OK;
-  }
+  e = pa::launch_ex(k_gmm_dots, dim3(L.nchunk, (g->max_rows + kDotRows - 1) / kDotRows), dim3(kThreads),
+                    dots_smem_bytes(g->K, L.chunk), g->st, 0, batch_x_dev, g->means, n_rows_dev, g->K, g->D,
+                    L.chunk, L.nchunk, g->max_rows, bulk, gacc2, ep, status);
   if (e == cudaSuccess)
     e = pa::launch_ex(k_gmm_out,
                       dim3((unsigned)((g->D + kOutCols - 1) / kOutCols), (g->max_rows + kOutRows - 1) / kOutRows),
@@ -1484,7 +947,7 @@ extern "C" pa_status pa_gmm_set_form(pa_gmm* g, int form) {
   if (!g) { pa::set_error("pa_gmm_set_form: NULL handle"); return PA_ERR_ARG; }
   if (form < 0 || form > 2) { pa::set_error("pa_gmm_set_form: form must be 0, 1 or 2"); return PA_ERR_ARG; }
   if (form == 1 && !g->tc_ok) {
-    pa::set_error("pa_gmm_set_form: tensor-core dot products need an sm_100-family GPU, D % 4 == 0, "
+    pa::set_error("pa_gmm_set_form: the tensor-core form needs an sm_100-family GPU, D % 4 == 0, "
                   "16-byte aligned means and enough shared memory");
     return PA_ERR_ARG;
   }
@@ -1493,7 +956,6 @@ extern "C" pa_status pa_gmm_set_form(pa_gmm* g, int form) {
                   "16-byte aligned means and enough shared memory");
     return PA_ERR_ARG;
   }
-  g->use_tc = form == 1;
   g->form = form;
   return PA_OK;
 }

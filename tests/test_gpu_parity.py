@@ -304,10 +304,10 @@ def test_gmm_kernel_against_oracle(wname, n, max_rows, form):
     (64, 16400, 100, 128, 1),                              # rows 4 bytes past a 16-byte boundary
     (16, 4096, 1500, 1600, 0), (5, 9000, 800, 800, 0),     # few components, many rows
     (128, 64, 19590, 19600, 0),                            # more row blocks than CTAs
+    (18, 1024, 7, 8, 0), (1, 64, 3, 3, 0),                 # fewer pieces than CTAs
     (100, 3000, 0, 256, 0)])                               # no rows
 def test_gmm_persistent_kernels(K, D, n, cap, shift):
-    """The persistent tensor-core denoiser (form 1 of a large problem) against
-    the fp64 oracle at the edges of its row blocks, column units and tiles,
+    """The persistent tensor-core denoiser (form 1) against the fp64 oracle at the edges of its row blocks, column units and tiles,
     twice in a row with bitwise equal results; rows past the count stay as
     they were. Tolerance as for the other forms."""
     import torch
@@ -316,7 +316,8 @@ def test_gmm_persistent_kernels(K, D, n, cap, shift):
     a, mu, idx, x, miss = _gmm_rows(w, max(n, 1))
     dev = torch.device("cuda")
     g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
-    assert g.form() == 1
+    if g.form() != 1:
+        g.set_form(1)
     l0 = g.launches()
     xd = torch.zeros(cap * D + shift, dtype=torch.float32, device=dev)[shift:].view(cap, D)
     xd[:n] = torch.from_numpy(x[:n]).to(dev)
@@ -368,6 +369,34 @@ def test_gmm_cuda_core_form(K, D, n, cap, shift):
     rel = np.abs(out[:n].cpu().numpy() - want).max(axis=1) / np.abs(want).max(axis=1)
     assert rel.max() <= 2e-6, rel.max()
     assert torch.isnan(out[n:]).all()
+    g.close()
+
+
+@pytest.mark.parametrize("K,D,cap,form", [
+    (17, 16384, 143, 0), (17, 16384, 144, 1), (32, 3001, 500, 1), (32, 3001, 400, 0),  # K D cap = 40e6
+    (65, 1024, 180, 0), (65, 1024, 181, 1),                                              # 12e6
+    (16, 8192, 327, 2), (16, 8192, 328, 0), (2, 64, 199, 2), (2, 64, 200, 0), (3, 10048, 500, 2),  # many short rows
+    (16, 16384, 953, 2), (16, 16384, 954, 1), (16, 32768, 511, 2),                       # 250e6, and 512 rows
+    (9, 16388, 700, 1), (9, 16388, 670, 0), (8, 16388, 800, 0), (9, 16387, 700, 0)])     # no cluster form: 100e6
+def test_gmm_default_form(K, D, cap, form):
+    """The form by sizes on both sides of each line, against the fp64 oracle
+    on one row in eight; tolerance as for the forms."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    n = cap // 8
+    w = W.SD15.with_(K=K, latent_shape=(1, 1, D))
+    a, mu, idx, x, miss = _gmm_rows(w, n)
+    dev = torch.device("cuda")
+    g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
+    assert g.form() == form
+    xd = torch.from_numpy(x).to(dev)
+    md = torch.from_numpy(miss).to(dev)
+    nd = torch.tensor([n], dtype=torch.int32, device=dev)
+    out = torch.full((cap, D), float("nan"), device=dev)
+    g.eps(xd.data_ptr(), md.data_ptr(), nd.data_ptr(), out)
+    want = gmm_eps(x.astype(np.float64), a[idx], mu.astype(np.float64), w.gmm_std)
+    rel = np.abs(out[:n].cpu().numpy() - want).max(axis=1) / np.abs(want).max(axis=1)
+    assert rel.max() <= 2e-6, rel.max()
     g.close()
 
 
