@@ -477,15 +477,18 @@ __global__ void __launch_bounds__(kThreads) k_gmm_out(const float* __restrict__ 
 constexpr int kClThreads = 256;
 constexpr int kClMaxK = 16;
 
-constexpr int kClCoefT = 2048;  // per-timestep scalars staged in shared memory up to this many timesteps
+// Per-timestep scalars are staged in shared memory where that is one load per
+// thread: a short generation's call saves a round trip (T 16 at 4x8x8, 0.7 us per
+// generation). A longer schedule's would not have landed when the rows do, 12 KB
+// per CTA at T 1000; there a row's three scalars are fetched while the rows are
+// on their way (a 1000-step generation of 4x64x64 with draws: 725 us with all of
+// them staged before the means, 643 so; T 100, eight trajectories, 239 / 237).
+constexpr int kClCoefT = kClThreads / 3;
 
 template <int CL, int RB>
 struct ClShape {
   static int ld(int chunk) { return chunk + 4; }  // padded row stride: the two half-warps' rows on other banks
-  static size_t coef_bytes(int T) { return T <= kClCoefT ? (size_t)3 * T * sizeof(float) : 0; }
-  static size_t smem_bytes(int chunk, int T) {
-    return (size_t)(kClMaxK + RB) * ld(chunk) * sizeof(float) + coef_bytes(T);
-  }
+  static size_t smem_bytes(int chunk) { return (size_t)(kClMaxK + RB) * ld(chunk) * sizeof(float); }
 };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -524,6 +527,7 @@ __global__ void __launch_bounds__(kClThreads, 2) k_gmm_cluster(const float* __re
   __shared__ float s_half[2][RB * kClMaxK];  // this CTA's partials from each half of its columns
   __shared__ __align__(16) float s_rt[kClMaxK * RB];  // responsibilities [k][row]
   __shared__ float s_sa[RB], s_q[RB], s_c[RB], s_cs[RB];
+  __shared__ float s_coef[3 * kClCoefT];
   __shared__ int s_bad;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -532,26 +536,30 @@ __global__ void __launch_bounds__(kClThreads, 2) k_gmm_cluster(const float* __re
   const int64_t c0 = (int64_t)rank * chunk;
   float* ms = reinterpret_cast<float*>(smem_raw);  // [kClMaxK][ld], rows >= K zero
   float* xs = ms + (size_t)kClMaxK * ld;           // [RB][ld]
-  float* s_coef = xs + (size_t)RB * ld;            // [3][T] when T <= kClCoefT
-  if (tid == 0) {
-    mbar_init(&bar_m, 1);
-    mbar_init(&bar_x, 1);
-    mbar_init(&bar_p, 1);
-    fence_barrier_init();
-    mbar_arrive_expect_tx(&bar_m, (uint32_t)chunk * sizeof(float) * (uint32_t)K);
-    // every CTA of the cluster stores its RB x kClMaxK partials here
-    mbar_arrive_expect_tx(&bar_p, (uint32_t)(CL * RB * kClMaxK * sizeof(float)));
-    s_bad = 0;
-  }
-  // ||mu_k||^2 of the component this thread takes in the softmax (constant)
+  // constants: ||mu_k||^2 of the component this thread takes in the softmax, and
+  // one of the staged scalars
   const float mn = (tid < RB * kClMaxK && (tid & (kClMaxK - 1)) < K) ? mnorm[tid & (kClMaxK - 1)] : 0.f;
-  for (int q = tid; q < (kClMaxK - K) * ld; q += kClThreads) ms[(size_t)K * ld + q] = 0.f;
-  const bool coef_staged = T <= kClCoefT;  // constants: staged before the dependency wait
-  if (coef_staged)
-    for (int q = tid; q < 3 * T; q += kClThreads) s_coef[q] = coef[q];
-  __syncthreads();
-  if (warp == 0)  // the means do not depend on the predecessor
+  const bool coef_staged = T <= kClCoefT;
+  const float cv = coef_staged && tid < 3 * T ? coef[tid] : 0.f;
+  // the means early: they do not depend on the predecessor, and how early they
+  // are asked for is what the dependency wait can hide of them
+  if (warp == 0) {
+    if (lane == 0) {
+      mbar_init(&bar_m, 1);
+      mbar_init(&bar_x, 1);
+      mbar_init(&bar_p, 1);
+      fence_barrier_init();
+      mbar_arrive_expect_tx(&bar_m, (uint32_t)chunk * sizeof(float) * (uint32_t)K);
+      // every CTA of the cluster stores its RB x kClMaxK partials here
+      mbar_arrive_expect_tx(&bar_p, (uint32_t)(CL * RB * kClMaxK * sizeof(float)));
+      s_bad = 0;
+    }
+    __syncwarp();
     for (int k = lane; k < K; k += 32) bulk_g2s(ms + (size_t)k * ld, mu + (int64_t)k * D + c0, chunk * 4u, &bar_m);
+  }
+  for (int q = tid; q < (kClMaxK - K) * ld; q += kClThreads) ms[(size_t)K * ld + q] = 0.f;
+  if (coef_staged && tid < 3 * T) s_coef[tid] = cv;
+  __syncthreads();
   pdl_wait();     // the rows, their count and their timesteps come from the kernel just before
   pdl_trigger();  // the successor may now run its prologue
   const int n_rows = min(*n_rows_dev, max_rows);
@@ -573,10 +581,11 @@ __global__ void __launch_bounds__(kClThreads, 2) k_gmm_cluster(const float* __re
   if (tid < nr) {
     const int i = miss_bt[2 * (r0 + tid) + 1];
     const float* cf = coef_staged ? s_coef : coef;
-    s_sa[tid] = cf[i];
-    s_q[tid] = cf[T + i];
-    s_c[tid] = cf[2 * T + i];
-    s_cs[tid] = cf[2 * T + i] * cf[i];
+    const float sa = cf[i], q = cf[T + i], c = cf[2 * T + i];
+    s_sa[tid] = sa;
+    s_q[tid] = q;
+    s_c[tid] = c;
+    s_cs[tid] = c * sa;
   }
   // bounded waits; a CTA whose copies did not land keeps to the cluster's
   // barriers (its peers wait for it there) and writes NaN
@@ -826,7 +835,7 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   g->cl_ok = false;
   if (e == cudaSuccess && major == 10 && K <= kClMaxK && D % (4 * kClSize) == 0 && rows16) {
     const int chunk = (int)(D / kClSize);
-    const size_t smem = ClShape<kClSize, kClRows>::smem_bytes(chunk, T);
+    const size_t smem = ClShape<kClSize, kClRows>::smem_bytes(chunk);
     auto kern = k_gmm_cluster<kClSize, kClRows>;
     cudaFuncAttributes fa = {};
     e = cudaFuncGetAttributes(&fa, kern);
@@ -899,7 +908,7 @@ extern "C" pa_status pa_gmm_eps(pa_gmm* g, const float* batch_x_dev, const int32
   if (g->form == 2 && bulk && vec_out) {  // one kernel: cluster of kClSize CTAs per kClRows rows
     const int chunk = (int)(g->D / kClSize);
     e = pa::launch_ex(k_gmm_cluster<kClSize, kClRows>, dim3(kClSize, (g->max_rows + kClRows - 1) / kClRows),
-                      dim3(kClThreads), ClShape<kClSize, kClRows>::smem_bytes(chunk, g->T), g->st, kClSize,
+                      dim3(kClThreads), ClShape<kClSize, kClRows>::smem_bytes(chunk), g->st, kClSize,
                       batch_x_dev, g->means, coef, g->T, miss_bt_dev, mnorm, n_rows_dev, g->K, g->D, chunk,
                       g->max_rows, batch_eps_dev, status);
     g->launches += 1;
