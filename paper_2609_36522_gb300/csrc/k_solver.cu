@@ -367,11 +367,11 @@ static_assert(kPlanThreads == kGatherThreads, "report_sums");
 constexpr int kPlanPerSm = 2;   // planning CTAs per SM (three: the launch bound makes the decision spill, slower)
 constexpr int kFusedMaxPairs = 1024;  // B*P planned in every CTA at most; beyond, one CTA plans
 // Beyond this many pairs one CTA plans and a separate gather follows unless
-// tau_cache adapts (only the every-CTA planner forms the next tau): at the SD
-// latent with 800 and 1000 pairs that measured 49.9 and 59.8 us per solver
-// step against 51.7 and 62.8 us, at 300 and 400 pairs 28.6 and 34.9 against
-// 27.9 and 34.4 us
-constexpr int kFusedPreferPairs = 512;
+// tau_cache adapts (only the every-CTA planner forms the next tau). A generation
+// with every CTA planning against one: windows of 100 at 4x64x64 with 500, 600,
+// 800 and 1000 pairs 343 / 360, 401 / 413, 515 / 520 and 640 / 636 us, windows of
+// 32 at 4x32x32 with 640 pairs 239 / 257.
+constexpr int kFusedPreferPairs = 900;
 static_assert(kFusedMaxPairs <= 32 * 32, "one miss mask per 32-position chunk, a lane each");
 
 // The decision's inputs as bits in shared memory (one-CTA planner).

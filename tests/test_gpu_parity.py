@@ -98,9 +98,14 @@ def test_large_latent():
     # once and copies every gridDim.y-th row
     W.Workload("4 x 100 pairs", T=100, window=100, batch=4, latent_shape=(4, 8, 8), K=4,
                tol=1e-3, cache_thresh=0.05, seed=19),
-    # past 512 pairs one CTA plans and a separate gather follows
+    # past 900 pairs one CTA plans and a separate gather follows
     W.Workload("10 x 100 pairs", T=100, window=100, batch=10, latent_shape=(4, 8, 8), K=4,
                tol=1e-3, cache_thresh=0.05, seed=20),
+    # the most pairs that every CTA plans, and one more
+    W.Workload("9 x 100 pairs", T=100, window=100, batch=9, latent_shape=(4, 8, 8), K=4,
+               tol=1e-3, cache_thresh=0.05, seed=22),
+    W.Workload("17 x 53 pairs", T=60, window=53, batch=17, latent_shape=(4, 8, 8), K=4,
+               tol=1e-3, cache_thresh=0.05, seed=24),
     # more than 1024 (trajectory, position) pairs: one CTA plans, a separate gather follows
     W.Workload("9 x 128 pairs", T=200, window=128, batch=9, latent_shape=(4, 4, 4), K=4,
                tol=1e-3, cache_thresh=0.05, seed=13),
