@@ -119,8 +119,8 @@ PA_API pa_status pa_create(pa_solver** out, int T, int window,
  * takes effect from the next iteration (call pa_init to restart cleanly).
  * With draws the default update is the register-resident bulk form (or the
  * staged bulk form, which copies the draws into shared memory) when
- * D % 4 == 0 and the window fits; otherwise the plain-load kernel runs.
- * Synchronises the solver's stream. */
+ * D % 4 == 0, batch_eps is 16-byte aligned and the window fits; otherwise the
+ * plain-load kernel runs. Synchronises the solver's stream. */
 PA_API pa_status pa_set_noise(pa_solver* s, double eta, const float* noise_dev);
 
 /* Start a generation: x_init [batch][D] fp32, HOST or DEVICE pointer (the copy

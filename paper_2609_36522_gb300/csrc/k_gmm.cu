@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kThreads) k_gmm_out(const float* __restrict__ 
 // [q * chunk, (q + 1) * chunk) with chunk = D / CL. Each CTA stages its chunk of
 // the means (before the dependency wait: the means do not change) and of the
 // rows, forms the rows' partial dot products x . mu_k over its columns in
-// registers (4 rows x 4 components per warp, packed fp32 pairs, 16-byte
+// registers (4 rows x 8 components per warp, packed fp32 pairs, 16-byte
 // shared loads), and the CL partials are summed through distributed shared
 // memory in rank order -- the same sums in every CTA of the cluster. Every CTA then
 // takes the logits and the max-subtracted softmax of the block's rows and

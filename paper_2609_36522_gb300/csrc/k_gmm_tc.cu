@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
 // so that the number of CTAs costs no precision), logits, softmax, and the
 // row's two scalars for the output.
 constexpr int kRespThreads = 512;
-constexpr int kBatch = 20;       // partial sums in flight per thread: at 64 components 152 of them in two trips
+constexpr int kBatch = 20;       // partial sums in flight per thread: 152 of them at 64 components in one trip
 constexpr int kRespGrid = 4096;  // rows beyond it are taken in turn
 
 template <int KP>

@@ -9,8 +9,8 @@
 // sums added into the iteration's fp64 accumulators.
 //
 // Shaped for few instructions per element and many resident warps:
-//  - a CTA owns a strip of 128 columns (4 per lane, 16-byte loads) of one
-//    trajectory; its NW warps take contiguous runs of at most LMAX positions
+//  - a CTA owns a strip of 128 columns (4 per lane, 16-byte loads, or four
+//    4-byte ones where rows start on no 16-byte boundary) of one trajectory; its NW warps take contiguous runs of at most LMAX positions
 //    (two passes joined by one CTA barrier: run totals, then the carry and
 //    the new states);
 //  - the step coefficients of every timestep are staged in shared memory

@@ -60,8 +60,9 @@ struct pa_solver {
   pa::Ctl* host_ring;        // pinned: two more mirrors, one per pending pa_poll_begin
   cudaEvent_t poll_ev[2];    // recorded behind each pending poll's copies
   int poll_head, poll_count;  // the oldest pending poll's mirror, polls pending
-  // the device-driven generation loop (pa_loop_*): a graph [clear the pass
-  // counter] -> [WHILE node; body: two iterations and the loop test]
+  // the device-driven generation loop (pa_loop_*): a graph of a WHILE node whose
+  // body holds the captured iterations; the last one's planning kernel sets the
+  // condition (a test kernel behind it where planning takes more than one launch)
   cudaGraph_t loop_graph;
   cudaGraphExec_t loop_exec;
   cudaGraphConditionalHandle loop_cond;

@@ -390,7 +390,8 @@ class GmmDenoiser:
         return abi.pa_gmm_launches(self.h)
 
     def set_form(self, form):
-        """1: dot products on the tensor cores; 0: on the CUDA cores."""
+        """2: one kernel on thread-block clusters; 1: on the tensor cores; 0: on
+        the CUDA cores."""
         abi.pa_gmm_set_form(self.h, form)
 
     def form(self):
