@@ -64,7 +64,7 @@ constexpr int kDotRows = 16;     // rows per dots CTA (two per warp)
 constexpr int kOutRows = 16;     // rows per output CTA
 constexpr int kOutCols = 256;    // columns per output CTA (four per thread)
 constexpr size_t kDotSmemBudget = 96 * 1024;
-constexpr int kDotCtas = 120;    // CTAs that a dots launch should have (of 152 SMs)
+constexpr int kDotCtas = 480;    // CTAs that a dots launch should have: about three per SM
 constexpr float kDotScale = 4294967296.f;  // 2^32: fixed-point scale of the dot-product accumulators
 
 // Default form by sizes (pa_gmm_create). K components, D columns, a capacity of R
@@ -123,8 +123,11 @@ int dots_chunk(int K, int64_t D, int max_rows) {
   int c = 512;
   while (c > 64 && (size_t)(kDotRows + K) * (c + 4) * sizeof(float) > kDotSmemBudget) c /= 2;
   while (c > 64 && (int64_t)c >= 2 * D) c /= 2;
-  // down to 128 while the chunks leave SMs without a CTA (48 rows of 5883
-  // columns: 36 CTAs of 512, 138 of 128)
+  // down to 128 while the launch has fewer CTAs than the SMs hold at a time, whose
+  // copies and sums then overlap. A generation with 60, 120, 240 and 480 in place
+  // of kDotCtas: 12810 columns, 50 rows, 16 components 110.8, 107.3, 102.7, 102.6
+  // us; 3600 columns, 144 rows, 30 components 129, 127.5, 122.3, 122.2; 13860
+  // columns, 150 rows, 12 components 152.0, 151.8, 152.0, 149.8
   const int64_t blocks = (max_rows + kDotRows - 1) / kDotRows;
   while (c > 128 && (D + c - 1) / c * blocks < kDotCtas) c /= 2;
   return c;

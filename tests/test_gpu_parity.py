@@ -352,7 +352,7 @@ def test_gmm_persistent_kernels(K, D, n, cap, shift):
 @pytest.mark.parametrize("K,D,n,cap,shift", [
     (8, 5883, 48, 48, 0), (8, 129, 5, 8, 0), (3, 513, 33, 40, 0),   # rows on no 16-byte boundary: 4-byte copies
     (16, 1001, 1, 16, 0), (40, 127, 17, 40, 0), (8, 1, 3, 4, 0),
-    (8, 4096, 30, 48, 1), (8, 2048, 640, 640, 0), (8, 2048, 100, 160, 0)])  # chunks of 512 and of 128 columns
+    (8, 4096, 30, 48, 1), (8, 8192, 640, 640, 0), (8, 2048, 100, 160, 0)])  # chunks of 512 and of 128 columns
 def test_gmm_cuda_core_form(K, D, n, cap, shift):
     """The CUDA-core denoiser (form 0) against the fp64 oracle over its column
     chunks and both ways of staging rows; tolerance as for the other forms."""
