@@ -21,9 +21,9 @@
 //                  thread)
 // The accumulators come in two sets used in turn. A call's dot-product kernel
 // reads the handle's epoch e, accumulates into set e mod 2, clears the other
-// set (read by the previous call's output kernel, which has completed) and
-// records e for the output kernel; the output kernel reads set e mod 2 and
-// advances the epoch. No kernel waits for another CTA, and the state lives on
+// set (read by the previous call's output kernel, complete behind the dependency
+// wait) and records e for the output kernel; the output kernel reads set e mod 2
+// and advances the epoch. No kernel waits for another CTA, and the state lives on
 // the device, so a captured CUDA graph replays correctly.
 // Per-timestep scalars (sqrt(a), 1/(2v), sqrt(1-a)/v) are computed on the
 // host in fp64 from alpha-bar and stored in fp32, so 1 - a never cancels in
@@ -212,11 +212,12 @@ __device__ __forceinline__ bool wait_staged(bool bulk, uint64_t* bar, int32_t* s
   return false;
 }
 
-// Start of a dot-product kernel: the accumulator set of this call (epoch e),
-// the other set cleared by all CTAs together (every CTA, also those without
-// rows), and e recorded for the output kernel.
-__device__ __forceinline__ long long* begin_dots(long long* gacc2, GmmEpoch* ep, int64_t set_size) {
-  const uint32_t e = ep->epoch;  // advanced by the previous call's output kernel, long finished
+// The accumulator set of a dot-product kernel whose call has epoch e; all CTAs
+// together (every CTA, also those without rows) clear the other set, and e is
+// recorded for the output kernel. Only behind the dependency wait: the previous
+// call's output kernel, which reads the other set and advances the epoch, may be
+// the kernel just before.
+__device__ __forceinline__ long long* begin_dots(long long* gacc2, GmmEpoch* ep, uint32_t e, int64_t set_size) {
   long long* other = gacc2 + (int64_t)((e + 1u) & 1u) * set_size;
   const int64_t cta = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
   const int64_t nthr = (int64_t)gridDim.x * gridDim.y * blockDim.x;
@@ -238,7 +239,6 @@ __global__ void __launch_bounds__(kThreads) k_gmm_dots(const float* __restrict__
                                                        GmmEpoch* ep, int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar_m, bar_x;
-  long long* gacc = begin_dots(gacc2, ep, (int64_t)max_rows * K);
   const int r0 = blockIdx.y * kDotRows;
   const int64_t c0 = (int64_t)blockIdx.x * chunk;
   const int ncol = (int)(((D - c0) < chunk) ? (D - c0) : chunk);
@@ -257,8 +257,10 @@ __global__ void __launch_bounds__(kThreads) k_gmm_dots(const float* __restrict__
   pdl_wait();  // the rows and their count come from the kernel just before
   pdl_trigger();  // the successor may now run its prologue
   const int n_rows = min(*n_rows_dev, max_rows);
+  const uint32_t epoch = ep->epoch;
   const int nr = min(kDotRows, n_rows - r0);
   if (nr <= 0) {  // no rows for this CTA: the means copy lands before it exits
+    begin_dots(gacc2, ep, epoch, (int64_t)max_rows * K);
     wait_staged(bulk, &bar_m, status);
     return;
   }
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(kThreads) k_gmm_dots(const float* __restrict__
   if (tid == 0 && bulk) mbar_arrive_expect_tx(&bar_x, (uint32_t)ncol * sizeof(float) * (uint32_t)nr);
   __syncthreads();
   stage_rows(xs, ld, X + (int64_t)r0 * D, D, c0, ncol, nr, bulk, &bar_x);
+  long long* gacc = begin_dots(gacc2, ep, epoch, (int64_t)max_rows * K);  // while the rows are on their way
   const bool ok_m = wait_staged(bulk, &bar_m, status);
   const bool ok = wait_staged(bulk, &bar_x, status) && ok_m;
   __syncthreads();

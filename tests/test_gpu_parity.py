@@ -329,11 +329,9 @@ def test_gmm_persistent_kernels(K, D, n, cap, shift):
     md = torch.zeros(cap, 2, dtype=torch.int32, device=dev)
     md[:n] = torch.from_numpy(miss[:n]).to(dev)
     nd = torch.tensor([n], dtype=torch.int32, device=dev)
-    outs = []
-    for _ in range(2):
-        out = torch.full((cap * D + shift,), float("nan"), device=dev)[shift:].view(cap, D)
+    outs = [torch.full((cap * D + shift,), float("nan"), device=dev)[shift:].view(cap, D) for _ in range(2)]
+    for out in outs:  # nothing between the two calls
         g.eps(xd.data_ptr(), md.data_ptr(), nd.data_ptr(), out)
-        outs.append(out)
     assert g.launches() - l0 == 6
     torch.cuda.synchronize()
     from paper_2609_36522_gb300 import abi
@@ -374,6 +372,48 @@ def test_gmm_cuda_core_form(K, D, n, cap, shift):
     rel = np.abs(out[:n].cpu().numpy() - want).max(axis=1) / np.abs(want).max(axis=1)
     assert rel.max() <= 2e-6, rel.max()
     assert torch.isnan(out[n:]).all()
+    g.close()
+
+
+@pytest.mark.parametrize("form,K,D,cap", [
+    (0, 8, 4096, 256), (0, 16, 129, 300), (0, 40, 1000, 33), (1, 20, 4096, 200), (2, 16, 4096, 256)])
+def test_gmm_calls_back_to_back(form, K, D, cap):
+    """Calls of one handle with nothing between them, on two batches of other
+    counts in turn, each bitwise equal to the same call by itself: the next
+    call's first kernel starts before the last call's last one has ended."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    w = W.SD15.with_(K=K, latent_shape=(1, 1, D))
+    a, mu, idx, x, miss = _gmm_rows(w, cap)
+    dev = torch.device("cuda")
+    g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
+    g.set_form(form)
+    batches = []
+    for n, order in ((cap, slice(None)), (cap - cap // 3, slice(None, None, -1))):
+        xd = torch.zeros(cap, D, device=dev)
+        md = torch.zeros(cap, 2, dtype=torch.int32, device=dev)
+        xd[:n] = torch.from_numpy(x[order][:n].copy()).to(dev)
+        md[:n] = torch.from_numpy(miss[order][:n].copy()).to(dev)
+        batches.append((xd, md, torch.tensor([n], dtype=torch.int32, device=dev), n))
+
+    def call(batch, out):
+        g.eps(batch[0].data_ptr(), batch[1].data_ptr(), batch[2].data_ptr(), out)
+
+    alone = []
+    for batch in batches:
+        out = torch.empty(cap, D, device=dev)
+        torch.cuda.synchronize()
+        call(batch, out)
+        torch.cuda.synchronize()
+        alone.append(out)
+    outs = [torch.empty(cap, D, device=dev) for _ in range(12)]
+    torch.cuda.synchronize()
+    for c, out in enumerate(outs):
+        call(batches[c & 1], out)
+    torch.cuda.synchronize()
+    for c, out in enumerate(outs):
+        n = batches[c & 1][3]
+        assert torch.equal(out[:n], alone[c & 1][:n]), c
     g.close()
 
 
