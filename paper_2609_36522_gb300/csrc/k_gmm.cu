@@ -823,10 +823,8 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   }
   const size_t dots_smem = dots_smem_bytes(K, L.chunk);
   const size_t out_smem = (size_t)(K + kOutRows) * kOutCols * sizeof(float);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gmm_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gmm_out, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out_smem);
+  if (e == cudaSuccess) e = pa::allow_smem(reinterpret_cast<const void*>(k_gmm_dots), dots_smem);
+  if (e == cudaSuccess) e = pa::allow_smem(reinterpret_cast<const void*>(k_gmm_out), out_smem);
   int dev = 0, major = 0, optin = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
@@ -846,7 +844,7 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
     cudaFuncAttributes fa = {};
     e = cudaFuncGetAttributes(&fa, kern);
     if (e == cudaSuccess && smem + fa.sharedSizeBytes <= (size_t)optin) {
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = pa::allow_smem(reinterpret_cast<const void*>(kern), smem);
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
@@ -1105,10 +1103,8 @@ extern "C" pa_status pa_gmm_eps_noalloc(const float* means_dev, int K, int64_t D
   if (e == cudaSuccess) e = cudaMemsetAsync(gacc2, 0, (size_t)2 * n_rows * K * sizeof(long long), st);
   const size_t dots_smem = dots_smem_bytes(K, chunk);
   const size_t out_smem = (size_t)(K + kOutRows) * kOutCols * sizeof(float);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gmm_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dots_smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gmm_out, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out_smem);
+  if (e == cudaSuccess) e = pa::allow_smem(reinterpret_cast<const void*>(k_gmm_dots), dots_smem);
+  if (e == cudaSuccess) e = pa::allow_smem(reinterpret_cast<const void*>(k_gmm_out), out_smem);
   if (e != cudaSuccess) {
     pa::set_error(std::string("pa_gmm_eps_noalloc: ") + cudaGetErrorString(e));
     return PA_ERR_CUDA;

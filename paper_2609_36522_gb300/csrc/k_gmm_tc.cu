@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) k_gmm_out_tc(const float* __res
 
 template <int KP>
 cudaError_t out_setup() {
-  return cudaFuncSetAttribute(k_gmm_out_tc<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OtShape<KP>::smem());
+  return allow_smem(reinterpret_cast<const void*>(k_gmm_out_tc<KP>), OtShape<KP>::smem());
 }
 
 // CTAs of the two large kernels: one per SM
@@ -825,8 +825,8 @@ cudaError_t gmm_tc_setup(int K, bool* ok) {
   if (major != 10 || OtShape<128>::smem() + 4096 > (size_t)optin || dt_smem(two) + 1024 > (size_t)optin) return e;
   auto dots = two ? k_gmm_dots_tc<true, true> : k_gmm_dots_tc<false, true>;
   auto dots1 = two ? k_gmm_dots_tc<true, false> : k_gmm_dots_tc<false, false>;
-  e = cudaFuncSetAttribute(dots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dt_smem(two));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dots1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dt_smem(two));
+  e = allow_smem(reinterpret_cast<const void*>(dots), dt_smem(two));
+  if (e == cudaSuccess) e = allow_smem(reinterpret_cast<const void*>(dots1), dt_smem(two));
   if (e == cudaSuccess) {
     const int KP = kpad(K);
     e = KP == 16 ? out_setup<16>() : KP == 32 ? out_setup<32>() : KP == 64 ? out_setup<64>() : out_setup<128>();

@@ -738,15 +738,9 @@ cudaError_t launch_seg(const Dev& d, const float* beps, int par, cudaStream_t st
   const int nstrip = (int)((d.D + Sh::SEG - 1) / Sh::SEG);
   const size_t smem = Sh::smem_bytes(d.P);
   auto kern = k_update_seg<V, NW, NOISE>;
-  static size_t configured[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static SmemGranted granted;
+  const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem, granted);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) configured[dev] = smem;
-  }
   return launch_ex(kern, dim3(nstrip, d.B, 1), dim3(NW * 32), smem, st, 0, d, beps, d.wait_limit, par);
 }
 
@@ -977,15 +971,9 @@ cudaError_t launch_reg(const Dev& d, const float* beps, int par, cudaStream_t st
   const int nstrip = (int)((d.D + Sh::SEG - 1) / Sh::SEG);
   const size_t smem = Sh::smem_bytes(d.P);
   auto kern = k_update_reg<V, NW, LMAX, NOISE, CB>;
-  static size_t configured[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static SmemGranted granted;
+  const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem, granted);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) configured[dev] = smem;
-  }
   return launch_ex(kern, dim3(nstrip, d.B, 1), dim3(NW * 32), smem, st, 0, d, beps, par);
 }
 
@@ -1032,16 +1020,9 @@ cudaError_t launch_tile(const Dev& d, const float* beps, int par, cudaStream_t s
   if (nbuf < 1) nbuf = 1;
   const size_t smem = Sh::smem_bytes(d.P, nbuf);
   auto kern = k_update_tile<V, NW, S, CLUSTER, WAIT_ALL>;
-  // largest dynamic shared memory granted so far, per device and instantiation
-  static size_t configured[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static SmemGranted granted;
+  const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem, granted);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) configured[dev] = smem;
-  }
   const int gx = CLUSTER ? (nstrip + kCluster - 1) / kCluster * kCluster : nstrip;
   return launch_ex(kern, dim3(gx, d.B, 1), dim3(NW * 32), smem, st, CLUSTER ? kCluster : 0, d, beps, nstrip,
                    nbuf, d.wait_limit, par);

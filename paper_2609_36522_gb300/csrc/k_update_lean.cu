@@ -525,15 +525,9 @@ cudaError_t launch_lean(const Dev& d, const float* beps, int par, cudaStream_t s
   const int nstrip = (int)((d.D + 127) / 128);
   const size_t smem = Sh::smem_bytes(d.T, d.P, COMP);
   auto kern = k_update_lean<NW, LMAX, MINB, NOISE, COMP, CB, FUSE, TAA, VEC>;
-  static size_t configured[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static SmemGranted granted;
+  const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem, granted);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) configured[dev] = smem;
-  }
   return launch_ex(kern, dim3(nstrip, d.B, 1), dim3(NW * 32), smem, st, 0, d, beps, par);
 }
 
@@ -555,20 +549,17 @@ cudaError_t launch_fused(const Dev& d, const float* beps, int par, cudaStream_t 
   const size_t smem = Sh::smem_bytes(d.T, d.P, COMP);
   if (smem > kLeanSmemMax) return cudaErrorNotSupported;
   auto kern = k_update_lean<NW, LMAX, MINB, NOISE, COMP, CB, true>;
-  // per device: the dynamic shared memory configured and the resident CTAs
-  // the whole GPU holds at that size
-  static size_t configured[64] = {};
+  // per device: the dynamic shared memory granted and the resident CTAs the
+  // whole GPU holds at a size
+  static SmemGranted granted;
   static size_t cap_smem[64] = {};
   static int capacity[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorNotSupported;
-  if (smem > configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured[dev] = smem;
-  }
+  e = allow_smem(reinterpret_cast<const void*>(kern), smem, granted);
+  if (e != cudaSuccess) return e;
   if (smem != cap_smem[dev]) {
     int per_sm = 0, nsm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);

@@ -2,6 +2,7 @@
 // kernels (k_solver.cu, k_update_bulk.cu). Not part of the public ABI.
 #pragma once
 
+#include <atomic>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -165,6 +166,17 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 
 bool on_current_device(const void* p);  // an address in the current device's memory (pa_solver.cpp)
 bool pdl_enabled();  // false when the environment sets PA_DISABLE_PDL=1
+
+// Let kernel `kern` take `bytes` of dynamic shared memory on the current device
+// (pa_solver.cpp). The limit belongs to the kernel, not to a handle: it is only
+// ever raised, whatever the handles and threads that share the kernel ask for.
+cudaError_t allow_smem(const void* kern, size_t bytes);
+// The same for a launch: asks once per device and larger size (`granted`: what
+// earlier launches were given, per device).
+struct SmemGranted {
+  std::atomic<size_t> on[64] = {};
+};
+cudaError_t allow_smem(const void* kern, size_t bytes, SmemGranted& granted);
 
 // cudaLaunchKernelEx with the PDL attribute (when enabled), an optional
 // cluster width along x (0 = no cluster attribute) and, with `coop`, the

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -27,6 +28,26 @@ bool on_current_device(const void* p) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
+cudaError_t allow_smem(const void* kern, size_t bytes) {
+  static std::mutex m;
+  const std::lock_guard<std::mutex> hold(m);
+  cudaFuncAttributes fa = {};
+  const cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+  if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+cudaError_t allow_smem(const void* kern, size_t bytes, SmemGranted& granted) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev >= 0 && dev < 64;
+  if (known && bytes <= granted.on[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+  e = allow_smem(kern, bytes);
+  if (e == cudaSuccess && known) granted.on[dev].store(bytes, std::memory_order_relaxed);
+  return e;
 }
 
 bool pdl_enabled() {

@@ -417,6 +417,50 @@ def test_gmm_calls_back_to_back(form, K, D, cap):
     g.close()
 
 
+@pytest.mark.parametrize("form,large,small", [
+    (0, (16, 12810, 640), (16, 12810, 50)),   # (K, D, capacity): a smaller capacity takes shorter chunks
+    (0, (100, 4096, 64), (3, 4096, 64)), (2, (16, 16384, 64), (16, 4096, 64))])
+def test_gmm_handles_share_kernels(form, large, small):
+    """A handle whose kernels need much shared memory works on when handles
+    and calls that need less have come after it: the limit is the kernel's."""
+    import torch
+    from paper_2609_36522_gb300 import abi
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    dev = torch.device("cuda")
+
+    def case(K, D, cap):
+        w = W.SD15.with_(K=K, latent_shape=(1, 1, D))
+        a, mu, idx, x, miss = _gmm_rows(w, 20)
+        g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
+        g.set_form(form)
+        xd = torch.zeros(cap, D, device=dev)
+        md = torch.zeros(cap, 2, dtype=torch.int32, device=dev)
+        xd[:20] = torch.from_numpy(x).to(dev)
+        md[:20] = torch.from_numpy(miss).to(dev)
+        return g, xd, md, torch.tensor([20], dtype=torch.int32, device=dev), w, list(a), mu, idx, x
+
+    def run(c):
+        out = torch.empty_like(c[1])
+        c[0].eps(c[1].data_ptr(), c[2].data_ptr(), c[3].data_ptr(), out)
+        return out[:20].cpu()
+
+    first = case(*large)
+    before = run(first)
+    second = case(*small)
+    w, a, mu = second[4:7]
+    out, mu_d = torch.empty_like(second[1]), torch.from_numpy(mu).to(dev)
+    abi.pa_gmm_eps_noalloc(mu_d.data_ptr(), w.K, w.D, w.gmm_std, a, second[1].data_ptr(), second[2].data_ptr(),
+                           20, out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    for c in (first, second):
+        w, a, mu, idx, x = c[4:]
+        want = gmm_eps(x.astype(np.float64), np.asarray(a)[idx], mu.astype(np.float64), w.gmm_std)
+        rel = np.abs(run(c).numpy() - want).max(axis=1) / np.abs(want).max(axis=1)
+        assert rel.max() <= 2e-6, rel.max()
+    assert torch.equal(run(first), before)
+    for c in (first, second):
+        c[0].close()
+
+
 @pytest.mark.parametrize("K,D,cap,form", [
     (17, 16384, 143, 0), (17, 16384, 144, 1), (32, 3001, 500, 1), (32, 3001, 400, 0),  # K D cap = 40e6
     (65, 1024, 180, 0), (65, 1024, 181, 1),                                              # 12e6
