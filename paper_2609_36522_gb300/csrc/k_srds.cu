@@ -683,6 +683,16 @@ void s_forget_loop(pa_srds* h) {
   h->loop_last = nullptr;
 }
 
+// Whether the sampler's kernels may take [batch][D] values where they lie: in
+// this device's memory, outside the workspace or in batch_x, which the kernels
+// that start and end a generation do not touch otherwise.
+bool s_in_place(const pa_srds* h, const float* x) {
+  const SLayout& L = h->L;
+  const size_t n = (size_t)h->d.B * h->d.D * sizeof(float);
+  return pa::on_current_device(x) && pa::apart(x, n, h->ws, L.batch_x) &&
+         pa::apart(x, n, h->ws + L.miss_bt, L.total - L.miss_bt);
+}
+
 Stage current_stage(const pa_srds* h) {
   Stage st{};
   st.iter = h->iter;
@@ -808,9 +818,8 @@ extern "C" pa_status pa_srds_init(pa_srds* h, const float* x_init) {
   if (!h || !x_init) return s_fail("pa_srds_init: NULL argument", PA_ERR_ARG);
   if (h->loop_capturing) return s_fail("pa_srds_init: a generation is being captured", PA_ERR_STATE);
   const SDev& d = h->d;
-  // x_init is widened into U_0 from where it lies, or, off this device's
-  // memory, staged in batch_x first
-  const bool here = pa::on_current_device(x_init);
+  // x_init is widened into U_0 from where it lies, or staged in batch_x first
+  const bool here = s_in_place(h, x_init);
   cudaError_t e = cudaSuccess;
   if (!here) e = cudaMemcpyAsync(d.batch_x, x_init, (size_t)d.B * d.D * sizeof(float), cudaMemcpyDefault, h->st);
   if (e != cudaSuccess) return s_fail(std::string("pa_srds_init: ") + cudaGetErrorString(e), PA_ERR_CUDA);
@@ -933,9 +942,9 @@ extern "C" pa_status pa_srds_result(pa_srds* h, float* x_out) {
   if (h->loop_capturing) return s_fail("pa_srds_result: synchronises; not inside a capture", PA_ERR_STATE);
   if (h->phase != 2) return s_fail("pa_srds_result: not finished", PA_ERR_STATE);
   const SDev& d = h->d;
-  // U_N narrowed to fp32 where it is wanted, or, off this device's memory, in
-  // batch_x (free once sampling is done) and then copied out
-  const bool here = pa::on_current_device(x_out);
+  // U_N narrowed to fp32 where it is wanted, or in batch_x (free once sampling
+  // is done) and then copied out
+  const bool here = s_in_place(h, x_out);
   cudaError_t e = pa::launch_ex(k_srds_store, dim3(32, d.B), dim3(256), 0, h->st, 0, d, here ? x_out : d.batch_x, d.N);
   h->launches++;
   if (e == cudaSuccess && !here)

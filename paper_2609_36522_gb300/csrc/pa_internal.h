@@ -165,6 +165,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 bool on_current_device(const void* p);  // an address in the current device's memory (pa_solver.cpp)
+// [p, p + n) and [q, q + m) share no byte.
+inline bool apart(const void* p, size_t n, const void* q, size_t m) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+  return a + n <= b || b + m <= a;
+}
 bool pdl_enabled();  // false when the environment sets PA_DISABLE_PDL=1
 
 // Let kernel `kern` take `bytes` of dynamic shared memory on the current device

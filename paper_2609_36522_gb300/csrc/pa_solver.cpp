@@ -228,24 +228,32 @@ bool loop_busy(pa_solver* s, const char* where) {
   return true;
 }
 
+// Whether the solver's kernels may take [batch][D] values where they lie.
+bool in_place(const pa_solver* s, const float* x) {
+  return pa::on_current_device(x) &&
+         pa::apart(x, (size_t)s->d.B * s->d.D * sizeof(float), s->ws, s->L.total);
+}
+
 // Enqueue the start of a generation: x_init ([batch][D], host or device) into
 // state 0 of every trajectory (the rest of the first window is lazy), the first
 // plan (every timestep a first entry), its batch, both sets of the reductions'
 // (and the Anderson Gram sums') accumulators cleared: one kernel, which reads
-// x_init itself where that lies in this device's memory.
+// x_init itself where that lies in this device's memory, outside the workspace
+// (a view of the last batch, say: the kernel writes the first batch there while
+// its other CTAs still read).
 cudaError_t begin_generation(pa_solver* s, const float* x_init) {
   const pa::Dev& d = s->d;
-  if (pa::on_current_device(x_init)) return pa::launch_init(d, x_init, s->st);
+  if (in_place(s, x_init)) return pa::launch_init(d, x_init, s->st);
   const cudaError_t e = cudaMemcpy2DAsync(d.X, (size_t)(d.P + 1) * d.D * sizeof(float), x_init, (size_t)d.D * sizeof(float),
                                           (size_t)d.D * sizeof(float), d.B, cudaMemcpyDefault, s->st);
   return e == cudaSuccess ? pa::launch_init(d, nullptr, s->st) : e;
 }
 
 // Enqueue the copies of x_T into x_out (unless NULL) and of the counters into
-// `mirror` (pinned): one kernel for an x_out in this device's memory, else two
+// `mirror` (pinned): one kernel for an x_out that it may write in place, else two
 // copies (a kernel's writes across to host memory are no quicker).
 cudaError_t copy_outcome(pa_solver* s, float* x_out, pa::Ctl* mirror) {
-  if (x_out && pa::on_current_device(x_out)) return pa::launch_poll(s->d, x_out, mirror, s->st);
+  if (x_out && in_place(s, x_out)) return pa::launch_poll(s->d, x_out, mirror, s->st);
   cudaError_t e = x_out ? copy_xt(s, x_out) : cudaSuccess;
   if (e == cudaSuccess) e = cudaMemcpyAsync(mirror, s->d.ctl, sizeof(pa::Ctl), cudaMemcpyDeviceToHost, s->st);
   return e;

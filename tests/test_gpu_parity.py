@@ -233,6 +233,61 @@ def test_host_x_init_equals_device_x_init():
     assert np.array_equal(a["x_final"], b["x_final"])
 
 
+@pytest.mark.parametrize("shape", [(4, 16, 16), (3, 5, 7), (4, 64, 64)])
+@pytest.mark.parametrize("sampler", ["picard", "srds"])
+def test_x_init_in_the_workspace(sampler, shape):
+    """A generation that starts from rows of the batch that the last step
+    handed out (a view of the workspace, which the first kernel of a
+    generation writes) is bit for bit the one that starts from a copy of them,
+    step by step and captured."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser, Solver, SrdsSolver
+    w = W.TINY.with_(T=20, window=12, latent_shape=shape, batch=3, seed=29)
+    a, x0, mu = W.inputs(w)
+    stream = torch.cuda.Stream()  # a capture needs a stream of its own
+    with torch.cuda.stream(stream):
+        if sampler == "srds":
+            s = SrdsSolver(w.T, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch, stream=stream)
+            rows = s.max_rows
+        else:
+            s = Solver(w.T, w.window, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch, stream=stream)
+            rows = w.batch * s.window
+        g = GmmDenoiser(torch.from_numpy(mu).cuda(), w.gmm_std, a, rows, stream=stream)
+        eps = torch.empty(rows, w.D, dtype=torch.float32, device="cuda")
+
+        def denoise(batch_x, miss_bt, n_miss):
+            g.eps(batch_x, miss_bt, n_miss, eps)
+            return eps
+
+        def steps(x):
+            s.init(x)
+            while (out := s.step()) is not None:
+                denoise(out.batch_x_ptr, out.miss_bt_ptr, s.n_miss_dev())
+                s.submit_eps(eps)
+            return s.result().clone()
+
+        def first_rows(shift):
+            s.init(torch.from_numpy(x0).cuda())
+            out = s.step()
+            batch = out.batch_x if shift == 0 else s._view(out.batch_x_ptr + 4 * shift * w.D, torch.float32, w.batch, w.D)
+            return batch[:w.batch]
+
+        for shift in (0, 10):  # the batch's first rows; rows of two trajectories
+            if sampler == "srds" and shift:
+                continue  # a Parareal generation's first stage has `batch` rows
+            view = first_rows(shift)
+            copy = view.clone()
+            from_view = steps(view)
+            assert torch.equal(from_view, steps(copy))
+            want = s.generate(copy, denoise).clone()  # captures; the next call only launches
+            view = first_rows(shift)
+            s.init(torch.from_numpy(x0).cuda())  # a loop is not launched between step and submit_eps
+            assert torch.equal(view, copy)
+            assert torch.equal(s.generate(view, denoise), want)
+    s.close()
+    g.close()
+
+
 def _gmm_rows(w, n, seed=0):
     a, _, mu = W.inputs(w)
     rng = np.random.default_rng(seed)
