@@ -128,8 +128,8 @@ PA_API pa_status pa_set_noise(pa_solver* s, double eta, const float* noise_dev);
  * x_init (Sec. 2.1 initial trajectory estimate); every first-window timestep is
  * a first entry, hence a miss (Sec. 2.2). Clears the cache and counters,
  * plans the first iteration and gathers its batch (one kernel, which reads
- * x_init itself where that is in the current device's memory outside the
- * workspace; a copy comes first otherwise), all asynchronous on the solver's
+ * x_init itself where that is in the solver's device's memory outside the
+ * workspace and that device is current; a copy comes first otherwise), all asynchronous on the solver's
  * stream. x_init may lie in the workspace: the batch of the last step, say. May be called again at any time to
  * restart. */
 PA_API pa_status pa_init(pa_solver* s, const float* x_init);

@@ -623,7 +623,7 @@ struct pa_srds {
   int iter;       // current iteration (0 = coarse initialisation)
   int stage;      // index within the iteration: fine stages first (iter >= 1), then coarse
   int64_t g;      // stages since pa_srds_init: the distance set of stage g is g mod 2
-  int nsm;        // SMs of the device
+  int dev, nsm;   // the device current at pa_srds_create, its SMs
   int64_t launches;
   SCtl* host_ctl;
   // a whole generation captured as one CUDA graph (pa_srds_loop_*): a chain
@@ -689,7 +689,7 @@ void s_forget_loop(pa_srds* h) {
 bool s_in_place(const pa_srds* h, const float* x) {
   const SLayout& L = h->L;
   const size_t n = (size_t)h->d.B * h->d.D * sizeof(float);
-  return pa::on_current_device(x) && pa::apart(x, n, h->ws, L.batch_x) &&
+  return pa::on_device(x, h->dev) && pa::apart(x, n, h->ws, L.batch_x) &&
          pa::apart(x, n, h->ws + L.miss_bt, L.total - L.miss_bt);
 }
 
@@ -798,9 +798,8 @@ extern "C" pa_status pa_srds_create(pa_srds** out, int T, const int64_t* latent_
     const int a0 = n * s, a1 = (n + 1) * s < T ? (n + 1) * s : T;
     jump(alphas_cumprod[a0], alphas_cumprod[a1], &hc[2 * T + n], &hc[2 * T + N + n]);
   }
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = cudaGetDevice(&h->dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
   if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&h->host_ctl), sizeof(SCtl), cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaMemcpyAsync(coef, hc.data(), hc.size() * sizeof(float2), cudaMemcpyHostToDevice, h->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.ctl, 0, sizeof(SCtl), h->st);

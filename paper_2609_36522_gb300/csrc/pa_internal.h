@@ -8,6 +8,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "pa_place.h"
+
 namespace pa {
 
 constexpr int kMaxWindow = 1024;
@@ -164,12 +166,9 @@ constexpr uint32_t kWaitLimit = 1u << 17;  // tries of an mbarrier wait (~1.3 s 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-bool on_current_device(const void* p);  // an address in the current device's memory (pa_solver.cpp)
-// [p, p + n) and [q, q + m) share no byte.
-inline bool apart(const void* p, size_t n, const void* q, size_t m) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
-  return a + n <= b || b + m <= a;
-}
+// An address that kernels on a stream of device `dev` may be launched to take:
+// in that device's memory, that device current (pa_solver.cpp).
+bool on_device(const void* p, int dev);
 bool pdl_enabled();  // false when the environment sets PA_DISABLE_PDL=1
 
 // Let kernel `kern` take `bytes` of dynamic shared memory on the current device

@@ -20,14 +20,14 @@ namespace pa {
 static thread_local std::string g_err;
 void set_error(const std::string& msg) { g_err = msg; }
 
-bool on_current_device(const void* p) {
+bool on_device(const void* p, int dev) {
   cudaPointerAttributes a = {};
-  int dev = -1;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+  int current = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&current) != cudaSuccess) {
     (void)cudaGetLastError();  // not an address the runtime knows: the copies sort it out
     return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == dev;
+  return kernels_reach(a.type == cudaMemoryTypeDevice, a.device, current, dev);
 }
 
 cudaError_t allow_smem(const void* kern, size_t bytes) {
@@ -71,6 +71,7 @@ struct pa_solver {
   pa::Layout L;
   char* ws;
   cudaStream_t st;
+  int dev;           // the device of st and the workspace: the one current at pa_create
   St state;
   int update_kind;   // requested: 0 plain, 1 bulk pipeline, 2 lean register form, 3 fused step
   int lean_shape;    // launch shape of the lean register form
@@ -230,7 +231,7 @@ bool loop_busy(pa_solver* s, const char* where) {
 
 // Whether the solver's kernels may take [batch][D] values where they lie.
 bool in_place(const pa_solver* s, const float* x) {
-  return pa::on_current_device(x) &&
+  return pa::on_device(x, s->dev) &&
          pa::apart(x, (size_t)s->d.B * s->d.D * sizeof(float), s->ws, s->L.total);
 }
 
@@ -382,7 +383,9 @@ pa_status pa_create(pa_solver** out, int T, int window, const int64_t* latent_sh
   s->loop_capturing = s->looped = false;
   s->plan_node = nullptr;
   s->loop_k0 = s->loop_launches0 = 0;
-  cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&s->host_ctl), 3 * sizeof(pa::Ctl), cudaHostAllocDefault);
+  cudaError_t e = cudaGetDevice(&s->dev);
+  if (e == cudaSuccess)
+    e = cudaHostAlloc(reinterpret_cast<void**>(&s->host_ctl), 3 * sizeof(pa::Ctl), cudaHostAllocDefault);
   if (e != cudaSuccess) {
     delete s;
     return cuda_fail("pa_create: cudaHostAlloc", e);

@@ -102,3 +102,42 @@ def test_null_handles_are_rejected(lib):
     assert L.pa_gmm_set_form(None, 0) == abi.PA_ERR_ARG
     h = C.c_void_p()
     assert L.pa_gmm_create(C.byref(h), 0, 16, None, 0.5, None, 4, 4, None, 0, None) == abi.PA_ERR_ARG
+
+
+PLACE_CHECK = r"""
+#include "pa_place.h"
+#include <cstdio>
+int main() {
+  using pa::apart;
+  using pa::kernels_reach;
+  char b[64];
+  int bad = 0;
+  // the rule for buffers: nothing shared, touching ends allowed
+  bad += !apart(b, 16, b + 16, 16) + !apart(b + 16, 16, b, 16) + !apart(b, 8, b + 32, 8);
+  bad += apart(b, 17, b + 16, 16) + apart(b + 8, 4, b, 64) + apart(b, 64, b + 8, 4) + apart(b, 8, b, 8);
+  // the rule for devices, over every buffer, current and solver device of two
+  for (int m = 0; m < 2; ++m)
+    for (int c = 0; c < 2; ++c)
+      for (int s = 0; s < 2; ++s) {
+        bad += kernels_reach(true, m, c, s) != (m == s && c == s);
+        bad += kernels_reach(false, m, c, s);
+      }
+  std::printf("%d\n", bad);
+  return bad != 0;
+}
+"""
+
+
+def test_buffers_that_kernels_take_in_place(tmp_path):
+    """x_init and x_out go through copies unless the solver's device holds them
+    and is current, and unless they keep clear of the workspace. (One GPU shows
+    no other device: the rule itself, compiled for the host.)"""
+    import os
+    import subprocess
+    src, exe = tmp_path / "place.cpp", tmp_path / "place"
+    src.write_text(PLACE_CHECK)
+    subprocess.run(["g++", "-std=c++17", "-I", pa_build.CSRC, str(src), "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)], capture_output=True, text=True).stdout == "0\n"
+    for f in ("pa_solver.cpp", "k_srds.cu"):  # every place that asks goes by the solver's device
+        text = open(os.path.join(pa_build.CSRC, f)).read()
+        assert "pa::on_device(x, " in text and "on_current_device" not in text

@@ -288,6 +288,54 @@ def test_x_init_in_the_workspace(sampler, shape):
     g.close()
 
 
+@pytest.mark.parametrize("shape", [(4, 16, 16), (4, 64, 64), (1, 1, 4)])
+@pytest.mark.parametrize("sampler", ["picard", "srds"])
+def test_buffers_off_the_16_byte_boundaries(sampler, shape):
+    """x_init and x_out 4 bytes past a 16-byte boundary, in device memory and
+    in pinned host memory, with rows of whole 16-byte pieces: bit for bit the
+    aligned generation, nothing written outside x_out."""
+    import torch
+    from paper_2609_36522_gb300 import abi
+    from paper_2609_36522_gb300.solver import GmmDenoiser, Solver, SrdsSolver
+    w = W.TINY.with_(T=20, window=12, latent_shape=shape, batch=3, seed=30)
+    a, x0, mu = W.inputs(w)
+    if sampler == "srds":
+        s = SrdsSolver(w.T, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch)
+        rows = s.max_rows
+    else:
+        s = Solver(w.T, w.window, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch)
+        rows = w.batch * s.window
+    g = GmmDenoiser(torch.from_numpy(mu).cuda(), w.gmm_std, a, rows)
+    eps = torch.empty(rows, w.D, dtype=torch.float32, device="cuda")
+    n = w.batch * w.D
+
+    def buffer(host, shift):
+        kw = {"pin_memory": True} if host else {"device": "cuda"}
+        b = torch.full((n + 2 * shift + 8,), 7.0, dtype=torch.float32, **kw)
+        assert b.data_ptr() % 16 == 0
+        return b, b[shift:shift + n].view(w.batch, w.D)
+
+    results = []
+    for host in (False, True):
+        for shift in (0, 1):
+            _, x = buffer(host, shift)
+            x.copy_(torch.from_numpy(x0).view(w.batch, w.D))
+            torch.cuda.synchronize()
+            (abi.pa_srds_init if sampler == "srds" else abi.pa_init)(s.h, x.data_ptr())
+            while (out := s.step()) is not None:
+                g.eps(out.batch_x_ptr, out.miss_bt_ptr, s.n_miss_dev(), eps)
+                s.submit_eps(eps)
+            whole, y = buffer(host, shift)
+            torch.cuda.synchronize()
+            (abi.pa_srds_result if sampler == "srds" else abi.pa_result)(s.h, y.data_ptr())
+            results.append(y.cpu().clone())
+            assert (whole[:shift] == 7.0).all() and (whole[shift + n:] == 7.0).all()
+    assert np.isfinite(results[0].numpy()).all()
+    assert all(torch.equal(r, results[0]) for r in results[1:])
+    s.close()
+    g.close()
+
+
 def _gmm_rows(w, n, seed=0):
     a, _, mu = W.inputs(w)
     rng = np.random.default_rng(seed)
