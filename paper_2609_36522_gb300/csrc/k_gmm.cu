@@ -13,8 +13,8 @@
 //   k_gmm_dots     dot products G = X M^T, split over column chunks of D
 //                  (16-row tiles staged in shared memory, 4 rows x 8
 //                  components per thread); each CTA adds its chunk sums, in
-//                  2^-32 fixed point, into int64 accumulators with integer
-//                  atomics (exact: the order of arrival does not matter)
+//                  fixed point, into int64 accumulators with integer atomics
+//                  (exact: the order of arrival does not matter)
 //   k_gmm_out      per 16-row block: logits and max-subtracted softmax of its
 //                  rows from the accumulators, then eps = a x - a sqrt(a) R M
 //                  over staged 16-row x 256-column tiles (4 x 4 outputs per
@@ -25,6 +25,8 @@
 // wait) and records e for the output kernel; the output kernel reads set e mod 2
 // and advances the epoch. No kernel waits for another CTA, and the state lives on
 // the device, so a captured CUDA graph replays correctly.
+// The fixed point goes by the means (fixed_scale); a sum beyond it marks its
+// accumulator, and the output kernel forms that dot product itself.
 // Per-timestep scalars (sqrt(a), 1/(2v), sqrt(1-a)/v) are computed on the
 // host in fp64 from alpha-bar and stored in fp32, so 1 - a never cancels in
 // fp32. Reductions run in a fixed order: results are bitwise reproducible.
@@ -65,7 +67,28 @@ constexpr int kOutRows = 16;     // rows per output CTA
 constexpr int kOutCols = 256;    // columns per output CTA (four per thread)
 constexpr size_t kDotSmemBudget = 96 * 1024;
 constexpr int kDotCtas = 480;    // CTAs that a dots launch should have: about three per SM
-constexpr float kDotScale = 4294967296.f;  // 2^32: fixed-point scale of the dot-product accumulators
+
+// The fixed point of the dot-product accumulators. Let 2^e be the root mean
+// square of the largest mean, rounded down; rows are of the order of the means
+// or of the unit noise, whichever is larger, so their products are of the order
+// of 2^(e + max(e, 0)), and a unit is 2^-32 of that: at unit scale 2^-32. A chunk
+// sum that leaves no room for `nchunk` of its size (2^59 units) is not added but
+// marks the accumulator, a value that is not finite with the higher mark; the
+// others' sums, below 2^59 in any order, move a mark by less than half of the
+// distance to the next. So dot products of any size come out as in fp32: the
+// output kernel forms a marked one from the row and the mean (up to kWideD
+// columns: 16 rows of them take it 27 ms at 16 components; beyond, the row is
+// NaN), and a row with a value that is not finite is NaN.
+constexpr float kFixedRoom = 0x1p59f;
+constexpr long long kMarkWide = 4ll << 60, kMarkNan = 6ll << 60;
+constexpr int64_t kWideD = 1 << 18;
+__device__ __forceinline__ int fixed_exponent(uint32_t norm_bits, int64_t D) {  // log2 of the units in 1
+  const float ms = __uint_as_float(norm_bits) / (float)D;  // mean square
+  if (!(ms > 0.f)) return 32;
+  const int e = max(-40, min(40, ((int)(__float_as_uint(ms) >> 23) - 127) >> 1));
+  return 32 - e - max(e, 0);
+}
+__device__ __forceinline__ float power_of_two(int e) { return __int_as_float((e + 127) << 23); }  // |e| <= 126
 
 // Default form by sizes (pa_gmm_create). K components, D columns, a capacity of R
 // rows; the figures are us per call on a batch filled to 4/5.
@@ -85,7 +108,8 @@ constexpr float kDotScale = 4294967296.f;  // 2^32: fixed-point scale of the dot
 // R 1000 (262e6) 63.1 / 56.4 / 58.6, R 1600 86.8 / 73.2 / 81.1; without the
 // cluster kernel form 0 / 1 at K 16, D 40000, R 256 (164e6) 42.4 / 38.1, at K 8,
 // R 1000 (320e6) 110 / 122, and with D % 4 != 0, where form 1 copies four bytes at
-// a time, at K 16, D 40001, R 1000 170 / 188.
+// a time, at K 16, D 40001, R 1000 170 / 188. Rows that form 0's fixed point does
+// not hold (kWideD) take form 1 above 16 components.
 constexpr int64_t kTcWork = 40 * 1000 * 1000;
 constexpr int64_t kTcWideWork = 12 * 1000 * 1000;
 constexpr int kManyRows = 200;        // many short rows: R >= kManyRows, D <= kShortRow,
@@ -107,6 +131,10 @@ struct GmmLayout {
 struct GmmEpoch {
   uint32_t epoch;   // advanced by the output kernel
   uint32_t cur;     // the epoch of the dot products just formed
+  float scale;      // units of the fixed point in 1, and its inverse
+  float unit;
+  uint32_t norm;    // the largest ||mu_k||^2, as the bits of the fp32 value
+  uint32_t norms;   // components whose norm is in it
 };
 
 size_t dots_smem_bytes(int K, int chunk) {
@@ -155,9 +183,10 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// ||mu_k||^2, one CTA per component, fixed-order tree.
+// ||mu_k||^2, one CTA per component, fixed-order tree; the last one to finish
+// takes the fixed point from the largest.
 __global__ void __launch_bounds__(256) k_gmm_norms(const float* __restrict__ mu, int64_t D,
-                                                   float* __restrict__ mnorm) {
+                                                   float* __restrict__ mnorm, GmmEpoch* ep) {
   __shared__ float s[8];
   const float* m = mu + (int64_t)blockIdx.x * D;
   float acc = 0.f;
@@ -169,6 +198,13 @@ __global__ void __launch_bounds__(256) k_gmm_norms(const float* __restrict__ mu,
     float t = 0.f;
     for (int w = 0; w < 8; ++w) t += s[w];
     mnorm[blockIdx.x] = t;
+    if (t > 0.f) atomicMax(&ep->norm, __float_as_uint(t));  // the bits of positive values are in their order
+    __threadfence();
+    if (atomicAdd(&ep->norms, 1u) == gridDim.x - 1) {
+      const int e = fixed_exponent(atomicMax(&ep->norm, 0u), D);
+      ep->scale = power_of_two(e);
+      ep->unit = power_of_two(-e);
+    }
   }
 }
 
@@ -234,7 +270,7 @@ __device__ __forceinline__ long long* begin_dots(long long* gacc2, GmmEpoch* ep,
 __global__ void __launch_bounds__(kThreads) k_gmm_dots(const float* __restrict__ X,
                                                        const float* __restrict__ mu,
                                                        const int32_t* __restrict__ n_rows_dev,
-                                                       int K, int64_t D, int chunk, int nchunk, int max_rows,
+                                                       int K, int64_t D, int chunk, float room, int max_rows,
                                                        bool bulk, long long* __restrict__ gacc2,
                                                        GmmEpoch* ep, int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -258,6 +294,7 @@ __global__ void __launch_bounds__(kThreads) k_gmm_dots(const float* __restrict__
   pdl_trigger();  // the successor may now run its prologue
   const int n_rows = min(*n_rows_dev, max_rows);
   const uint32_t epoch = ep->epoch;
+  const float scale = ep->scale;
   const int nr = min(kDotRows, n_rows - r0);
   if (nr <= 0) {  // no rows for this CTA: the means copy lands before it exits
     begin_dots(gacc2, ep, epoch, (int64_t)max_rows * K);
@@ -320,8 +357,39 @@ __global__ void __launch_bounds__(kThreads) k_gmm_dots(const float* __restrict__
     }
     for (; cs < CS; ++cs) a4[0] += ro[cs];
     const float sum = (a4[0] + a4[1]) + (a4[2] + a4[3]);
-    atomicAdd(reinterpret_cast<unsigned long long*>(gacc + (int64_t)r0 * K + o),
-              static_cast<unsigned long long>(__float2ll_rn(sum * kDotScale)));
+    long long* acc_o = gacc + (int64_t)r0 * K + o;
+    if (fabsf(sum * scale) < room)  // and not NaN
+      atomicAdd(reinterpret_cast<unsigned long long*>(acc_o), static_cast<unsigned long long>(__float2ll_rn(sum * scale)));
+    else
+      atomicMax(acc_o, fabsf(sum) <= 3.402823466e38f ? kMarkWide : kMarkNan);
+  }
+}
+
+// The logits of a row block whose dot products the fixed point did not hold (the
+// value `wide` in s_r), by the whole CTA in a fixed order. Seldom: kept out of
+// the output kernel's code.
+__device__ __noinline__ void form_wide(const float* __restrict__ X, const float* __restrict__ mu,
+                                       const float* __restrict__ mnorm, int K, int64_t D, int nr, float wide,
+                                       const float* s_sa, const float* s_q, float* s_r, float* s_part) {
+  const int tid = threadIdx.x;
+  for (int q = 0; q < nr * K; ++q) {
+    if (__float_as_uint(s_r[q]) != __float_as_uint(wide)) continue;  // the same for every thread
+    const int rr = q / K, k = q % K;
+    const float* xr = X + (int64_t)rr * D;
+    const float* mk = mu + (int64_t)k * D;
+    float dot = 0.f;
+#pragma unroll 8
+    for (int64_t c = tid; c < D; c += kThreads) dot = fmaf(xr[c], mk[c], dot);
+    dot = warp_sum(dot);
+    if ((tid & 31) == 0) s_part[tid >> 5] = dot;
+    __syncthreads();
+    if (tid == 0) {
+      dot = 0.f;
+      for (int w = 0; w < kThreads / 32; ++w) dot += s_part[w];
+      const float sa = s_sa[rr];
+      s_r[q] = (2.f * sa * dot - sa * sa * mnorm[k]) * s_q[rr];
+    }
+    __syncthreads();
   }
 }
 
@@ -346,6 +414,7 @@ __global__ void __launch_bounds__(kThreads) k_gmm_out(const float* __restrict__ 
   __shared__ float s_r[kOutRows * kMaxK];
   __shared__ float s_c[kOutRows * 2];
   __shared__ float s_sa[kOutRows], s_q[kOutRows];
+  __shared__ float s_part[kThreads / 32];
   const int n_rows = min(*n_rows_dev, max_rows);  // written two kernels back
   const int r0 = blockIdx.y * kOutRows;
   if (r0 >= n_rows) {  // every CTA passes the dependency wait before it exits
@@ -380,22 +449,33 @@ __global__ void __launch_bounds__(kThreads) k_gmm_out(const float* __restrict__ 
   // status word (one round trip): a dot-product kernel that timed out left
   // the sums incomplete
   const uint32_t cur = ep->cur;
+  const float unit = ep->unit;
   const int dots_status = __ldcg(status);
   const int64_t set_size = (int64_t)max_rows * K;
   __syncthreads();
+  const float nan = __int_as_float(0x7fc00000), wide = __int_as_float(0x7fc00001);  // a marked sum until it is formed
+  bool any_wide = false;
   for (int q = tid; q < kOutRows * K; q += kThreads) {
     float l = 0.f;
     if (q < nr * K) {
       const int rr = q / K, k = q % K;
       const long long v0 = __ldcg(gacc2 + (int64_t)r0 * K + q);
       const long long v1 = __ldcg(gacc2 + set_size + (int64_t)r0 * K + q);
-      const float dot = __ll2float_rn((cur & 1u) ? v1 : v0) * (1.f / kDotScale);  // exact scale
-      const float sa = s_sa[rr];
-      l = (2.f * sa * dot - sa * sa * mnorm[k]) * s_q[rr];
+      const long long v = (cur & 1u) ? v1 : v0;
+      if (v >= 3ll << 60) {
+        const bool form = v < 5ll << 60 && D <= kWideD;
+        l = form ? wide : nan;
+        any_wide |= form;
+      } else {
+        const float dot = __ll2float_rn(v) * unit;  // exact scale
+        const float sa = s_sa[rr];
+        l = (2.f * sa * dot - sa * sa * mnorm[k]) * s_q[rr];
+      }
     }
     s_r[q] = l;
   }
-  __syncthreads();
+  if (__syncthreads_or(any_wide))
+    form_wide(X + (int64_t)r0 * D, mu, mnorm, K, D, nr, wide, s_sa, s_q, s_r, s_part);
   // softmax per row: a half-warp per row when K <= 16 (two rows per warp and
   // pass), else a warp; the reductions are the same trees either way
   {
@@ -765,7 +845,7 @@ constexpr int kClRows = 8;    // rows per cluster
 // See the constants above. (`rows16`: the means' rows start on 16-byte boundaries.)
 int default_form(const pa_gmm& g, bool rows16) {
   const double work = (double)g.K * (double)g.D * g.max_rows;
-  if (g.K > kClMaxK) return g.per && work >= (g.K > 64 ? kTcWideWork : kTcWork) ? 1 : 0;
+  if (g.K > kClMaxK) return g.per && (work >= (g.K > 64 ? kTcWideWork : kTcWork) || g.D > kWideD) ? 1 : 0;
   if (!g.cl_ok) return g.per && rows16 && g.K >= kTcFewMinK && work >= kTcFewWork0 ? 1 : 0;
   if (g.max_rows >= kManyRows && g.D <= kShortRow && g.D <= kShortPerRow * g.max_rows) return 0;
   return g.per && g.max_rows >= kTcFewRows && work >= kTcFewWork ? 1 : 2;
@@ -817,7 +897,8 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   if (e == cudaSuccess) e = cudaMemsetAsync(g->ws + L.epoch, 0, sizeof(GmmEpoch), g->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(g->ws + L.gacc, 0, (size_t)2 * max_rows * K * sizeof(long long), g->st);
   if (e == cudaSuccess) {
-    k_gmm_norms<<<K, 256, 0, g->st>>>(means_dev, D, reinterpret_cast<float*>(g->ws + L.mnorm));
+    k_gmm_norms<<<K, 256, 0, g->st>>>(means_dev, D, reinterpret_cast<float*>(g->ws + L.mnorm),
+                                      reinterpret_cast<GmmEpoch*>(g->ws + L.epoch));
     g->launches++;
     e = cudaGetLastError();
   }
@@ -925,7 +1006,7 @@ extern "C" pa_status pa_gmm_eps(pa_gmm* g, const float* batch_x_dev, const int32
   }
   e = pa::launch_ex(k_gmm_dots, dim3(L.nchunk, (g->max_rows + kDotRows - 1) / kDotRows), dim3(kThreads),
                     dots_smem_bytes(g->K, L.chunk), g->st, 0, batch_x_dev, g->means, n_rows_dev, g->K, g->D,
-                    L.chunk, L.nchunk, g->max_rows, bulk, gacc2, ep, status);
+                    L.chunk, kFixedRoom / (float)L.nchunk, g->max_rows, bulk, gacc2, ep, status);
   if (e == cudaSuccess)
     e = pa::launch_ex(k_gmm_out,
                       dim3((unsigned)((g->D + kOutCols - 1) / kOutCols), (g->max_rows + kOutRows - 1) / kOutRows),
@@ -1111,10 +1192,10 @@ extern "C" pa_status pa_gmm_eps_noalloc(const float* means_dev, int K, int64_t D
   }
   const bool bulk = D % 4 == 0 && ((reinterpret_cast<uintptr_t>(batch_x_dev) |
                                     reinterpret_cast<uintptr_t>(means_dev)) & 15) == 0;
-  k_gmm_norms<<<K, 256, 0, st>>>(means_dev, D, mnorm);
+  k_gmm_norms<<<K, 256, 0, st>>>(means_dev, D, mnorm, ep);
   const bool vec_out = D % 4 == 0 && (reinterpret_cast<uintptr_t>(batch_eps_dev) & 15) == 0;
   k_gmm_dots<<<dim3(nchunk, (n_rows + kDotRows - 1) / kDotRows), kThreads, dots_smem, st>>>(
-      batch_x_dev, means_dev, nrows_dev, K, D, chunk, nchunk, n_rows, bulk, gacc2, ep, status);
+      batch_x_dev, means_dev, nrows_dev, K, D, chunk, kFixedRoom / (float)nchunk, n_rows, bulk, gacc2, ep, status);
   k_gmm_out<<<dim3((unsigned)((D + kOutCols - 1) / kOutCols), (n_rows + kOutRows - 1) / kOutRows), kThreads,
               out_smem, st>>>(batch_x_dev, means_dev, gacc2, ep, coef, T, miss_bt_dev, mnorm, nrows_dev, K, D,
                               n_rows, bulk, vec_out, batch_eps_dev, status);

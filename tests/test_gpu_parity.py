@@ -520,6 +520,65 @@ def test_gmm_calls_back_to_back(form, K, D, cap):
     g.close()
 
 
+@pytest.mark.parametrize("K,D,scale,factor", [
+    (20, 49152, 255.0, 1.0),    # bytes as values: dot products past 2^31
+    (17, 1000, 1e6, 1.0), (8, 8192, 1e-4, 1.0), (40, 515, 1e-6, 1.0), (3, 64, 1e15, 1.0),
+    (8, 2048, 1.0, 1e7), (17, 3001, 1e-3, 1e9)])  # rows far larger than the means
+def test_gmm_cuda_core_form_at_any_scale(K, D, scale, factor):
+    """The CUDA-core denoiser's fixed-point dot products at other scales than
+    one: means and rows of size `scale`, rows times `factor`, up to sums that
+    the fixed point does not hold. Against the fp64 oracle, each value within
+    8 fp32 roundings of the larger of its two terms (x and the mean), where
+    the weights are those of one mean (all rows here but for chance)."""
+    import torch
+    from oracle.gmm import gmm_eps
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    rng = np.random.default_rng(K * D)
+    n, std = 20, 0.5
+    a = W.inputs(W.SD15)[0]
+    mu = (scale * np.abs(rng.standard_normal((K, D)))).astype(np.float32)
+    idx = np.linspace(0, len(a) - 2, n).astype(np.int32)
+    x = (factor * np.sqrt(a[idx])[:, None] * mu[rng.integers(0, K, n)]
+         + min(scale, 1.0) * np.sqrt(1 - a[idx])[:, None] * rng.standard_normal((n, D))).astype(np.float32)
+    dev = torch.device("cuda")
+    g = GmmDenoiser(torch.from_numpy(mu).to(dev), std * min(scale, 1.0), a, 32)
+    g.set_form(0)
+    xd = torch.zeros(32, D, device=dev)
+    xd[:n] = torch.from_numpy(x).to(dev)
+    miss = np.stack([np.zeros(n, np.int32), idx], axis=1)
+    md = torch.zeros(32, 2, dtype=torch.int32, device=dev)
+    md[:n] = torch.from_numpy(miss).to(dev)
+    nd = torch.tensor([n], dtype=torch.int32, device=dev)
+    out = torch.empty(32, D, device=dev)
+    for _ in range(2):
+        g.eps(xd.data_ptr(), md.data_ptr(), nd.data_ptr(), out)
+    got = out[:n].cpu().numpy().astype(np.float64)
+    ai = a[idx][:, None]
+    v = ai * (std * min(scale, 1.0)) ** 2 + 1 - ai
+    want = gmm_eps(x.astype(np.float64), a[idx], mu.astype(np.float64), std * min(scale, 1.0))
+    # the logits' own error in fp32, and how far it moves the weights: not at all
+    # where one mean leads by more than it and e^40
+    dots = np.abs(x.astype(np.float64)) @ np.abs(mu.astype(np.float64)).T
+    norms = (mu.astype(np.float64) ** 2).sum(1)
+    logits = np.sort((2 * np.sqrt(ai) * (x.astype(np.float64) @ mu.astype(np.float64).T) - ai * norms) / (2 * v))
+    err = (4 * 2.0 ** -24 * (2 * np.sqrt(ai) * dots + ai * norms) / (2 * v)).max(1)
+    moved = np.where(logits[:, -1] - logits[:, -2] - 2 * err > 40, 0.0, np.minimum(1.0, 2 * err))
+    c = np.sqrt(1 - ai) / v
+    bound = c * (8 * 2.0 ** -24 * (np.abs(x) + np.sqrt(ai) * np.abs(mu).max(0))
+                 + moved[:, None] * np.sqrt(ai) * np.abs(mu).max(0))
+    assert (np.abs(got - want) <= bound).all(), (np.abs(got - want) / bound).max()
+    assert (moved < 1e-3).sum() >= n // 4
+    assert torch.isfinite(out[:n]).all()
+    # one row that is not finite: its row is NaN, the others stay bit for bit
+    for bad in (float("nan"), float("inf")):
+        xd[7, D // 2] = bad
+        again = torch.empty_like(out)
+        g.eps(xd.data_ptr(), md.data_ptr(), nd.data_ptr(), again)
+        keep = [r for r in range(n) if r != 7]
+        assert torch.isnan(again[7]).all() and torch.equal(again[keep], out[keep])
+    g.close()
+
+
 @pytest.mark.parametrize("form,large,small", [
     (0, (16, 12810, 640), (16, 12810, 50)),   # (K, D, capacity): a smaller capacity takes shorter chunks
     (0, (100, 4096, 64), (3, 4096, 64)), (2, (16, 16384, 64), (16, 4096, 64))])
