@@ -489,6 +489,10 @@ __global__ void __launch_bounds__(kSThreads) k_srds_apply(SDev d, Stage st, cons
   }
 }
 
+// The larger value, NaN if one is (fmax drops it): a trajectory with a NaN
+// boundary has not converged.
+__device__ __forceinline__ double nan_max(double a, double b) { return b > a || b != b ? b : a; }
+
 // Convergence of every trajectory after iteration `iter` (one CTA, a warp per
 // trajectory at a time, a lane per boundary): the boundaries' Eq. 2 sums from
 // the apply CTAs' partials in order, then their maximum.
@@ -512,10 +516,10 @@ __global__ void __launch_bounds__(kSFinishThreads) k_srds_finish(SDev d, int ite
         double sum = 0.0;
 #pragma unroll 16
         for (int k = 0; k < d.nstrip; ++k) sum += pt[k];
-        err = fmax(err, sum);
+        err = nan_max(err, sum);
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
+      for (int o = 16; o > 0; o >>= 1) err = nan_max(err, __shfl_xor_sync(0xffffffffu, err, o));
       err /= (double)d.D;  // one division: the fp64 unit takes two operations per clock
       more = !(err <= d.tol || iter >= d.N);
       if (lane == 0) {

@@ -265,3 +265,39 @@ def test_srds_generation_graph_call_order():
     assert torch.equal(s.generate(x0d, denoise), want)
     s.close()
     g.close()
+
+
+def test_srds_nan_is_not_converged():
+    """A NaN in one row of one fine stage: that trajectory's error is NaN from
+    then on and it runs to the last iteration, unconverged; the other
+    trajectory is the one of a clean run."""
+    import torch
+    from paper_2609_36522_gb300.solver import SrdsSolver, GmmDenoiser
+    w = W.TINY.with_(T=25, latent_shape=(4, 8, 8), K=3, sampler="srds", batch=2, seed=33)
+    a, x0, mu = W.inputs(w)
+
+    def run(poison):
+        s = SrdsSolver(w.T, w.latent_shape, a, w.tol, w.cache_thresh, batch=w.batch)
+        g = GmmDenoiser(torch.from_numpy(mu).cuda(), w.gmm_std, a, s.max_rows)
+        eps = torch.empty(s.max_rows, w.D, dtype=torch.float32, device="cuda")
+        s.init(torch.from_numpy(x0).cuda())
+        stage = 0
+        while (out := s.step()) is not None:
+            g.eps(out.batch_x_ptr, out.miss_bt_ptr, s.n_miss_dev(), eps)
+            if poison and stage == s.blocks + 1:  # iteration 1, its second fine stage
+                rows = out.miss_bt[:, 0] == 0
+                eps[:out.n_miss][rows.nonzero()[1]] = float("nan")
+            s.submit_eps(eps)
+            stage += 1
+        s.poll()
+        res = s.result().cpu().numpy(), s.errors(), s.stats()["iters"], s.blocks
+        s.close()
+        g.close()
+        return res
+
+    clean_x, clean_err, clean_iters, blocks = run(False)
+    x, err, iters, _ = run(True)
+    assert clean_iters < blocks and iters == blocks
+    assert np.isnan(err[:, 0]).all() and np.isnan(x[0]).any()
+    assert np.array_equal(x[1], clean_x[1])
+    assert np.array_equal(err[:clean_iters, 1], clean_err[:clean_iters, 1])
