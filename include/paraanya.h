@@ -571,13 +571,13 @@ PA_API int64_t pa_gmm_launches(const pa_gmm* g);
  * D and alignment; operands split into parts so that the result keeps fp32
  * accuracy. form 0: fp32 multiply-adds on the CUDA cores, two kernels.
  * The default goes by sizes: for K > 16 form 1 where K D max_rows is 40e6 or
- * more (12e6 for K > 64), else form 0; for K <= 16 form 2 where it is available,
+ * more (12e6 for K > 64) or D > 2^18, else form 0; for K <= 16 form 2 where it is available,
  * except form 0 for max_rows >= 200 with D <= 10000 and D <= 25 max_rows, and
  * form 1 where K D max_rows is 250e6 or more with max_rows >= 512; where form 2 is not available form 0, except form
  * 1 for K > 8, D % 4 == 0, aligned means and K D max_rows of 100e6 or more.
  * A call whose batch_x or batch_eps is not 16-byte aligned uses form 0 in place
- * of form 2. Forms 1 and 2 need a GPU of the sm_100 family, and to be set here
- * D % 4 == 0 and 16-byte aligned means. The forms agree to fp32 rounding; each
+ * of form 2. Forms 1 and 2 need a GPU of the sm_100 family, form 2 also 16-byte
+ * aligned means. The forms agree to fp32 rounding; each
  * is bitwise reproducible. Returns PA_ERR_ARG for a form that is not
  * available. */
 PA_API pa_status pa_gmm_set_form(pa_gmm* g, int form);

@@ -833,7 +833,6 @@ struct pa_gmm {
   cudaStream_t st;
   int64_t launches;
   bool per;     // the tensor-core kernels fit this device
-  bool tc_ok;   // ... and pa_gmm_set_form gives them for these sizes and means
   bool cl_ok;   // the single-kernel cluster form fits these sizes and this device
   int form;     // 0 CUDA cores, 1 tensor cores, 2 cluster form
 };
@@ -913,7 +912,6 @@ extern "C" pa_status pa_gmm_create(pa_gmm** out, int K, int64_t D, const float* 
   const bool rows16 = D % 4 == 0 && (reinterpret_cast<uintptr_t>(means_dev) & 15) == 0;
   g->per = false;
   if (e == cudaSuccess) e = pa::gmm_tc_setup(K, &g->per);
-  g->tc_ok = g->per && rows16;
   // The single-kernel cluster form for K <= 16 when D splits into kClSize
   // 16-byte-aligned column chunks whose tiles fit in shared memory and a
   // cluster of kClSize CTAs can be resident.
@@ -1040,9 +1038,8 @@ extern "C" int64_t pa_gmm_launches(const pa_gmm* g) { return g ? g->launches : -
 extern "C" pa_status pa_gmm_set_form(pa_gmm* g, int form) {
   if (!g) { pa::set_error("pa_gmm_set_form: NULL handle"); return PA_ERR_ARG; }
   if (form < 0 || form > 2) { pa::set_error("pa_gmm_set_form: form must be 0, 1 or 2"); return PA_ERR_ARG; }
-  if (form == 1 && !g->tc_ok) {
-    pa::set_error("pa_gmm_set_form: the tensor-core form needs an sm_100-family GPU, D % 4 == 0, "
-                  "16-byte aligned means and enough shared memory");
+  if (form == 1 && !g->per) {
+    pa::set_error("pa_gmm_set_form: the tensor-core form needs an sm_100-family GPU and enough shared memory");
     return PA_ERR_ARG;
   }
   if (form == 2 && !g->cl_ok) {

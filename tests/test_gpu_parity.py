@@ -413,7 +413,8 @@ def test_gmm_kernel_against_oracle(wname, n, max_rows, form):
     (16, 4096, 1500, 1600, 0), (5, 9000, 800, 800, 0),     # few components, many rows
     (128, 64, 19590, 19600, 0),                            # more row blocks than CTAs
     (18, 1024, 7, 8, 0), (1, 64, 3, 3, 0),                 # fewer pieces than CTAs
-    (100, 3000, 0, 256, 0)])                               # no rows
+    (100, 3000, 0, 256, 0),                                # no rows
+    (3, 37, 5, 8, 0), (17, 129, 20, 20, 3), (70, 1, 130, 140, 0), (33, 95, 300, 301, 2)])  # small and odd: 4-byte copies
 def test_gmm_persistent_kernels(K, D, n, cap, shift):
     """The persistent tensor-core denoiser (form 1) against the fp64 oracle at the edges of its row blocks, column units and tiles,
     twice in a row with bitwise equal results; rows past the count stay as
@@ -424,8 +425,9 @@ def test_gmm_persistent_kernels(K, D, n, cap, shift):
     a, mu, idx, x, miss = _gmm_rows(w, max(n, 1))
     dev = torch.device("cuda")
     g = GmmDenoiser(torch.from_numpy(mu).to(dev), w.gmm_std, a, cap)
-    if g.form() != 1:
-        g.set_form(1)
+    g.set_form(0)
+    g.set_form(1)  # any D and alignment, also where it is not the default
+    assert g.form() == 1
     l0 = g.launches()
     xd = torch.zeros(cap * D + shift, dtype=torch.float32, device=dev)[shift:].view(cap, D)
     xd[:n] = torch.from_numpy(x[:n]).to(dev)
