@@ -172,7 +172,7 @@ GmmLayout gmm_layout(int K, int64_t D, int max_rows, int T) {
   L.gacc = take((size_t)2 * max_rows * K * sizeof(long long));  // two sets, used in turn
   L.epoch = take(sizeof(GmmEpoch));
   L.status = take(sizeof(int32_t));
-  L.tc = take(pa::gmm_tc_layout(K, max_rows).total);
+  L.tc = take(pa::gmm_tc_layout(K, D, max_rows).total);
   L.total = o;
   return L;
 }

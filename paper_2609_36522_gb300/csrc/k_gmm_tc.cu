@@ -42,6 +42,15 @@ namespace {
 
 constexpr int kRows = 128;       // rows of a row block: at most an MMA's N / 2
 constexpr int kMaxCtas = 160;    // CTAs of the dot products at most (one per SM)
+constexpr int kUnit = 32;        // columns of a piece of the dot products
+
+// The CTAs that the dot products of up to max_rows rows keep busy, `limit` at most.
+inline int dots_ctas(int64_t D, int max_rows, int limit) {
+  const int64_t pieces = ((int64_t)max_rows + kRows - 1) / kRows * ((D + kUnit - 1) / kUnit);
+  return pieces < limit ? (int)pieces : limit;
+}
+// Rows of a slot of partial sums: a row block, or all rows of a handle that has fewer.
+__host__ __device__ inline int slot_rows(int max_rows) { return max_rows < kRows ? max_rows : kRows; }
 
 // components as stored: R rows and partial sums are padded to this many
 __host__ __device__ inline int kpad(int K) { return K <= 16 ? 16 : K <= 32 ? 32 : K <= 64 ? 64 : 128; }
@@ -139,7 +148,6 @@ __device__ __forceinline__ void named_sync(int id, int threads) {
 // A copy takes a microsecond and more, an operand stage's turn (split, MMAs)
 // less: with raw values in rings of their own up to five units are on their
 // way (four stages that held a unit from its copy to its MMAs: 20 us a call).
-constexpr int kUnit = 32;
 constexpr int kDtConvWarps = 16;
 constexpr int kDtGroupWarps = kDtConvWarps / 2;
 constexpr int kDtConv = kDtConvWarps * 32;
@@ -324,7 +332,7 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
       take_until(nc);
       // TMEM lane = component; up to 64 components lane 64 + k holds the products
       // with the means' lo parts
-      float* out = part + (int64_t)sh.slot(blk, u0) * kRows * KP;
+      float* out = part + (int64_t)sh.slot(blk, u0) * slot_rows(max_rows) * KP;
       float* sc = stage0;  // [kRows][64]: every MMA that reads the stages is complete
       if constexpr (!TWO) {
         if (q4 >= 2) {
@@ -434,14 +442,15 @@ __global__ void __launch_bounds__(kRespThreads) k_gmm_resp(const float* __restri
       pdl_trigger();  // the successor may now run its prologue
       waited = true;
     }
-    const float* p = part + ((int64_t)sh.slot(blk, 0) * kRows + r - blk * kRows) * KP + k;
+    const int64_t slot = (int64_t)slot_rows(max_rows) * KP;
+    const float* p = part + sh.slot(blk, 0) * slot + (int64_t)(r - blk * kRows) * KP + k;
     float hi = 0.f, lo = 0.f;
     for (int s = grp; s < members; s += kBatch * kGroups) {
       float v[kBatch];  // kBatch loads in flight
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
         v[u] = 0.f;
-        if (s + u * kGroups < members) v[u] = __ldcg(p + (int64_t)(s + u * kGroups) * kRows * KP);
+        if (s + u * kGroups < members) v[u] = __ldcg(p + (s + u * kGroups) * slot);
       }
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {  // TwoSum
@@ -788,12 +797,12 @@ cudaError_t sm_count(int* out) {
 }
 
 template <int KP>
-cudaError_t launch_tail(const GmmTcArgs& a, const GmmTcLayout& L, int grid, cudaStream_t st) {
+cudaError_t launch_tail(const GmmTcArgs& a, const GmmTcLayout& L, int dots_grid, int grid, cudaStream_t st) {
   const float* part = reinterpret_cast<const float*>(a.ws + L.part);
   float* resp = reinterpret_cast<float*>(a.ws + L.resp);
   float* rcoef = reinterpret_cast<float*>(a.ws + L.rcoef);
   cudaError_t e = launch_ex(k_gmm_resp<KP>, dim3(a.max_rows < kRespGrid ? a.max_rows : kRespGrid), dim3(kRespThreads), 0,
-                            st, 0, part, grid, a.coef, a.T, a.miss_bt, a.mnorm, a.n_rows, a.K, a.D, a.max_rows, resp,
+                            st, 0, part, dots_grid, a.coef, a.T, a.miss_bt, a.mnorm, a.n_rows, a.K, a.D, a.max_rows, resp,
                             rcoef);
   if (e != cudaSuccess) return e;
   return launch_ex(k_gmm_out_tc<KP>, dim3(grid), dim3(kOtThreads), OtShape<KP>::smem(), st, 0, a.X, a.mu,
@@ -802,12 +811,13 @@ cudaError_t launch_tail(const GmmTcArgs& a, const GmmTcLayout& L, int grid, cuda
 
 }  // namespace
 
-GmmTcLayout gmm_tc_layout(int K, int max_rows) {
+GmmTcLayout gmm_tc_layout(int K, int64_t D, int max_rows) {
   GmmTcLayout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, kAlign); return at; };
   const size_t blocks = ((size_t)max_rows + kRows - 1) / kRows;
-  L.part = take((kMaxCtas > blocks ? kMaxCtas : blocks) * kRows * kpad(K) * sizeof(float));  // a slot per CTA or block
+  const size_t ctas = (size_t)dots_ctas(D, max_rows, kMaxCtas);
+  L.part = take((ctas > blocks ? ctas : blocks) * slot_rows(max_rows) * kpad(K) * sizeof(float));  // a slot per CTA or block
   L.resp = take((size_t)max_rows * kpad(K) * sizeof(float));
   L.rcoef = take((size_t)2 * max_rows * sizeof(float));
   L.total = o;
@@ -839,20 +849,21 @@ cudaError_t gmm_tc_launch(const GmmTcArgs& a, cudaStream_t st) {
   int grid = 0;
   cudaError_t e = sm_count(&grid);
   if (e != cudaSuccess) return e;
-  const GmmTcLayout L = gmm_tc_layout(a.K, a.max_rows);
+  const int dots_grid = dots_ctas(a.D, a.max_rows, grid);
+  const GmmTcLayout L = gmm_tc_layout(a.K, a.D, a.max_rows);
   // 16-byte loads of the rows and the means where all of them are aligned
   const bool vec = a.D % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.X) | reinterpret_cast<uintptr_t>(a.mu)) & 15) == 0;
   const bool two = a.K > 64;
   auto dots = two ? (vec ? k_gmm_dots_tc<true, true> : k_gmm_dots_tc<true, false>)
                   : (vec ? k_gmm_dots_tc<false, true> : k_gmm_dots_tc<false, false>);
-  e = launch_ex(dots, dim3(grid), dim3(kDtThreads), dt_smem(two), st, 0, a.X, a.mu, a.n_rows, a.K, a.D, a.max_rows,
+  e = launch_ex(dots, dim3(dots_grid), dim3(kDtThreads), dt_smem(two), st, 0, a.X, a.mu, a.n_rows, a.K, a.D, a.max_rows,
                 reinterpret_cast<float*>(a.ws + L.part), a.status);
   if (e != cudaSuccess) return e;
   switch (kpad(a.K)) {
-    case 16: return launch_tail<16>(a, L, grid, st);
-    case 32: return launch_tail<32>(a, L, grid, st);
-    case 64: return launch_tail<64>(a, L, grid, st);
-    default: return launch_tail<128>(a, L, grid, st);
+    case 16: return launch_tail<16>(a, L, dots_grid, grid, st);
+    case 32: return launch_tail<32>(a, L, dots_grid, grid, st);
+    case 64: return launch_tail<64>(a, L, dots_grid, grid, st);
+    default: return launch_tail<128>(a, L, dots_grid, grid, st);
   }
 }
 

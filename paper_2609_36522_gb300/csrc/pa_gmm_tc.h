@@ -12,7 +12,7 @@ namespace pa {
 struct GmmTcLayout {
   size_t part, resp, rcoef, total;  // byte offsets, total bytes
 };
-GmmTcLayout gmm_tc_layout(int K, int max_rows);
+GmmTcLayout gmm_tc_layout(int K, int64_t D, int max_rows);
 
 // The shared memory of its kernels fits the current device (and is granted).
 cudaError_t gmm_tc_setup(int K, bool* ok);

@@ -37,6 +37,11 @@ def test_workspace_sizes(lib):
     assert abi.pa_workspace_bytes(16, 8, 16, 65) == 0
     assert abi.pa_gmm_workspace_bytes(16, 16384, 100, 100) > 0
     assert abi.pa_gmm_workspace_bytes(129, 16384, 100, 100) == 0
+    # the tensor-core form's partial sums: a slot per CTA that has a piece, of the rows there are
+    assert abi.pa_gmm_workspace_bytes(4, 256, 8, 16) < 16 << 10
+    assert abi.pa_gmm_workspace_bytes(128, 256, 8, 16) < 128 << 10
+    assert abi.pa_gmm_workspace_bytes(128, 16384, 128, 16) >= 160 * 128 * 128 * 4
+    assert abi.pa_gmm_workspace_bytes(128, 64, 19600, 16) >= 154 * 128 * 128 * 4
 
 
 def test_status_strings(lib):
