@@ -49,8 +49,6 @@ inline int dots_ctas(int64_t D, int max_rows, int limit) {
   const int64_t pieces = ((int64_t)max_rows + kRows - 1) / kRows * ((D + kUnit - 1) / kUnit);
   return pieces < limit ? (int)pieces : limit;
 }
-// Rows of a slot of partial sums: a row block, or all rows of a handle that has fewer.
-__host__ __device__ inline int slot_rows(int max_rows) { return max_rows < kRows ? max_rows : kRows; }
 
 // components as stored: R rows and partial sums are padded to this many
 __host__ __device__ inline int kpad(int K) { return K <= 16 ? 16 : K <= 32 ? 32 : K <= 64 ? 64 : 128; }
@@ -191,7 +189,8 @@ __device__ __forceinline__ void copies_drain() { asm volatile("cp.async.wait_all
 template <bool TWO, bool VEC>
 __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __restrict__ X, const float* __restrict__ mu,
                                                               const int32_t* __restrict__ n_rows_dev, int K, int64_t D,
-                                                              int max_rows, float* __restrict__ part, int32_t* status) {
+                                                              int max_rows, float* __restrict__ part, int slots,
+                                                              int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr int kMuRows = dt_mu_rows(TWO), kRaws = dt_raws(TWO), kRawFloats = dt_raw_floats(TWO);
   constexpr int kStageFloats = 2 * kRawFloats;
@@ -332,7 +331,7 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
       take_until(nc);
       // TMEM lane = component; up to 64 components lane 64 + k holds the products
       // with the means' lo parts
-      float* out = part + (int64_t)sh.slot(blk, u0) * slot_rows(max_rows) * KP;
+      float* out = part + (int64_t)sh.slot(blk, u0) * KP;
       float* sc = stage0;  // [kRows][64]: every MMA that reads the stages is complete
       if constexpr (!TWO) {
         if (q4 >= 2) {
@@ -346,7 +345,7 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
           if constexpr (!TWO) acc[i] += sc[(rb + i) * 64 + k];
-          if (rb + i < nr && k < KP) out[(int64_t)(rb + i) * KP + k] = acc[i];
+          if (rb + i < nr && k < KP) out[(int64_t)(rb + i) * slots * KP + k] = acc[i];
         }
       }
       tc_fence_before_sync();
@@ -414,7 +413,7 @@ constexpr int kBatch = 20;       // partial sums in flight per thread: 152 of th
 constexpr int kRespGrid = 4096;  // rows beyond it are taken in turn
 
 template <int KP>
-__global__ void __launch_bounds__(kRespThreads) k_gmm_resp(const float* __restrict__ part, int dots_grid,
+__global__ void __launch_bounds__(kRespThreads) k_gmm_resp(const float* __restrict__ part, int slots, int dots_grid,
                                                            const float* __restrict__ coef, int T,
                                                            const int32_t* __restrict__ miss_bt,
                                                            const float* __restrict__ mnorm,
@@ -442,15 +441,14 @@ __global__ void __launch_bounds__(kRespThreads) k_gmm_resp(const float* __restri
       pdl_trigger();  // the successor may now run its prologue
       waited = true;
     }
-    const int64_t slot = (int64_t)slot_rows(max_rows) * KP;
-    const float* p = part + sh.slot(blk, 0) * slot + (int64_t)(r - blk * kRows) * KP + k;
+    const float* p = part + ((int64_t)(r - blk * kRows) * slots + sh.slot(blk, 0)) * KP + k;
     float hi = 0.f, lo = 0.f;
     for (int s = grp; s < members; s += kBatch * kGroups) {
       float v[kBatch];  // kBatch loads in flight
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
         v[u] = 0.f;
-        if (s + u * kGroups < members) v[u] = __ldcg(p + (s + u * kGroups) * slot);
+        if (s + u * kGroups < members) v[u] = __ldcg(p + (int64_t)(s + u * kGroups) * KP);
       }
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {  // TwoSum
@@ -802,7 +800,7 @@ cudaError_t launch_tail(const GmmTcArgs& a, const GmmTcLayout& L, int dots_grid,
   float* resp = reinterpret_cast<float*>(a.ws + L.resp);
   float* rcoef = reinterpret_cast<float*>(a.ws + L.rcoef);
   cudaError_t e = launch_ex(k_gmm_resp<KP>, dim3(a.max_rows < kRespGrid ? a.max_rows : kRespGrid), dim3(kRespThreads), 0,
-                            st, 0, part, dots_grid, a.coef, a.T, a.miss_bt, a.mnorm, a.n_rows, a.K, a.D, a.max_rows, resp,
+                            st, 0, part, L.slots, dots_grid, a.coef, a.T, a.miss_bt, a.mnorm, a.n_rows, a.K, a.D, a.max_rows, resp,
                             rcoef);
   if (e != cudaSuccess) return e;
   return launch_ex(k_gmm_out_tc<KP>, dim3(grid), dim3(kOtThreads), OtShape<KP>::smem(), st, 0, a.X, a.mu,
@@ -817,7 +815,9 @@ GmmTcLayout gmm_tc_layout(int K, int64_t D, int max_rows) {
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, kAlign); return at; };
   const size_t blocks = ((size_t)max_rows + kRows - 1) / kRows;
   const size_t ctas = (size_t)dots_ctas(D, max_rows, kMaxCtas);
-  L.part = take((ctas > blocks ? ctas : blocks) * slot_rows(max_rows) * kpad(K) * sizeof(float));  // a slot per CTA or block
+  L.slots = (int)(ctas > blocks ? ctas : blocks);
+  // [row of a block][CTA, or block where there are more][component]
+  L.part = take((size_t)(max_rows < kRows ? max_rows : kRows) * L.slots * kpad(K) * sizeof(float));
   L.resp = take((size_t)max_rows * kpad(K) * sizeof(float));
   L.rcoef = take((size_t)2 * max_rows * sizeof(float));
   L.total = o;
@@ -857,7 +857,7 @@ cudaError_t gmm_tc_launch(const GmmTcArgs& a, cudaStream_t st) {
   auto dots = two ? (vec ? k_gmm_dots_tc<true, true> : k_gmm_dots_tc<true, false>)
                   : (vec ? k_gmm_dots_tc<false, true> : k_gmm_dots_tc<false, false>);
   e = launch_ex(dots, dim3(dots_grid), dim3(kDtThreads), dt_smem(two), st, 0, a.X, a.mu, a.n_rows, a.K, a.D, a.max_rows,
-                reinterpret_cast<float*>(a.ws + L.part), a.status);
+                reinterpret_cast<float*>(a.ws + L.part), L.slots, a.status);
   if (e != cudaSuccess) return e;
   switch (kpad(a.K)) {
     case 16: return launch_tail<16>(a, L, dots_grid, grid, st);

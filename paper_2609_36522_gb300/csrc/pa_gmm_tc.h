@@ -11,6 +11,7 @@ namespace pa {
 // every CTA, responsibilities, the rows' scalars.
 struct GmmTcLayout {
   size_t part, resp, rcoef, total;  // byte offsets, total bytes
+  int slots;                        // partial sums kept per row: one per CTA of its block
 };
 GmmTcLayout gmm_tc_layout(int K, int64_t D, int max_rows);
 
