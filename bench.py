@@ -62,9 +62,8 @@ FLUSH_BYTES = 256 << 20
 E2E_CHUNK = 4      # Picard iterations issued between two pa_poll calls in the end-to-end run
 GMM_FORMS = {2: "one kernel: clusters of 16 CTAs per 8 rows, CUDA-core dot products summed through "
                 "distributed shared memory",
-             1: "three persistent kernels: dot products on the tensor cores (tcgen05 kind::tf32, split "
-                "operands), responsibilities, output contraction on the tensor cores (kind::f16, exact "
-                "three-part bfloat16 operands)",
+             1: "three persistent kernels: dot products on the tensor cores, responsibilities, output "
+                "contraction on the tensor cores (both tcgen05 kind::f16, exact three-part bfloat16 operands)",
              0: "CUDA-core dot products (fp32 FMA) + output kernel"}
 PEAKS_PATH = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0

@@ -7,25 +7,23 @@
 //   k_gmm_out_tc    eps = a x - a sqrt(a) R M, tiles of 128 columns x up to
 //                   128 rows
 //
-// fp32 accuracy from shorter operands: the dot products split every value in
-// two tf32 parts, v = hi + lo with hi = tf32(v), lo = tf32(v - hi), and add up
-// the products hi hi + hi lo + lo hi (and, where it costs nothing, lo lo) in
-// fp32; the output splits it in three bfloat16 parts.
+// fp32 accuracy from shorter operands: every value is split in three bfloat16
+// parts, which hold it exactly, and the products of parts down to 2^-26 of a
+// product are added up in fp32.
 //
 // What bounds it: at 118 rows of 4x128x128 and 64 components a call reads the
 // rows twice and the means twice and writes eps once, 126 MB (19 us at the copy
-// rate, less for what the 126 MB L2 still holds). The two contractions are three
-// times 1 GFLOP of tf32 each, 3 to 4 us on all SMs, so both large
+// rate, less for what the 126 MB L2 still holds). The two contractions are 1
+// GFLOP each, in bfloat16 six to eight times that, 3 to 5 us on all SMs, so both large
 // kernels are one CTA per SM that keeps copies in flight while the tensor core
 // works: asynchronous copies into a ring of shared-memory stages, warps that
 // split what has landed, one thread that issues a stage's MMAs as soon as it is
 // full, mbarriers (tcgen05.commit) that free it again. Loads into registers
 // cost the loop their latency wherever the value was moved. A
 // row block belongs to a group of CTAs, so any row count fills the SMs about
-// evenly and partial sums are written once per CTA and row block, not added
-// with atomics; R's kernel adds them in CTA order, so a result is reproducible
-// bit for bit. The means are read as they lie: no image
-// of them is kept.
+// evenly; a CTA's partial sums of a row block have a place of their own, and R's
+// kernel adds them in CTA order, so a result is reproducible bit for bit. The
+// means are read as they lie: no image of them is kept.
 //
 // Every wait is bounded. A wait that runs out records kDevTimeout, the thread
 // stops waiting, runs on with in-bounds accesses only, and eps is written as
@@ -76,16 +74,6 @@ struct Share {
   __device__ int slot(int blk, int member) const { return grouped() ? first(blk) + member : blk; }
 };
 
-struct Hilo {
-  float4 hi, lo;
-};
-__device__ __forceinline__ Hilo split4(float4 v) {
-  Hilo r;
-  r.hi = make_float4(to_tf32(v.x), to_tf32(v.y), to_tf32(v.z), to_tf32(v.w));
-  r.lo = make_float4(to_tf32(v.x - r.hi.x), to_tf32(v.y - r.hi.y), to_tf32(v.z - r.hi.z), to_tf32(v.w - r.hi.w));
-  return r;
-}
-
 // Eight values as three bfloat16 parts each, v = a + b + c exactly (8 + 8 + 8
 // bits): 16 bytes per part, a half of a core-matrix pair's row.
 struct Parts {
@@ -125,24 +113,33 @@ __device__ __forceinline__ void named_sync(int id, int threads) {
 }
 
 // ---------------------------------------------------------------------------
-// Dot products. A unit is kUnit columns of a row block. The MMA's A operand is
-// the means (M = 128 rows: the hi and lo parts of 64 components, or, for more
-// than 64, the hi parts and in MMAs of their own the lo parts of 128), its B
-// operand the rows (N: the block's rows, rounded up to 16, hi and lo parts). So
-// TMEM lane = component, column = row, and a row block of few rows costs few
+// Dot products. A unit is kUnit columns of a row block. Every value is held
+// exactly, as three bfloat16 parts a + b + c. The MMA's A operand is the means (M
+// = 128 rows: parts a and b of 64 components, then part c above rows of zeros;
+// for more than 64 components a part of 128), its B operand the rows (N: the
+// block's rows, rounded up to 16; parts a and b together, or one part). So TMEM
+// lane = component, column = row, and a row block of few rows costs few
 // columns. Operand rows past the counts hold whatever was there: they only
-// reach accumulators that nobody reads.
+// reach accumulators that nobody reads. The products a a have accumulators of
+// their own; a b, b a, a c, c a, b b (and b c up to 64 components) go to others
+// and are added once per chunk; the rest is below 2^-26 of a product.
 // The tensor core's running fp32 sum drops bits as it grows (with one
 // accumulator over all of a CTA's columns the dot products were off by five
 // times as much), so it runs over kDtChunk units only, in two accumulators used
 // in turn, and the converter warps add the finished chunk into registers,
-// rounding to nearest, while the next is multiplied. The products with a lo
-// part are 2^-11 smaller and have columns of their own.
+// rounding to nearest, while the next is multiplied.
+// (Two tf32 parts per value, 8 bytes of an operand stage in place of 6 and as
+// much time of the tensor core, lost a bit of one value in four: error of the
+// responsibilities against 64 bits, for rows of noise and small means, relative
+// to the same with fp32 multiply-adds, 1.42 at 16 components and 1500 rows of
+// 16384 columns, 1.15 at 64 components and 100 rows, 1.19 at 128 and 130 rows
+// of 6000; 0.97, 0.93 and 1.01 so. A call at 118 rows of 4x128x128 and 64
+// components takes 40.6 us, 41.4 with tf32 parts.)
 //
 // Warps: four loaders issue 16-byte asynchronous copies (cp.async) of a unit's
 // rows and means into a ring of raw stages, already in core-matrix order;
 // sixteen converters, in two groups that take units in turn, write a raw
-// stage's hi and lo parts into an operand stage; one thread issues the MMAs.
+// stage's parts into an operand stage; one thread issues the MMAs.
 // A copy takes a microsecond and more, an operand stage's turn (split, MMAs)
 // less: with raw values in rings of their own up to five units are on their
 // way (four stages that held a unit from its copy to its MMAs: 20 us a call).
@@ -153,14 +150,20 @@ constexpr int kDtLoadWarps = 4;
 constexpr int kDtLoad = kDtLoadWarps * 32;
 constexpr int kDtThreads = kDtConv + kDtLoad + 32;
 constexpr int kDtChunk = 2;                   // units per accumulator
+constexpr int kDtFold = 8;                    // chunks per running sum (see the sums' part of the kernel)
 constexpr uint32_t kDtTmem = 512;             // two accumulators of up to 256 columns
 
 __host__ __device__ constexpr int dt_mu_rows(bool two) { return two ? 128 : 64; }
 __host__ __device__ constexpr int dt_raw_floats(bool two) { return (kRows + dt_mu_rows(two)) * kUnit; }
 __host__ __device__ constexpr int dt_raws(bool two) { return two ? 3 : 5; }
-constexpr int kDtStages = 2;                  // operand stages: hi and lo parts
+constexpr int kDtStages = 2;                  // operand stages: three parts of 2 bytes
+constexpr int kDtPart = kUnit * 2;            // bytes of a row's part
+// the rows' parts, the means' parts, up to 64 components 64 rows of zeros
+__host__ __device__ constexpr int dt_stage_bytes(bool two) {
+  return (3 * kRows + 3 * dt_mu_rows(two) + (two ? 0 : 64)) * kDtPart;
+}
 __host__ inline size_t dt_smem(bool two) {
-  return (size_t)(dt_raws(two) + 2 * kDtStages) * dt_raw_floats(two) * sizeof(float);
+  return (size_t)dt_raws(two) * dt_raw_floats(two) * sizeof(float) + (size_t)kDtStages * dt_stage_bytes(two);
 }
 
 __device__ __forceinline__ void copy1(uint32_t dst, const float* src, bool there) {
@@ -193,13 +196,21 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
                                                               int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr int kMuRows = dt_mu_rows(TWO), kRaws = dt_raws(TWO), kRawFloats = dt_raw_floats(TWO);
-  constexpr int kStageFloats = 2 * kRawFloats;
-  constexpr int kMu = 2 * kRows * kUnit, kMlo = kMuRows * kUnit;  // the means' and their lo parts' offsets in an operand stage
+  // the means in an operand stage and the distance of their parts, in bytes
+  constexpr int kMu = 3 * kRows * kDtPart, kMuPart = kMuRows * kDtPart;
   __shared__ __align__(8) uint64_t raw[kRaws], rfree[kRaws], full[kDtStages], empty[kDtStages], done[2], afree[2];
   __shared__ uint32_t s_taddr;
-  float* stage0 = reinterpret_cast<float*>(smem_raw);
-  float* raw0 = stage0 + kDtStages * kStageFloats;
+  unsigned char* stage0 = smem_raw;
+  float* raw0 = reinterpret_cast<float*>(stage0 + kDtStages * dt_stage_bytes(TWO));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if constexpr (!TWO) {  // the rows below part c
+    for (int q = tid; q < kDtStages * 64 * kDtPart / 16; q += kDtThreads) {
+      const int s = q / (64 * kDtPart / 16);
+      reinterpret_cast<uint4*>(stage0 + s * dt_stage_bytes(TWO) + kMu + 3 * kMuPart)[q % (64 * kDtPart / 16)] =
+          make_uint4(0, 0, 0, 0);
+    }
+    fence_proxy_async_smem();
+  }
   if (tid == 0) {
     for (int s = 0; s < kRaws; ++s) {
       mbar_init(&raw[s], kDtLoad);
@@ -266,15 +277,36 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
       float acc[32];
 #pragma unroll
       for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+      // a chunk's two sums first, so that the running sum is rounded once
       auto add = [&](uint32_t col) {
 #pragma unroll
         for (int h = 0; h < 32; h += 8) {
           if (rb + h < Nb) {
-            float t[8];
-            tmem_ld8(tl + col + h, t);
+            float t[8], u[8];
+            tmem_ld8x2(tl + col + h, tl + col + (uint32_t)Nb + h, t, u);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[h + i] += t[i];
+            for (int i = 0; i < 8; ++i) acc[h + i] += t[i] + u[i];
           }
+        }
+      };
+      // TMEM lane = component; up to 64 components lane 64 + k holds the products
+      // with the means' part b
+      // A CTA's share of a block can be hundreds of units long (K 16, D 65536, 600
+      // rows: 68), and one fp32 sum over all of its chunks is then off by more than
+      // fp32 multiply-adds are: every kDtFold chunks the running sum goes to memory
+      // and starts again.
+      auto fold = [&](bool more) {
+        const int k = 32 * q4 + lane, rows = k < KP ? nr - rb : 0;
+        float* o = part + ((int64_t)rb * slots + sh.slot(blk, u0)) * KP + k;
+#pragma unroll
+        for (int i = 0; i < 32; ++i, o += (int64_t)slots * KP) {
+          if (i < rows) {
+            if (more)
+              atomicAdd(o, acc[i]);  // this thread's alone: an addition that nothing waits for
+            else
+              *o = acc[i];
+          }
+          acc[i] = 0.f;
         }
       };
       int taken = 0;  // chunks of this block added so far
@@ -285,10 +317,10 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
           __syncwarp();
           tc_fence_after_sync();
           add((c & 1u) * 256u);
-          add((c & 1u) * 256u + (uint32_t)Nb);
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(&afree[c & 1u]);
+          if ((TWO || q4 < 2) && taken % kDtFold == kDtFold - 1 && taken + 1 < nc) fold(taken >= kDtFold);
         }
       };
       for (int w = group; w < n; w += 2) {
@@ -296,6 +328,16 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
         // the values in storage order: consecutive threads, consecutive 16 bytes
         constexpr int kGroup = kDtGroupWarps * 32, kX = kRows * kUnit / 4 / kGroup, kM = kMuRows * kUnit / 4 / kGroup;
         const int rr = (gt >> 6) * 8 + (gt & 7);  // this thread's first row; the next is kGroup / 8 rows on
+        // its place in a part: 8 columns of 8 rows to a core matrix, 4 to a thread
+        const int at = (gt >> 6) * (8 * kDtPart) + ((gt >> 4) & 3) * 128 + (gt & 7) * 16 + ((gt >> 3) & 1) * 8;
+        constexpr int kNext = kGroup / 8 * kDtPart;
+        auto put = [&](unsigned char* to, float4 f, int part) {
+#pragma unroll
+          for (int p = 0; p < 3; ++p, to += part) {
+            const uint32_t lo = split2(f.x, f.y), hi = split2(f.z, f.w);
+            *reinterpret_cast<uint2*>(to) = make_uint2(lo, hi);
+          }
+        };
         float4 val[kX + kM];
         wait_or_fail(&raw[rs], (u / kRaws) & 1u, &bad, status);
         const float4* from = reinterpret_cast<const float4*>(raw0 + rs * kRawFloats) + gt;
@@ -304,24 +346,14 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
         __syncwarp();
         if (lane == 0) mbar_arrive(&rfree[rs]);
         if (u >= kDtStages) wait_or_fail(&empty[s], (u / kDtStages - 1) & 1u, &bad, status);
-        float4* xs = reinterpret_cast<float4*>(stage0 + s * kStageFloats) + gt;
-        float4* ms = xs + kMu / 4;
+        unsigned char* xs = stage0 + s * dt_stage_bytes(TWO) + at;
+        unsigned char* ms = xs + kMu;
 #pragma unroll
-        for (int i = 0; i < kX; ++i) {
-          if (rr + i * (kGroup / 8) < nr) {
-            const Hilo h = split4(val[i]);
-            xs[i * kGroup] = h.hi;
-            xs[i * kGroup + Nb * (kUnit / 4)] = h.lo;  // behind the Nb hi rows
-          }
-        }
+        for (int i = 0; i < kX; ++i)
+          if (rr + i * (kGroup / 8) < nr) put(xs + i * kNext, val[i], Nb * kDtPart);
 #pragma unroll
-        for (int i = 0; i < kM; ++i) {
-          if (rr + i * (kGroup / 8) < K) {
-            const Hilo h = split4(val[kX + i]);
-            ms[i * kGroup] = h.hi;
-            ms[i * kGroup + kMlo / 4] = h.lo;
-          }
-        }
+        for (int i = 0; i < kM; ++i)
+          if (rr + i * (kGroup / 8) < K) put(ms + i * kNext, val[kX + i], kMuPart);
         fence_proxy_async_smem();  // the tensor core reads what the threads wrote
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[s]);
@@ -329,10 +361,9 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
         take_until(w / kDtChunk);
       }
       take_until(nc);
-      // TMEM lane = component; up to 64 components lane 64 + k holds the products
-      // with the means' lo parts
-      float* out = part + (int64_t)sh.slot(blk, u0) * KP;
-      float* sc = stage0;  // [kRows][64]: every MMA that reads the stages is complete
+      // [kRows][64]: every MMA that reads the stages is complete (and the zeros lie behind)
+      float* sc = reinterpret_cast<float*>(stage0);
+      static_assert(TWO || kRows * 64 * (int)sizeof(float) <= kMu + 3 * kMuPart, "the zeros stay");
       if constexpr (!TWO) {
         if (q4 >= 2) {
 #pragma unroll
@@ -341,12 +372,11 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
         named_sync(1, kDtConv);
       }
       if (TWO || q4 < 2) {
-        const int k = 32 * q4 + lane;
+        if constexpr (!TWO) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if constexpr (!TWO) acc[i] += sc[(rb + i) * 64 + k];
-          if (rb + i < nr && k < KP) out[(int64_t)(rb + i) * slots * KP + k] = acc[i];
+          for (int i = 0; i < 32; ++i) acc[i] += sc[(rb + i) * 64 + 32 * q4 + lane];
         }
+        fold(nc > kDtFold);
       }
       tc_fence_before_sync();
     } else if (loader) {
@@ -365,8 +395,8 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
         copies_arrive(&raw[s]);
       }
     } else if (lane == 0) {
-      const uint32_t idesc = tc_idesc_tf32(128, 2 * Nb), idesc1 = tc_idesc_tf32(128, Nb);
-      constexpr uint32_t sbo = (kUnit / 4) * 128;  // next 8-row group
+      const uint32_t idesc = tc_idesc_bf16(128, 2 * Nb), idesc1 = tc_idesc_bf16(128, Nb);
+      constexpr uint32_t sbo = (kUnit / 8) * 128;  // next 8-row group
       uint32_t c = ck;
       for (int w = 0; w < n; ++w) {
         const uint32_t s = (v + w) % kDtStages;
@@ -374,16 +404,24 @@ __global__ void __launch_bounds__(kDtThreads, 1) k_gmm_dots_tc(const float* __re
         if (first && c >= 2) wait_or_fail(&afree[c & 1u], ((c >> 1) - 1) & 1u, &bad, status);
         wait_or_fail(&full[s], ((v + w) / kDtStages) & 1u, &bad, status);
         tc_fence_after_sync();
-        const uint32_t xs = smem_u32(stage0 + s * kStageFloats), ms = xs + kMu * 4;
-        const uint32_t sum = taddr + (c & 1u) * 256u;
+        const uint32_t xs = smem_u32(stage0 + s * dt_stage_bytes(TWO)), ms = xs + kMu;
+        const uint32_t sum = taddr + (c & 1u) * 256u, small = sum + (uint32_t)Nb;
 #pragma unroll
-        for (int ks = 0; ks < kUnit / 8; ++ks) {
+        for (int ks = 0; ks < kUnit / 16; ++ks) {
           const uint32_t ko = (uint32_t)ks * 256;  // two core matrices along the columns per step
-          const uint64_t a = tc_smem_desc(ms + ko, 128, sbo);
-          const uint64_t b = tc_smem_desc(xs + ko, 128, sbo);  // hi rows, then lo rows
-          tc_mma_tf32(sum, a, b, idesc, !first || ks > 0 ? 1u : 0u);
-          if constexpr (TWO)  // the lo means' products with the hi rows join the corrections
-            tc_mma_tf32(sum + (uint32_t)Nb, tc_smem_desc(ms + kMlo * 4 + ko, 128, sbo), b, idesc1, 1u);
+          uint64_t m[3], x[3];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            m[i] = tc_smem_desc(ms + i * kMuPart + ko, 128, sbo);
+            x[i] = tc_smem_desc(xs + (uint32_t)(i * Nb * kDtPart) + ko, 128, sbo);
+          }
+          tc_mma_f16(sum, m[0], x[0], idesc, !first || ks > 0 ? 1u : 0u);  // the rows' parts a and b
+          tc_mma_f16(small, m[0], x[2], idesc1, 1u);
+          if constexpr (TWO) {
+            tc_mma_f16(small, m[1], x[1], idesc1, 1u);
+            tc_mma_f16(small, m[1], x[0], idesc1, 1u);
+          }
+          tc_mma_f16(small, m[2], x[0], idesc1, 1u);
         }
         tc_commit(&empty[s]);
         if (w % kDtChunk == kDtChunk - 1 || w == n - 1) {

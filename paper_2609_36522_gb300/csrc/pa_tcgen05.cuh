@@ -1,10 +1,10 @@
 // Inline-PTX helpers for the 5th-generation tensor cores on sm_103a: TMEM
-// allocation, tcgen05.mma with kind::tf32 and bfloat16 operands in shared memory, commit to
-// an mbarrier, and TMEM -> register loads. One CTA, no clusters
+// allocation, tcgen05.mma with bfloat16 operands in shared memory, commit to an
+// mbarrier, and TMEM -> register loads. One CTA, no clusters
 // (cta_group::1). Operand tiles are K-major without swizzle: 8-row x 16-byte
-// core matrices, the two core matrices of one K step (8 tf32 or 16 bfloat16
-// values) 128 bytes apart (leading byte offset) and consecutive 8-row groups `sbo` bytes apart
-// (stride byte offset).
+// core matrices, the two core matrices of one K step (16 values) 128 bytes apart
+// (leading byte offset) and consecutive 8-row groups `sbo` bytes apart (stride
+// byte offset).
 #pragma once
 
 #include <stdint.h>
@@ -12,14 +12,6 @@
 #include "pa_bulk.cuh"
 
 namespace pa {
-
-// fp32 -> tf32 (round to nearest, ties away from zero), in a 32-bit container
-// whose low 13 mantissa bits are zero.
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
 
 // Shared-memory matrix descriptor: start address, leading and stride byte
 // offsets (all multiples of 16), descriptor version 1, no swizzle.
@@ -31,13 +23,8 @@ __device__ __forceinline__ uint64_t tc_smem_desc(uint32_t saddr, uint32_t lbo, u
   return d;
 }
 
-// Instruction descriptor for kind::tf32: fp32 accumulator, A and B tf32, both
+// Instruction descriptor for kind::f16: fp32 accumulator, A and B bfloat16, both
 // K-major, dense, M x N.
-__host__ __device__ constexpr uint32_t tc_idesc_tf32(int M, int N) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// The same for kind::f16: A and B bfloat16.
 __host__ __device__ constexpr uint32_t tc_idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
@@ -56,17 +43,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// One thread: D[tmem] (+)= A[smem] * B[smem]^T (accumulate = 0 overwrites).
-__device__ __forceinline__ void tc_mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// The same with 16-bit operands (a K step is 16 values, two core matrices).
+// One thread: D[tmem] (+)= A[smem] * B[smem]^T (accumulate = 0 overwrites); a K
+// step is 16 values, two core matrices.
 __device__ __forceinline__ void tc_mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                            uint32_t accumulate) {
   asm volatile(
@@ -100,6 +78,24 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Two such loads behind one wait.
+__device__ __forceinline__ void tmem_ld8x2(uint32_t ta, uint32_t tb, float (&v)[8], float (&w)[8]) {
+  uint32_t r[8], q[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(q[0]),
+        "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7])
+      : "r"(ta), "r"(tb)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[i] = __uint_as_float(r[i]);
+    w[i] = __uint_as_float(q[i]);
+  }
 }
 
 }  // namespace pa

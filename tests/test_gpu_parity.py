@@ -581,6 +581,42 @@ def test_gmm_cuda_core_form_at_any_scale(K, D, scale, factor):
     g.close()
 
 
+@pytest.mark.parametrize("K,D,n,cap", [
+    (16, 16384, 1500, 1600), (16, 65536, 600, 640),  # a CTA's share of a block up to 68 units
+    (64, 16384, 100, 128), (128, 6000, 130, 260), (40, 2001, 300, 400)])
+def test_gmm_dot_products_keep_fp32_precision(K, D, n, cap):
+    """The tensor-core form's dot products are no further from 64 bits than the
+    CUDA-core form's fp32 multiply-adds. Rows of noise and means of norm 4: the
+    logits are of order 10 and the responsibilities carry the dot products' own
+    error, got back from eps by the means' Gram matrix. The two rms errors come
+    from 3 x n x K weights; equal ones differ by up to 5 % (measured over six
+    seeds), a bit of one operand in four lost makes it 15 % and more."""
+    import torch
+    from paper_2609_36522_gb300.solver import GmmDenoiser
+    sa, v = 0.5 ** 0.5, 0.5 * 0.25 + 0.5
+    errs = {0: [], 1: []}
+    for seed in range(3):
+        gen = torch.Generator(device="cuda").manual_seed(seed * 11 + K)
+        mu = 4.0 / D ** 0.5 * torch.randn(K, D, generator=gen, device="cuda")
+        x = torch.zeros(cap, D, device="cuda")
+        x[:n] = torch.randn(n, D, generator=gen, device="cuda")
+        md = torch.zeros(cap, 2, dtype=torch.int32, device="cuda")
+        nd = torch.tensor([n], dtype=torch.int32, device="cuda")
+        m, xx = mu.double(), x[:n].double()
+        r = torch.softmax((2 * sa * (xx @ m.T) - 0.5 * (m * m).sum(1)) / (2 * v), 1)
+        gram = torch.linalg.inv(m @ m.T)
+        for form in errs:
+            g = GmmDenoiser(mu, 0.5, np.full(17, 0.5), cap)
+            g.set_form(form)
+            out = torch.empty(cap, D, device="cuda")
+            g.eps(x.data_ptr(), md.data_ptr(), nd.data_ptr(), out)
+            torch.cuda.synchronize()
+            got = ((xx - out[:n].double() * v / sa) / sa) @ m.T @ gram
+            errs[form].append(float((got - r).pow(2).mean()))
+            g.close()
+    assert sum(errs[1]) ** 0.5 <= 1.1 * sum(errs[0]) ** 0.5, errs
+
+
 @pytest.mark.parametrize("form,large,small", [
     (0, (16, 12810, 640), (16, 12810, 50)),   # (K, D, capacity): a smaller capacity takes shorter chunks
     (0, (100, 4096, 64), (3, 4096, 64)), (2, (16, 16384, 64), (16, 4096, 64))])
