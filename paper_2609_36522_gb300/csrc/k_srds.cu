@@ -50,12 +50,21 @@
 
 #include "../../include/paraanya.h"
 #include "pa_internal.h"
+#include "pa_pair.h"
 
 namespace pa {
 void set_error(const std::string& msg);  // pa_solver.cpp
 }
 
 namespace {
+
+using pa::Pair;
+using pa::pair_add;
+using pa::pair_mul;
+using pa::pair_or;
+using pa::pair_sub;
+using pa::pair_sub_full;
+using pa::pair_value;
 
 constexpr int kSThreads = 256;
 constexpr int kSCols = 4;            // values per thread: 32 bytes of an fp64 row
@@ -131,42 +140,6 @@ __device__ __forceinline__ bool row_info(const SDev& d, const Stage& st, int r, 
 __device__ __forceinline__ double quantize_sum(double v) {
   return ceil(v * 4294967296.0) * (1.0 / 4294967296.0);
 }
-
-// ---- pairs: an unevaluated sum h + l of two fp32 values, |l| <= ulp(h) / 2.
-// Error-free sums and products (Dekker, Knuth: TwoSum, FastTwoSum, and TwoProd
-// by fused multiply-add); an operation's result is within a few 2^-48 of the
-// exact one. Where a value is not finite the error terms are not either, and
-// the plain fp32 result stands alone.
-struct Pair {
-  float h, l;
-};
-// (the _rn intrinsics: nothing here may be contracted into a multiply-add)
-__device__ __forceinline__ Pair pair_quick(float a, float b) {  // |a| >= |b|
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ Pair pair_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
-  const Pair s = pair_sum(a.h, b.h);
-  return pair_quick(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ Pair pair_sub(Pair a, Pair b) { return pair_add(a, Pair{-b.h, -b.l}); }
-__device__ __forceinline__ Pair pair_mul(Pair a, float b) {
-  const float p = __fmul_rn(a.h, b);
-  return {p, fmaf(a.l, b, fmaf(a.h, b, -p))};
-}
-__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
-  const float p = __fmul_rn(a.h, b.h);
-  return {p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
-}
-__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
-__device__ __forceinline__ Pair pair_or(Pair a, float plain) {  // the pair, or the fp32 value where it is not finite
-  return finite(__fadd_rn(a.h, a.l)) ? a : Pair{plain, 0.f};
-}
-__device__ __forceinline__ double pair_value(Pair a) { return (double)a.h + (double)a.l; }
 
 // The sum over a warp (in every lane): a butterfly of pairs, beside one of
 // plain values for a sum that is not finite.
@@ -448,7 +421,7 @@ __global__ void __launch_bounds__(kSThreads) k_srds_apply(SDev d, Stage st, cons
   for (int k = 0; k < kSCols; ++k) {
     const Pair dr = pair_add(pair_mul(Pair{cm1.x, cm1.y}, xv[k]), pair_mul(Pair{ec.x, ec.y}, ev[k]));
     g[k] = pair_or(pair_add(xv[k], dr), xv[k].h + fmaf(cm1.x, xv[k].h, ec.x * ev[k]));
-    nv[k] = corr ? pair_or(pair_add(g[k], pair_sub(fv[k], gv[k])), g[k].h + (fv[k].h - gv[k].h)) : g[k];
+    nv[k] = corr ? pair_or(pair_add(g[k], pair_sub_full(fv[k], gv[k])), g[k].h + (fv[k].h - gv[k].h)) : g[k];
     if (k < pc.n) {
       if (nhas) {
         const Pair df = pair_sub(nv[k], xh1[k]);

@@ -79,3 +79,46 @@ def test_unquantized_fp64_sums_depend_on_the_order():
             sums.add(s)
         differs += len(sums) > 1
     assert differs > 0
+
+
+PAIR_CHECK = r"""
+#include "pa_pair.h"
+#include <cstdint>
+#include <cstdio>
+int main() {
+  uint64_t s = 88172645463325252ull;
+  auto rnd = [&] { s ^= s << 13; s ^= s >> 7; s ^= s << 17; return s; };
+  int64_t bad = 0, short_bad = 0;
+  for (int i = 0; i < 2000000; ++i) {
+    // whole numbers, so that sums are exact in 64 bits: a high part of 24 bits in
+    // units of 2^32 and a low part of 24 bits in units of 1 to 128
+    const int64_t ah = (int64_t)(rnd() >> 41) + (1 << 22), dh = (int64_t)(rnd() >> 41) >> (rnd() % 24);
+    auto low = [&] { return ((int64_t)(rnd() >> 40) - (1 << 23)) * ((int64_t)1 << (rnd() % 8)); };
+    const int64_t al = low(), bl = low(), bh = -(ah - dh);  // from nearly -a to unrelated
+    const pa::Pair a = {(float)ah * 0x1p32f, (float)al}, b = {(float)bh * 0x1p32f, (float)bl};
+    const double want = (double)(((ah + bh) << 32) + al + bl), bound = 4 * 0x1p-48 * (want < 0 ? -want : want);
+    auto off = [&](pa::Pair r) { const double d = pa::pair_value(r) - want; return (d < 0 ? -d : d) > bound; };
+    bad += off(pa::pair_sub_full(a, pa::Pair{-b.h, -b.l}));
+    short_bad += off(pa::pair_sub(a, pa::Pair{-b.h, -b.l}));
+  }
+  std::printf("%lld %d\n", (long long)bad, short_bad > 0);
+  return 0;
+}
+"""
+
+
+def test_pair_differences_are_accurate_where_they_cancel(tmp_path):
+    """The difference F - G of a Parareal correction, compiled for the host: its
+    error is bounded by the result however far the operands cancel, which that
+    of the shorter subtraction is not."""
+    import os
+    import subprocess
+    from paper_2609_36522_gb300 import build as pa_build
+    src, exe = tmp_path / "pair.cpp", tmp_path / "pair"
+    src.write_text(PAIR_CHECK)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-I", pa_build.CSRC, str(src), "-o", str(exe)],
+                   check=True)
+    out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
+    assert out == "0 1\n"
+    with open(os.path.join(pa_build.CSRC, "k_srds.cu")) as f:
+        assert "pair_sub_full(fv[k], gv[k])" in f.read()
