@@ -577,7 +577,6 @@ struct ClShape {
   static size_t smem_bytes(int chunk) { return (size_t)(kClMaxK + RB) * ld(chunk) * sizeof(float); }
 };
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }

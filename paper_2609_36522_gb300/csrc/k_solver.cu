@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(kPlanOneThreads) k_plan_one(Dev d, int par) {
       }
     }
   }
-  decide_run<kPlanOneThreads>(d, ds, RedBits{s_conv, s_near}, par, true, -1);  // starts with a barrier
+  decide_run<kPlanOneThreads>(d, ds, RedBits{s_conv, s_near}, par, true);  // starts with a barrier
 }
 
 }  // namespace

@@ -203,7 +203,7 @@ __device__ __forceinline__ void step_tail(const Dev& d, DecideShared& ds, int pa
   const int cta = blockIdx.y * gridDim.x + blockIdx.x;
   stage_decision_bits(d, ds, par, cta, (int)ncta);
   __syncthreads();
-  decide_par(d, ds, par, cta, (int)ncta, -1);
+  decide_par(d, ds, par, cta, (int)ncta);
   __syncthreads();  // the next plan (ds.tn, ds.pn, chunk masks and bases) is known
   if (xn == nullptr || !live || nj <= 0) return;
   // a4 of the next iteration: its timestep i (tn <= i < tn + pn) reads state

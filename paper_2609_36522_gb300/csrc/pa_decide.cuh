@@ -26,7 +26,6 @@ struct DecideShared {
   int pts;                       // decide_par: window positions planned
   int total, active, iter;
   long long nfe, hits;
-  int target_b, target_i;  // the miss of the requested batch row, if any
 };
 
 // The plan of iteration k (copy par = k mod 2). It was written by the previous
@@ -42,8 +41,6 @@ __device__ void decide_load(const Dev& d, DecideShared& sh, int par) {
     sh.nfe = c.nfe;
     sh.hits = c.hits;
     sh.total = 0;
-    sh.target_b = -1;
-    sh.target_i = 0;
   }
   const Traj* tr0 = d.traj + par * d.B;
   for (int b = tid; b < d.B; b += NT) {
@@ -66,14 +63,13 @@ __device__ void decide_load(const Dev& d, DecideShared& sh, int par) {
 //  2. plans the next iteration: a timestep of the new window with a cache
 //     entry (i < e) hits iff delta < tau_cache (strict, Eq. 5), everything else
 //     misses; misses are compacted trajectory-major with a block-wide prefix
-//     sum; publish writes rank[b][j] (each miss's batch row) and miss_bt, and
-//     every CTA notes the miss of batch row `target` (target_b, target_i);
+//     sum; publish writes rank[b][j] (each miss's batch row) and miss_bt;
 //  3. publish writes the new trajectories and counters to copy par ^ 1 and
 //     the host-visible counters.
 // When no trajectory is active the plan is carried over unchanged. Starts
 // with a barrier (after decide_load) and ends with one.
 template <int NT, typename Red>
-__device__ void decide_run(const Dev& d, DecideShared& sh, const Red& red, int par, bool publish, int target) {
+__device__ void decide_run(const Dev& d, DecideShared& sh, const Red& red, int par, bool publish) {
   int* s_t = sh.t; int* s_p = sh.p; int* s_e = sh.e;
   int* s_tn = sh.tn; int* s_pn = sh.pn; int* s_m = sh.m; int* s_h1 = sh.h1;
   int* s_om = sh.om; int* s_oh1 = sh.oh1; int* s_warp = sh.warp_tot;
@@ -169,17 +165,6 @@ __device__ void decide_run(const Dev& d, DecideShared& sh, const Red& red, int p
   }
   __syncthreads();
   int r = s_warp[warp] + incl - cnt;
-  if (target >= r && target < r + cnt) {  // the requested batch row is one of this thread's misses
-    int rr = r;
-    for (int q = q0; q < q1; ++q) {
-      if (!is_miss(q)) continue;
-      if (rr == target) {
-        sh.target_b = q / P;
-        sh.target_i = s_tn[q / P] + q % P;
-      }
-      ++rr;
-    }
-  }
   if (publish) {
     for (int q = q0; q < q1; ++q) {
       const int b = q / P, j = q % P;
@@ -332,13 +317,12 @@ __device__ __forceinline__ void carry_plan(const Dev& d, int par) {
 //     (an exclusive scan): misses are ranked trajectory-major, ascending t.
 // Then, after one CTA barrier, every warp handles chunks: the ranks and the
 // miss list are written by publishing CTAs (chunk c by the CTA whose pub_id is
-// c mod pub_count; pub_id < 0 writes nothing) and every CTA notes the miss of
-// batch row `target` (target_b, target_i); the CTA with pub_id 0 also writes
+// c mod pub_count; pub_id < 0 writes nothing); the CTA with pub_id 0 also writes
 // the trajectories, counters and iteration log. Gives the same plan, ranks and
 // counters as decide_run. Every thread of the CTA calls it; the caller
 // synchronises the CTA afterwards. (The fused step's form; the planning
 // kernel's, which spreads it over the CTA's warps, is decide_grid.)
-__device__ inline void decide_par(const Dev& d, DecideShared& sh, int par, int pub_id, int pub_count, int target) {
+__device__ inline void decide_par(const Dev& d, DecideShared& sh, int par, int pub_id, int pub_count) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int B = d.B, P = d.P, T = d.T;
   const int N = B * P, nchunk = (N + 31) / 32;
@@ -414,28 +398,21 @@ __device__ inline void decide_par(const Dev& d, DecideShared& sh, int par, int p
     if (lane == 0) sh.pts = pts;
   }
   __syncthreads();
-  // the misses' ranks and miss list (trajectory-major, ascending t), the requested row
+  // the misses' ranks and miss list (trajectory-major, ascending t)
   for (int c = warp; c < nchunk; c += nw) {
-    const bool writes = pub_id >= 0 && c % pub_count == pub_id;
-    if (!writes && target < 0) continue;
+    if (pub_id < 0 || c % pub_count != pub_id) continue;
     const int q = c * 32 + lane;
     if (q >= N) continue;
     const unsigned mm = sh.cmiss[c];
     const int miss = (mm >> lane) & 1u;
     const int b = q / P, j = q - b * P;
     const int r = sh.cbase[c] + __popc(mm & ((1u << lane) - 1u));
-    if (miss && r == target) {
-      sh.target_b = b;
-      sh.target_i = sh.tn[b] + j;
-    }
-    if (writes) {
-      if (miss) {
-        d.rank[q] = r;
-        d.miss_bt[2 * r] = b;
-        d.miss_bt[2 * r + 1] = sh.tn[b] + j;
-      } else {
-        d.rank[q] = -1;
-      }
+    if (miss) {
+      d.rank[q] = r;
+      d.miss_bt[2 * r] = b;
+      d.miss_bt[2 * r + 1] = sh.tn[b] + j;
+    } else {
+      d.rank[q] = -1;
     }
   }
   if (pub_id == 0) {
