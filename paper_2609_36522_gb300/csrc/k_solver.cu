@@ -352,10 +352,10 @@ __global__ void __launch_bounds__(kPlainThreads) k_update_plain(Dev d, const flo
 // ---------------------------------------------------------------------------
 // Planning kernel (a10, a2, a3 after iteration k, then a4 of iteration k+1),
 // one launch. The update kernel left complete fp64 sums of the Eq. 2 errors
-// and Eq. 4 distances; every CTA reads them (B*P of each), divides by D and
-// takes the whole decision in shared memory -- the same inputs and the same
-// arithmetic give the same plan in every CTA -- then copies the column range
-// blockIdx.x of batch rows blockIdx.y, blockIdx.y + gridDim.y, ... that hold
+// and Eq. 4 distances; every CTA reads them (B*P of each), compares them with tol
+// D and tau_cache D (by their bits) and takes the whole decision in shared
+// memory -- the same inputs and the same arithmetic give the same plan in every
+// CTA -- then copies the column range blockIdx.x of batch rows blockIdx.y, blockIdx.y + gridDim.y, ... that hold
 // a miss (one row per CTA unless the rows outnumber one wave of CTAs). A CTA of
 // the last row also publishes the plan (copy par ^ 1 of the trajectories and
 // counters, ranks, miss list, iteration log), one of the row before reports the

@@ -67,7 +67,7 @@ using pa::pair_sub_full;
 using pa::pair_value;
 
 constexpr int kSThreads = 256;
-constexpr int kSCols = 4;            // values per thread: 32 bytes of an fp64 row
+constexpr int kSCols = 4;            // values per thread: 16 bytes of a row's high and of its low half
 constexpr int kSChunk = kSThreads * kSCols;  // columns per apply CTA
 constexpr int kSMaxRows = 2048;      // B * N
 
@@ -817,7 +817,7 @@ extern "C" pa_status pa_srds_step_async(pa_srds* h, const float** batch_x, const
   const SDev& d = h->d;
   const Stage st = current_stage(h);
   const int rows = st.kind == kFine ? d.B * d.N : d.B;
-  // every CTA plans: about two CTAs per SM in all, each narrowing a longer part of its row
+  // every CTA plans: about two CTAs per SM in all, each copying its part of a row's high half
   int gx = d.nstrip;
   const int gcap = (2 * h->nsm + rows - 1) / rows;
   if (gx > gcap) gx = gcap;

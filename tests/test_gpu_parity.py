@@ -359,12 +359,12 @@ def test_gmm_kernel_against_oracle(wname, n, max_rows, form):
     products on the tensor cores (form 1) and on the CUDA cores (form 0), on
     rows spread over the whole schedule, with the device row count below the
     capacity and not a multiple of the cluster form's 8-row blocks, and over
-    three calls in a row (the fixed-point accumulators and the tickets are
-    reused). Rows past the count hold NaN: the cluster form copies them with
-    the block and must keep them out of every counted row. With 64 components: one row, 70 rows (a ragged second 64-row
-    block of the tensor-core form's row tiles is not reached; rows past 48
-    are), and full 128-row tiles; exactly 32 components; 3 components over 64
-    columns (4 columns per CTA of the cluster form)."""
+    three calls in a row (form 0's two sets of fixed-point accumulators are
+    used in turn). Rows past the count hold NaN: the cluster form copies them
+    with the block and must keep them out of every counted row. With 64
+    components: one row, 48 and 70 rows, and a full row block of 128; exactly 32
+    components; 3 components over 64 columns (4 columns per CTA of the cluster
+    form)."""
     import torch
     from paper_2609_36522_gb300 import abi
     from paper_2609_36522_gb300.solver import GmmDenoiser
@@ -725,9 +725,9 @@ def test_gmm_in_cuda_graph():
 
 @pytest.mark.parametrize("form", [1, 0])
 def test_sd15_other_denoiser_forms(form):
-    """Whole-pipeline parity with the denoiser's two-kernel forms (dot
-    products on the tensor cores, the default only above 16 components, or
-    on the CUDA cores) in place of the cluster form."""
+    """Whole-pipeline parity with the denoiser's other forms (three kernels on
+    the tensor cores, two on the CUDA cores) in place of the cluster form, the
+    default at this size."""
     w = W.SD15
     assert compare(w, oracle_run(w), gpu_run(w, gmm_form=form)).max() <= REL_TOL
 
