@@ -77,20 +77,20 @@ NOMINAL_HBM_GBS = 8000.0
 NCU_TRAFFIC = {
     # per iteration: k_update_lean + k_plan_gather read + write bytes, averaged
     # over the first generation's launches
-    ("851a1ecc31635a05", "sd15"): 8265152,       # 6,251,776 + 2,013,376 (no DRAM writes)
-    ("851a1ecc31635a05", "batched"): 30291968,   # 24,590,165 + 5,701,803
-    ("851a1ecc31635a05", "large"): 79398949,     # 70,548,919 + 8,850,030
+    ("d3a904210ec3b64d", "sd15"): 8262592,        # 6,248,576 + 2,014,016 (no DRAM writes)
+    ("d3a904210ec3b64d", "batched"): 30283861,    # 24,581,760 + 5,702,101
+    ("d3a904210ec3b64d", "large"): 79398144,      # 70,548,480 + 8,849,664
 }
 # ncu average duration per launch (cold cache, serialised) of the solver-step
 # and denoiser kernels over the launches of a launch list (`--metrics
 # gpu__time_duration.sum`, the launch lists kept under profiles/), the same key.
 NCU_LAUNCH_US = {
-    ("851a1ecc31635a05", "sd15"): {"k_update_lean": 9.91, "k_plan_gather": 7.68, "k_gmm_cluster": 11.18,
-                                   "k_init": 7.10},
-    ("851a1ecc31635a05", "batched"): {"k_update_lean": 19.37, "k_plan_gather": 9.63, "k_gmm_cluster": 20.93,
-                                      "k_init": 9.81},
-    ("851a1ecc31635a05", "large"): {"k_update_lean": 35.51, "k_plan_gather": 11.00, "k_gmm_dots_tc": 20.94,
-                                    "k_gmm_resp": 6.26, "k_gmm_out_tc": 19.32, "k_init": 11.89},
+    ("d3a904210ec3b64d", "sd15"): {"k_update_lean": 9.91, "k_plan_gather": 7.65, "k_gmm_cluster": 11.23,
+                                   "k_init": 7.12},
+    ("d3a904210ec3b64d", "batched"): {"k_update_lean": 19.44, "k_plan_gather": 9.68, "k_gmm_cluster": 21.02,
+                                      "k_init": 9.88},
+    ("d3a904210ec3b64d", "large"): {"k_update_lean": 35.64, "k_plan_gather": 11.02, "k_gmm_dots_tc": 20.15,
+                                    "k_gmm_resp": 6.28, "k_gmm_out_tc": 19.41, "k_init": 12.06},
 }
 
 
