@@ -412,6 +412,7 @@ def test_gmm_kernel_against_oracle(wname, n, max_rows, form):
     (64, 16400, 100, 128, 1),                              # rows 4 bytes past a 16-byte boundary
     (16, 4096, 1500, 1600, 0), (5, 9000, 800, 800, 0),     # few components, many rows
     (128, 64, 19590, 19600, 0),                            # more row blocks than CTAs
+    (16, 16384, 1500, 1600, 0), (100, 8192, 1500, 1536, 0),  # running sums folded into memory
     (18, 1024, 7, 8, 0), (1, 64, 3, 3, 0),                 # fewer pieces than CTAs
     (100, 3000, 0, 256, 0),                                # no rows
     (3, 37, 5, 8, 0), (17, 129, 20, 20, 3), (70, 1, 130, 140, 0), (33, 95, 300, 301, 2)])  # small and odd: 4-byte copies
